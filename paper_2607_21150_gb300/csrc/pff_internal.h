@@ -296,9 +296,23 @@ template <typename T>
 cudaError_t launch_dscale(T* y, const T* x, const T* d, long long n, cudaStream_t st);
 cudaError_t launch_d2f(float* y, const double* x, long long n, cudaStream_t st);
 cudaError_t launch_f2d(double* y, const float* x, long long n, cudaStream_t st);
-cudaError_t launch_q1_spmv(const MeshDev& mc, const double* A, const double* x, double* y, cudaStream_t st);
-// The same with an FP32 copy of the stencil and FP32 arithmetic (FP64 vectors).
-cudaError_t launch_q1_spmv32(const MeshDev& mc, const float* A, const double* x, double* y, cudaStream_t st);
+// Stencil product A v (or A^T v) of the assembled order-1 operators with the
+// update that consumes it:
+//   kStProduct   y = A v              kStScaled   y = D^-1 A v
+//   kStResidual  y = b - A v          kStChebInit r = D^-1 (b - A v), y = cr r
+//   kStChebStep  x += v (xset: x = v); r -= D^-1 A v; y = cd v + cr r;
+//                last: x += that y instead, r and y not written
+// y must not be v.  f32: A is the FP32 copy of the stencil (FP32 arithmetic).
+enum StencilMode { kStProduct, kStScaled, kStResidual, kStChebInit, kStChebStep };
+struct StencilArgs {
+  MeshDev mesh;
+  const void* A;
+  const double *v, *b, *diag;
+  double *y, *r, *x;
+  double cd, cr;
+  int xset, last;
+};
+cudaError_t launch_q1_stencil(int mode, bool f32, bool transpose, const StencilArgs& a, cudaStream_t st);
 cudaError_t launch_q1_diag(const MeshDev& mc, const double* A, double* d, cudaStream_t st);
 // Sum-factorised element matrices (Ke: [nel][32][32] work space) and a
 // deterministic gather into the stencil storage.
@@ -307,7 +321,6 @@ cudaError_t launch_q1_diag(const MeshDev& mc, const double* A, double* d, cudaSt
 cudaError_t launch_q1_assemble_sf(const MeshDev& mc, int Q, const double* lin, const float* lin32, const double* B1,
                                   const double* D1, const uint8_t* maskc, double* Ke, double* A, int kx,
                                   cudaStream_t st);
-cudaError_t launch_q1_spmv_t(const MeshDev& mc, const double* A, const double* x, double* y, cudaStream_t st);
 // Geometric h-hierarchy on the order-1 grid (full coarsening, trilinear
 // transfers): Galerkin element matrices of the coarse grid, their gather into
 // the stencil storage, the coarse mask, and the transfers.
@@ -318,8 +331,13 @@ cudaError_t launch_q1_gather(const MeshDev& mc, const double* Ke, const uint8_t*
 cudaError_t launch_hmask(const MeshDev& mf, const MeshDev& mc, const uint8_t* maskf, uint8_t* maskc, cudaStream_t st);
 cudaError_t launch_hprolong_add(const MeshDev& mc, const MeshDev& mf, const double* xc, double* xf,
                                 const uint8_t* maskc, const uint8_t* maskf, cudaStream_t st);
+// ... and the coarse level's first smoothing vectors r = D^-1 r_c, d = inv_theta r.
 cudaError_t launch_hrestrict(const MeshDev& mc, const MeshDev& mf, const double* rf, double* rc,
-                             const uint8_t* maskc, const uint8_t* maskf, cudaStream_t st);
+                             const uint8_t* maskc, const uint8_t* maskf, const double* diag, double inv_theta,
+                             double* r, double* d, cudaStream_t st);
+// The same from a given b (vectors of n entries).
+template <typename T>
+cudaError_t launch_cheb_zero(long long n, const T* b, const T* diag, T* r, T* d, double inv_theta, cudaStream_t st);
 cudaError_t launch_sel_scale(double* y, const uint8_t* sel, double s, long long n, cudaStream_t st);
 cudaError_t launch_zero_masked(double* y, const uint8_t* mask, long long n, cudaStream_t st);
 

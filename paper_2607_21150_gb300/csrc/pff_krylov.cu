@@ -167,74 +167,125 @@ cudaError_t launch_f2d(double* y, const float* x, long long n, cudaStream_t st) 
 // offset (dx+1) + 3 (dy+1) + 9 (dz+1); Dirichlet rows and columns are zero
 // with a unit diagonal.
 
-// y = A x with the stencil storage (FP64), one thread per node.
-__global__ void k_q1_spmv(MeshDev mc, const double* __restrict__ A, const double* __restrict__ x,
-                          double* __restrict__ y) {
-  const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (n >= mc.nn) return;
-  const int nnz_ = (int)(mc.nn / ((long long)mc.nnx * mc.nny));
-  const int I = (int)(n % mc.nnx), J = (int)((n / mc.nnx) % mc.nny), K = (int)(n / ((long long)mc.nnx * mc.nny));
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int slot = 0; slot < 27; ++slot) {
-    const int dx = slot % 3 - 1, dy = (slot / 3) % 3 - 1, dz = slot / 9 - 1;
-    const int I2 = I + dx, J2 = J + dy, K2 = K + dz;
-    if (I2 < 0 || J2 < 0 || K2 < 0 || I2 >= mc.nnx || J2 >= mc.nny || K2 >= nnz_) continue;
-    const long long m = I2 + (long long)mc.nnx * (J2 + (long long)mc.nny * K2);
-    double xv[4];
-    for (int g = 0; g < 4; ++g) xv[g] = x[g * mc.nn + m];
-    for (int f = 0; f < 4; ++f)
-      for (int g = 0; g < 4; ++g) acc[f] += A[(long long)(slot * 16 + f * 4 + g) * mc.nn + n] * xv[g];
+// Products with the stencil storage and the vector updates that consume them,
+// one kernel per product.  A block takes 32 consecutive nodes; its nine warps
+// take the nine (dy, dz) rows of the stencil, three slots each, so that a
+// node's 432 entries are loaded by nine threads with 48 loads in flight
+// (every load 32 consecutive nodes); the nine partial sums meet in shared
+// memory and 128 threads (node, field) apply the update.
+//
+// On the coarse grids of the solver (16^3 elements and below) everything lives
+// in L2 and a product is one latency chain.  One thread per node, as before,
+// walked 27 slots one after the other on 20 blocks: 29.5 us per product on
+// 17^3 nodes, and the vector updates were launches of their own.  On 65^3
+// nodes the product streams 474 MB (FP32), which either form does at HBM speed.
+//
+// TA = double: FP64 entries and arithmetic; float (the mixed solver's coarse
+// level, which only preconditions): an FP32 copy of the stencil and FP32
+// arithmetic on FP64 vectors, v taken to FP32 by truncation of its significand
+// (integer operations: the conversion instructions run at the FP64 rate).
+// TR: A^T, whose row (g, n) gathers the entries A[(f, m), (g, n)] of the nodes
+// m = n - offset(slot).
+constexpr int kStNodes = 32, kStRows = 9, kStThreads = kStNodes * kStRows;
+
+template <typename TA> __device__ __forceinline__ TA st_vec(double v);
+template <> __device__ __forceinline__ double st_vec<double>(double v) { return v; }
+template <> __device__ __forceinline__ float st_vec<float>(double v) { return df_split(v).hi; }
+__device__ __forceinline__ double st_sum(double v) { return v; }
+__device__ __forceinline__ double st_sum(float v) { return df_f2d(v); }
+
+template <typename TA, bool TR, int MODE>
+__global__ void __launch_bounds__(kStThreads) k_q1_stencil(const StencilArgs a) {
+  __shared__ TA red[kStRows][4][kStNodes];
+  const int t = threadIdx.x, lane = t & 31, row = t >> 5;
+  const int nn = (int)a.mesh.nn, nnx = a.mesh.nnx, nny = a.mesh.nny, nnz = nn / (nnx * nny);
+  const int n = blockIdx.x * kStNodes + lane;
+  // operands of the update, requested together with the entries
+  const bool owner = t < 4 * kStNodes && n < nn;
+  const long long i = (long long)row * nn + n;  // field `row` of node n
+  double b = 0.0, dg = 1.0, r = 0.0, v = 0.0, x = 0.0;
+  if (owner) {
+    if (MODE == kStResidual || MODE == kStChebInit) b = a.b[i];
+    if (MODE == kStScaled || MODE == kStChebInit || MODE == kStChebStep) dg = a.diag[i];
+    if (MODE == kStChebStep) {
+      r = a.r[i];
+      v = a.v[i];
+      if (!a.xset) x = a.x[i];
+    }
   }
-  for (int f = 0; f < 4; ++f) y[f * mc.nn + n] = acc[f];
-}
-// The same product with an FP32 copy of the stencil, FP32 arithmetic, FP64
-// vectors in and out (the mixed solver's coarse level: a preconditioner, whose
-// FP64 product is bound by the FP64 pipe at 432 multiply-adds per node).  x is
-// taken to FP32 by truncation of its significand (integer operations: the
-// conversion instructions run at the FP64 rate).
-__global__ void k_q1_spmv32(MeshDev mc, const float* __restrict__ A, const double* __restrict__ x,
-                            double* __restrict__ y) {
-  const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (n >= mc.nn) return;
-  const int nnz_ = (int)(mc.nn / ((long long)mc.nnx * mc.nny));
-  const int I = (int)(n % mc.nnx), J = (int)((n / mc.nnx) % mc.nny), K = (int)(n / ((long long)mc.nnx * mc.nny));
-  float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  for (int slot = 0; slot < 27; ++slot) {
-    const int dx = slot % 3 - 1, dy = (slot / 3) % 3 - 1, dz = slot / 9 - 1;
-    const int I2 = I + dx, J2 = J + dy, K2 = K + dz;
-    if (I2 < 0 || J2 < 0 || K2 < 0 || I2 >= mc.nnx || J2 >= mc.nny || K2 >= nnz_) continue;
-    const long long m = I2 + (long long)mc.nnx * (J2 + (long long)mc.nny * K2);
-    float xv[4];
-    for (int g = 0; g < 4; ++g) xv[g] = df_split(x[g * mc.nn + m]).hi;
-    for (int f = 0; f < 4; ++f)
-      for (int g = 0; g < 4; ++g) acc[f] = fmaf(A[(long long)(slot * 16 + f * 4 + g) * mc.nn + n], xv[g], acc[f]);
+  TA acc[4] = {0, 0, 0, 0};
+  if (n < nn) {
+    const TA* __restrict__ A = static_cast<const TA*>(a.A);
+    const int I = n % nnx, J = (n / nnx) % nny, K = n / (nnx * nny);
+    const int sg = TR ? -1 : 1, dy = sg * (row % 3 - 1), dz = sg * (row / 3 - 1);
+    if (J + dy >= 0 && J + dy < nny && K + dz >= 0 && K + dz < nnz) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const int dx = sg * (c - 1);
+        if (I + dx < 0 || I + dx >= nnx) continue;
+        const int m = n + dx + nnx * (dy + nny * dz);
+        const TA* __restrict__ As = A + (long long)(row * 3 + c) * 16 * nn + (TR ? m : n);
+        TA vm[4];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) vm[g] = st_vec<TA>(a.v[(long long)g * nn + m]);
+#pragma unroll
+        for (int f = 0; f < 4; ++f)
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            const TA w = As[(long long)(f * 4 + g) * nn];
+            if (TR) acc[g] += w * vm[f];
+            else acc[f] += w * vm[g];
+          }
+      }
+    }
   }
-  for (int f = 0; f < 4; ++f) y[f * mc.nn + n] = df_f2d(acc[f]);
-}
-// y = A^T x with the stencil storage: row (g, m) of A^T gathers the entries
-// A[(f, n), (g, m)] of the nodes n = m - offset(slot).
-__global__ void k_q1_spmv_t(MeshDev mc, const double* __restrict__ A, const double* __restrict__ x,
-                            double* __restrict__ y) {
-  const long long m = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (m >= mc.nn) return;
-  const int nnz_ = (int)(mc.nn / ((long long)mc.nnx * mc.nny));
-  const int I = (int)(m % mc.nnx), J = (int)((m / mc.nnx) % mc.nny), K = (int)(m / ((long long)mc.nnx * mc.nny));
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int slot = 0; slot < 27; ++slot) {
-    const int dx = slot % 3 - 1, dy = (slot / 3) % 3 - 1, dz = slot / 9 - 1;
-    const int I2 = I - dx, J2 = J - dy, K2 = K - dz;
-    if (I2 < 0 || J2 < 0 || K2 < 0 || I2 >= mc.nnx || J2 >= mc.nny || K2 >= nnz_) continue;
-    const long long n = I2 + (long long)mc.nnx * (J2 + (long long)mc.nny * K2);
-    double xv[4];
-    for (int f = 0; f < 4; ++f) xv[f] = x[f * mc.nn + n];
-    for (int f = 0; f < 4; ++f)
-      for (int g = 0; g < 4; ++g) acc[g] += A[(long long)(slot * 16 + f * 4 + g) * mc.nn + n] * xv[f];
+#pragma unroll
+  for (int f = 0; f < 4; ++f) red[row][f][lane] = acc[f];
+  __syncthreads();
+  if (!owner) return;
+  TA sum = 0;
+#pragma unroll
+  for (int w = 0; w < kStRows; ++w) sum += red[w][row][lane];
+  const double Av = st_sum(sum);
+  if (MODE == kStProduct) a.y[i] = Av;
+  if (MODE == kStScaled) a.y[i] = Av / dg;
+  if (MODE == kStResidual) a.y[i] = b - Av;
+  if (MODE == kStChebInit) {
+    const double ri = (b - Av) / dg;
+    a.r[i] = ri;
+    a.y[i] = ri * a.cr;
   }
-  for (int g = 0; g < 4; ++g) y[g * mc.nn + m] = acc[g];
+  if (MODE == kStChebStep) {
+    const double ri = r - Av / dg;
+    const double di = a.cd * v + a.cr * ri;
+    double xi = a.xset ? v : x + v;
+    if (a.last) {
+      xi += di;
+    } else {
+      a.r[i] = ri;
+      a.y[i] = di;
+    }
+    a.x[i] = xi;
+  }
 }
-cudaError_t launch_q1_spmv_t(const MeshDev& mc, const double* A, const double* x, double* y, cudaStream_t st) {
-  k_q1_spmv_t<<<(unsigned)((mc.nn + 255) / 256), 256, 0, st>>>(mc, A, x, y); note_launch();
+
+template <typename TA, bool TR>
+static cudaError_t stencil_mode(int mode, const StencilArgs& a, cudaStream_t st) {
+  const unsigned nb = (unsigned)((a.mesh.nn + kStNodes - 1) / kStNodes);
+  switch (mode) {
+    case kStProduct: k_q1_stencil<TA, TR, kStProduct><<<nb, kStThreads, 0, st>>>(a); break;
+    case kStScaled: k_q1_stencil<TA, TR, kStScaled><<<nb, kStThreads, 0, st>>>(a); break;
+    case kStResidual: k_q1_stencil<TA, TR, kStResidual><<<nb, kStThreads, 0, st>>>(a); break;
+    case kStChebInit: k_q1_stencil<TA, TR, kStChebInit><<<nb, kStThreads, 0, st>>>(a); break;
+    default: k_q1_stencil<TA, TR, kStChebStep><<<nb, kStThreads, 0, st>>>(a); break;
+  }
+  note_launch();
   return cudaGetLastError();
+}
+cudaError_t launch_q1_stencil(int mode, bool f32, bool transpose, const StencilArgs& a, cudaStream_t st) {
+  if (a.mesh.nn == 0) return cudaSuccess;
+  if (transpose) return f32 ? stencil_mode<float, true>(mode, a, st) : stencil_mode<double, true>(mode, a, st);
+  return f32 ? stencil_mode<float, false>(mode, a, st) : stencil_mode<double, false>(mode, a, st);
 }
 
 // y = s * sel (uint8 selector to FP64), and zeroing of Dirichlet entries.
@@ -260,14 +311,6 @@ __global__ void k_q1_diag(MeshDev mc, const double* __restrict__ A, double* __re
   const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (n >= mc.nn) return;
   for (int f = 0; f < 4; ++f) d[f * mc.nn + n] = A[(long long)(13 * 16 + f * 4 + f) * mc.nn + n];
-}
-cudaError_t launch_q1_spmv(const MeshDev& mc, const double* A, const double* x, double* y, cudaStream_t st) {
-  k_q1_spmv<<<(unsigned)((mc.nn + 255) / 256), 256, 0, st>>>(mc, A, x, y); note_launch();
-  return cudaGetLastError();
-}
-cudaError_t launch_q1_spmv32(const MeshDev& mc, const float* A, const double* x, double* y, cudaStream_t st) {
-  k_q1_spmv32<<<(unsigned)((mc.nn + 255) / 256), 256, 0, st>>>(mc, A, x, y); note_launch();
-  return cudaGetLastError();
 }
 cudaError_t launch_q1_diag(const MeshDev& mc, const double* A, double* d, cudaStream_t st) {
   k_q1_diag<<<(unsigned)((mc.nn + 255) / 256), 256, 0, st>>>(mc, A, d); note_launch();
@@ -548,61 +591,62 @@ __global__ void k_hmask(MeshDev mf, MeshDev mc, const uint8_t* __restrict__ mask
   for (int f = 0; f < 4; ++f) maskc[f * mc.nn + N] = maskf ? maskf[f * mf.nn + n] : 0;
 }
 
-// x_f += P x_c on unmasked fine DoFs (trilinear, one thread per fine vertex).
+// x_f += P x_c on unmasked fine DoFs (trilinear), one thread per fine vertex
+// and field: at most eight independent loads.
 __global__ void k_hprolong_add(MeshDev mc, MeshDev mf, const double* __restrict__ xc, double* __restrict__ xf,
                                const uint8_t* __restrict__ maskc, const uint8_t* __restrict__ maskf) {
-  const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (n >= mf.nn) return;
-  const int i = (int)(n % mf.nnx), j = (int)((n / mf.nnx) % mf.nny), k = (int)(n / ((long long)mf.nnx * mf.nny));
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int dz = 0; dz < 2; ++dz) {
-    if (dz && !(k & 1)) break;
-    const int K = (k >> 1) + dz;
-    const double wz = (k & 1) ? 0.5 : 1.0;
-    for (int dy = 0; dy < 2; ++dy) {
-      if (dy && !(j & 1)) break;
-      const int J = (j >> 1) + dy;
-      const double wy = (j & 1) ? 0.5 : 1.0;
-      for (int dx = 0; dx < 2; ++dx) {
-        if (dx && !(i & 1)) break;
-        const int I = (i >> 1) + dx;
-        const double w = wz * wy * ((i & 1) ? 0.5 : 1.0);
-        const long long N = I + (long long)mc.nnx * (J + (long long)mc.nny * K);
-        for (int f = 0; f < 4; ++f)
-          if (!(maskc && maskc[f * mc.nn + N])) acc[f] += w * xc[f * mc.nn + N];
-      }
-    }
+  const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (g >= 4 * mf.nn) return;
+  if (maskf && maskf[g]) return;
+  const int f = (int)(g / mf.nn), n = (int)(g % mf.nn);
+  const int i = n % mf.nnx, j = (n / mf.nnx) % mf.nny, k = n / (mf.nnx * mf.nny);
+  const double* x = xc + f * mc.nn;
+  const uint8_t* m = maskc ? maskc + f * mc.nn : nullptr;
+  double acc = 0.0;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
+    if ((dx && !(i & 1)) || (dy && !(j & 1)) || (dz && !(k & 1))) continue;
+    const double w = ((i & 1) ? 0.5 : 1.0) * ((j & 1) ? 0.5 : 1.0) * ((k & 1) ? 0.5 : 1.0);
+    const long long N = (i >> 1) + dx + (long long)mc.nnx * ((j >> 1) + dy + (long long)mc.nny * ((k >> 1) + dz));
+    const double v = x[N];
+    if (!(m && m[N])) acc += w * v;
   }
-  for (int f = 0; f < 4; ++f)
-    if (!(maskf && maskf[f * mf.nn + n])) xf[f * mf.nn + n] += acc[f];
+  xf[g] += acc;
 }
 
-// r_c = P^T r_f (zero on masked DoFs), one thread per coarse vertex gathering
-// the fine vertices within one fine spacing.
+// r_c = P^T r_f (zero on masked DoFs), one thread per coarse vertex and field
+// gathering the 27 fine vertices within one fine spacing (independent loads;
+// one thread per vertex with a rolled loop took 12 us per call on 9^3 coarse
+// nodes, a latency chain), and the first Chebyshev residual and direction of
+// the coarse level's smoothing from x = 0: r = D^-1 r_c, d = r / theta.
 __global__ void k_hrestrict(MeshDev mc, MeshDev mf, const double* __restrict__ rf, double* __restrict__ rc,
-                            const uint8_t* __restrict__ maskc, const uint8_t* __restrict__ maskf) {
-  const long long N = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (N >= mc.nn) return;
-  const int I = (int)(N % mc.nnx), J = (int)((N / mc.nnx) % mc.nny), K = (int)(N / ((long long)mc.nnx * mc.nny));
+                            const uint8_t* __restrict__ maskc, const uint8_t* __restrict__ maskf,
+                            const double* __restrict__ diag, double inv_theta, double* __restrict__ r,
+                            double* __restrict__ d) {
+  const long long G = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (G >= 4 * mc.nn) return;
+  const int f = (int)(G / mc.nn), N = (int)(G % mc.nn);
+  const int I = N % mc.nnx, J = (N / mc.nnx) % mc.nny, K = N / (mc.nnx * mc.nny);
   const int nnzf = (int)(mf.nn / ((long long)mf.nnx * mf.nny));
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int dz = -1; dz <= 1; ++dz) {
-    const int k = 2 * K + dz;
-    if (k < 0 || k >= nnzf) continue;
-    for (int dy = -1; dy <= 1; ++dy) {
-      const int j = 2 * J + dy;
-      if (j < 0 || j >= mf.nny) continue;
-      for (int dx = -1; dx <= 1; ++dx) {
-        const int i = 2 * I + dx;
-        if (i < 0 || i >= mf.nnx) continue;
-        const double w = (dx ? 0.5 : 1.0) * (dy ? 0.5 : 1.0) * (dz ? 0.5 : 1.0);
-        const long long n = i + (long long)mf.nnx * (j + (long long)mf.nny * k);
-        for (int f = 0; f < 4; ++f)
-          if (!(maskf && maskf[f * mf.nn + n])) acc[f] += w * rf[f * mf.nn + n];
-      }
-    }
+  const double* x = rf + f * mf.nn;
+  const uint8_t* m = maskf ? maskf + f * mf.nn : nullptr;
+  double acc = 0.0;
+#pragma unroll
+  for (int s = 0; s < 27; ++s) {
+    const int dx = s % 3 - 1, dy = (s / 3) % 3 - 1, dz = s / 9 - 1;
+    const int i = 2 * I + dx, j = 2 * J + dy, k = 2 * K + dz;
+    if (i < 0 || j < 0 || k < 0 || i >= mf.nnx || j >= mf.nny || k >= nnzf) continue;
+    const double w = (dx ? 0.5 : 1.0) * (dy ? 0.5 : 1.0) * (dz ? 0.5 : 1.0);
+    const long long n = i + (long long)mf.nnx * (j + (long long)mf.nny * k);
+    const double v = x[n];
+    if (!(m && m[n])) acc += w * v;
   }
-  for (int f = 0; f < 4; ++f) rc[f * mc.nn + N] = (maskc && maskc[f * mc.nn + N]) ? 0.0 : acc[f];
+  if (maskc && maskc[G]) acc = 0.0;
+  rc[G] = acc;
+  const double ri = acc / diag[G];
+  r[G] = ri;
+  d[G] = ri * inv_theta;
 }
 
 cudaError_t launch_q1_coarsen(const MeshDev& mf, const MeshDev& mc, const uint8_t* maskf, const double* Kef,
@@ -624,12 +668,14 @@ cudaError_t launch_hmask(const MeshDev& mf, const MeshDev& mc, const uint8_t* ma
 }
 cudaError_t launch_hprolong_add(const MeshDev& mc, const MeshDev& mf, const double* xc, double* xf,
                                 const uint8_t* maskc, const uint8_t* maskf, cudaStream_t st) {
-  k_hprolong_add<<<(unsigned)((mf.nn + 255) / 256), 256, 0, st>>>(mc, mf, xc, xf, maskc, maskf); note_launch();
+  k_hprolong_add<<<(unsigned)((4 * mf.nn + 127) / 128), 128, 0, st>>>(mc, mf, xc, xf, maskc, maskf); note_launch();
   return cudaGetLastError();
 }
 cudaError_t launch_hrestrict(const MeshDev& mc, const MeshDev& mf, const double* rf, double* rc,
-                             const uint8_t* maskc, const uint8_t* maskf, cudaStream_t st) {
-  k_hrestrict<<<(unsigned)((mc.nn + 255) / 256), 256, 0, st>>>(mc, mf, rf, rc, maskc, maskf); note_launch();
+                             const uint8_t* maskc, const uint8_t* maskf, const double* diag, double inv_theta,
+                             double* r, double* d, cudaStream_t st) {
+  k_hrestrict<<<(unsigned)((4 * mc.nn + 127) / 128), 128, 0, st>>>(mc, mf, rf, rc, maskc, maskf, diag, inv_theta, r, d);
+  note_launch();
   return cudaGetLastError();
 }
 

@@ -125,6 +125,18 @@ int axpby_level(const LevelWork& w, void* y, const void* x, double a, double b, 
 
 int coarse_gmres(pff_solver* s, cudaStream_t st);
 
+// The assembled coarse level in the form of an h-level.
+HLevel coarse_level(pff_solver* s) {
+  HLevel h;
+  h.mesh = s->lv.back().L->mesh;
+  h.n = s->lv.back().n;
+  h.A = s->A;
+  h.A32 = s->A32;
+  h.diag = s->cdiag;
+  h.work = s->cwork;
+  return h;
+}
+
 int level_apply(pff_solver* s, const LevelWork& w, const void* x, void* y, cudaStream_t st) {
   if (s->transpose) return pff_jacobian_transpose_apply(w.L, (pff_prec)w.prec, x, y, st);
   return pff_jacobian_apply(w.L, (pff_prec)w.prec, x, y, st);
@@ -163,44 +175,81 @@ int cheb_level(pff_solver* s, LevelWork& w, int degree, double lmin, double lmax
   return PFF_OK;
 }
 
-// Products with the assembled coarse level: FP64, or with the mixed solver
-// the FP32 copy of the stencil (the coarse level only preconditions; the
-// transposed product of the adjoint stays FP64).
-int coarse_spmv(pff_solver* s, const MeshDev& mc, const double* x, double* y, cudaStream_t st) {
-  if (s->transpose) S_CK(launch_q1_spmv_t(mc, s->A, x, y, st));
-  else if (s->A32) S_CK(launch_q1_spmv32(mc, s->A32, x, y, st));
-  else S_CK(launch_q1_spmv(mc, s->A, x, y, st));
+// Stencil product of an assembled level with the update that consumes it: the
+// FP64 stencil, or with the mixed solver its FP32 copy (the coarse level only
+// preconditions; the transposed product of the adjoint stays FP64).
+int h_stencil(pff_solver* s, const HLevel& h, int mode, StencilArgs a, cudaStream_t st) {
+  const bool f32 = h.A32 && !s->transpose;
+  a.mesh = h.mesh;
+  a.A = f32 ? (const void*)h.A32 : (const void*)h.A;
+  a.diag = h.diag;
+  S_CK(launch_q1_stencil(mode, f32, s->transpose != 0, a, st));
   return PFF_OK;
+}
+int h_spmv(pff_solver* s, const HLevel& h, const double* x, double* y, cudaStream_t st) {
+  StencilArgs a{};
+  a.v = x;
+  a.y = y;
+  return h_stencil(s, h, kStProduct, a, st);
+}
+
+// Chebyshev-Jacobi smoothing (Saad, Alg. 12.1) of A x = b on an assembled
+// level, degree - 1 products, each with its updates in one kernel.  from_zero:
+// x = 0 on entry (its contents are not read) and h.work already holds
+// r = D^-1 b and d = r / theta (launch_hrestrict or launch_cheb_zero).
+int h_cheb(pff_solver* s, HLevel& h, const double* b, double* x, int degree, double lmin, double lmax, bool from_zero,
+           cudaStream_t st) {
+  const long long n = h.n;
+  double *r = h.work, *d = h.work + n, *dn = h.work + 2 * n;
+  const double theta = 0.5 * (lmax + lmin), delta = 0.5 * (lmax - lmin), sigma = theta / delta;
+  double rho = 1.0 / sigma;
+  StencilArgs a{};
+  a.b = b;
+  a.x = x;
+  a.r = r;
+  if (!from_zero) {
+    a.v = x;
+    a.y = d;
+    a.cr = 1.0 / theta;
+    S_RC(h_stencil(s, h, kStChebInit, a, st));
+  }
+  if (degree == 1) {
+    if (from_zero) S_CK(cudaMemcpyAsync(x, d, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
+    else S_CK(launch_axpby<double>(x, d, 1.0, 1.0, n, st));
+  }
+  for (int k = 0; k + 1 < degree; ++k) {
+    const double rho_new = 1.0 / (2.0 * sigma - rho);
+    a.v = d;
+    a.y = dn;
+    a.cd = rho_new * rho;
+    a.cr = 2.0 * rho_new / delta;
+    a.xset = from_zero && k == 0;
+    a.last = k + 2 == degree;
+    S_RC(h_stencil(s, h, kStChebStep, a, st));
+    std::swap(d, dn);
+    rho = rho_new;
+  }
+  return PFF_OK;
+}
+
+// Smoothing interval of h-level l: [lo, cheb_hi] lambda_max, with the coarsest
+// grid's lower end; 1 / theta of it.
+double h_inv_theta(const pff_solver* s, size_t l) {
+  const double lo = l + 1 == s->hl.size() ? s->prm.coarse_lo : s->prm.cheb_lo;
+  return 2.0 / (s->hl[l].lmax * (s->prm.cheb_hi + lo));
 }
 
 int coarse_cheb(pff_solver* s, cudaStream_t st) {
   if (s->prm.coarse_solver >= 1) return coarse_gmres(s, st);
   // FP64 Chebyshev-Jacobi on the assembled coarse operator, from x = 0.
   LevelWork& c = s->lv.back();
-  const MeshDev& mc = c.L->mesh;
   const long long n = c.n;
-  double* r = s->cwork;
-  double* d = s->cwork + n;
-  double* Ad = s->cwork + 2 * n;
+  HLevel h = coarse_level(s);
   if (c.prec == PFF_F64) S_CK(cudaMemcpyAsync(s->cb, c.b, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
   else S_CK(launch_f2d(s->cb, (const float*)c.b, n, st));
-  S_CK(cudaMemsetAsync(s->cx, 0, sizeof(double) * n, st));
   const double lmax = s->clmax * s->prm.cheb_hi, lmin = s->clmax * s->prm.coarse_lo;
-  const double theta = 0.5 * (lmax + lmin), delta = 0.5 * (lmax - lmin), sigma = theta / delta;
-  double rho = 1.0 / sigma;
-  S_CK(cudaMemsetAsync(Ad, 0, sizeof(double) * n, st));
-  S_CK(launch_cheb_init<double>(n, s->cb, Ad, s->cdiag, r, d, 1.0 / theta, st));
-  const int deg = s->prm.coarse_degree;
-  for (int k = 0; k < deg; ++k) {
-    if (k == deg - 1) {
-      S_CK(launch_cheb_step<double>(n, s->cx, d, r, Ad, s->cdiag, 0.0, 0.0, 1, st));
-      break;
-    }
-    S_RC(coarse_spmv(s, mc, d, Ad, st));
-    const double rho_new = 1.0 / (2.0 * sigma - rho);
-    S_CK(launch_cheb_step<double>(n, s->cx, d, r, Ad, s->cdiag, rho_new * rho, 2.0 * rho_new / delta, 0, st));
-    rho = rho_new;
-  }
+  S_CK(launch_cheb_zero<double>(n, s->cb, s->cdiag, h.work, h.work + n, 2.0 / (lmax + lmin), st));
+  S_RC(h_cheb(s, h, s->cb, s->cx, s->prm.coarse_degree, lmin, lmax, true, st));
   if (c.prec == PFF_F64) S_CK(cudaMemcpyAsync(c.x, s->cx, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
   else S_CK(launch_d2f((float*)c.x, s->cx, n, st));
   return PFF_OK;
@@ -229,58 +278,34 @@ int vcycle(pff_solver* s, int l, cudaStream_t st) {
 }
 
 // ---- geometric h-multigrid on the assembled order-1 grid ------------------
-int h_spmv(pff_solver* s, const HLevel& h, const double* x, double* y, cudaStream_t st) {
-  if (s->transpose) S_CK(launch_q1_spmv_t(h.mesh, h.A, x, y, st));
-  else if (h.A32) S_CK(launch_q1_spmv32(h.mesh, h.A32, x, y, st));
-  else S_CK(launch_q1_spmv(h.mesh, h.A, x, y, st));
-  return PFF_OK;
-}
-
-// Chebyshev-Jacobi (Saad, Alg. 12.1) on an assembled level, from x = 0 or from
-// the given x.
-int h_cheb(pff_solver* s, HLevel& h, int degree, double lmin, double lmax, bool zero_init, cudaStream_t st) {
-  const long long n = h.n;
-  double* r = h.work;
-  double* d = h.work + n;
-  double* Ad = h.work + 2 * n;
-  const double theta = 0.5 * (lmax + lmin), delta = 0.5 * (lmax - lmin), sigma = theta / delta;
-  double rho = 1.0 / sigma;
-  if (zero_init) {
-    S_CK(cudaMemsetAsync(h.x, 0, sizeof(double) * n, st));
-    S_CK(cudaMemsetAsync(Ad, 0, sizeof(double) * n, st));
-  } else {
-    S_RC(h_spmv(s, h, h.x, Ad, st));
-  }
-  S_CK(launch_cheb_init<double>(n, h.b, Ad, h.diag, r, d, 1.0 / theta, st));
-  for (int k = 0; k < degree; ++k) {
-    if (k == degree - 1) {
-      S_CK(launch_cheb_step<double>(n, h.x, d, r, Ad, h.diag, 0.0, 0.0, 1, st));
-      break;
-    }
-    S_RC(h_spmv(s, h, d, Ad, st));
-    const double rho_new = 1.0 / (2.0 * sigma - rho);
-    S_CK(launch_cheb_step<double>(n, h.x, d, r, Ad, h.diag, rho_new * rho, 2.0 * rho_new / delta, 0, st));
-    rho = rho_new;
-  }
-  return PFF_OK;
-}
-
-// V-cycle on h-level l for A_l x = b_l (x from zero): Chebyshev pre- and
-// post-smoothing, residual restriction by P^T, coarse correction, trilinear
-// prolongation; the coarsest grid takes Chebyshev(coarse_degree).
-int hcycle(pff_solver* s, int l, cudaStream_t st) {
+// V-cycle on h-level l for A_l x = b (x from zero; h.work holds the first
+// smoothing vectors, see h_cheb): Chebyshev pre- and post-smoothing, residual
+// restriction by P^T, coarse correction, trilinear prolongation; the coarsest
+// grid takes Chebyshev(coarse_degree).
+int hcycle(pff_solver* s, int l, const double* b, double* x, cudaStream_t st) {
   HLevel& h = s->hl[l];
   const pff_solver_params& p = s->prm;
   if (l + 1 == (int)s->hl.size())
-    return h_cheb(s, h, p.coarse_degree, p.coarse_lo * h.lmax, p.cheb_hi * h.lmax, true, st);
-  S_RC(h_cheb(s, h, p.cheb_degree, p.cheb_lo * h.lmax, p.cheb_hi * h.lmax, true, st));
-  S_RC(h_spmv(s, h, h.x, h.r, st));
-  S_CK(launch_bminus<double>(h.r, h.b, h.n, st));
+    return h_cheb(s, h, b, x, p.coarse_degree, p.coarse_lo * h.lmax, p.cheb_hi * h.lmax, true, st);
+  S_RC(h_cheb(s, h, b, x, p.cheb_degree, p.cheb_lo * h.lmax, p.cheb_hi * h.lmax, true, st));
+  StencilArgs a{};
+  a.v = x;
+  a.b = b;
+  a.y = h.r;
+  S_RC(h_stencil(s, h, kStResidual, a, st));
   HLevel& c = s->hl[l + 1];
-  S_CK(launch_hrestrict(c.mesh, h.mesh, h.r, c.b, c.mask, h.mask, st));
-  S_RC(hcycle(s, l + 1, st));
-  S_CK(launch_hprolong_add(c.mesh, h.mesh, c.x, h.x, c.mask, h.mask, st));
-  return h_cheb(s, h, p.cheb_degree, p.cheb_lo * h.lmax, p.cheb_hi * h.lmax, false, st);
+  S_CK(launch_hrestrict(c.mesh, h.mesh, h.r, c.b, c.mask, h.mask, c.diag, h_inv_theta(s, l + 1), c.work, c.work + c.n,
+                        st));
+  S_RC(hcycle(s, l + 1, c.b, c.x, st));
+  S_CK(launch_hprolong_add(c.mesh, h.mesh, c.x, x, c.mask, h.mask, st));
+  return h_cheb(s, h, b, x, p.cheb_degree, p.cheb_lo * h.lmax, p.cheb_hi * h.lmax, false, st);
+}
+
+// One V-cycle x = M_h^-1 b on h-level 0 (x and b distinct).
+int hcycle_top(pff_solver* s, const double* b, double* x, cudaStream_t st) {
+  HLevel& h = s->hl[0];
+  S_CK(launch_cheb_zero<double>(h.n, b, h.diag, h.work, h.work + h.n, h_inv_theta(s, 0), st));
+  return hcycle(s, 0, b, x, st);
 }
 
 // Spectral radius of a small dense matrix (row-major k x k) by power iteration
@@ -377,16 +402,17 @@ int arnoldi_level(pff_solver* s, LevelWork& w, cudaStream_t st) {
 
 int arnoldi_hlevel(pff_solver* s, HLevel& h, cudaStream_t st) {
   auto op = [&](const double* vj, double* wv) -> int {
-    S_RC(h_spmv(s, h, vj, wv, st));
-    S_CK(launch_dscale<double>(wv, wv, h.diag, h.n, st));
-    return PFF_OK;
+    StencilArgs a{};
+    a.v = vj;
+    a.y = wv;
+    return h_stencil(s, h, kStScaled, a, st);
   };
   return arnoldi_lmax(s, h.n, op, &h.lmax, st);
 }
 
 int power_coarse(pff_solver* s, cudaStream_t st) {
-  LevelWork& c = s->lv.back();
-  const long long n = c.n;
+  const HLevel lev = coarse_level(s);
+  const long long n = lev.n;
   double* v = s->cx;
   double* y = s->cb;
   S_CK(cudaMemcpyAsync(v, s->pw64, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
@@ -395,8 +421,10 @@ int power_coarse(pff_solver* s, cudaStream_t st) {
   S_CK(launch_axpby<double>(v, v, 1.0 / std::sqrt(h), 0.0, n, st));
   double lam = 1.0;
   for (int it = 0; it < s->prm.power_iters; ++it) {
-    S_RC(coarse_spmv(s, c.L->mesh, v, y, st));
-    S_CK(launch_dscale<double>(y, y, s->cdiag, n, st));
+    StencilArgs a{};
+    a.v = v;
+    a.y = y;
+    S_RC(h_stencil(s, lev, kStScaled, a, st));
     S_RC(dev_dots(s, y, 0, 1, y, n, &h, st));
     lam = std::sqrt(h);
     if (!(lam > 0.0) || !std::isfinite(lam)) return sfail(PFF_ERR_DEVICE, "coarse power iteration failed");
@@ -547,7 +575,7 @@ int precondition(pff_solver* s, const double* v, double* z, cudaStream_t st) {
 // (coarse_solver 1) or by one h-multigrid V-cycle (coarse_solver 2).
 int coarse_gmres(pff_solver* s, cudaStream_t st) {
   LevelWork& c = s->lv.back();
-  const MeshDev& mc = c.L->mesh;
+  const HLevel lev = coarse_level(s);
   const long long n = c.n;
   if (c.prec == PFF_F64) S_CK(cudaMemcpyAsync(s->cb, c.b, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
   else S_CK(launch_f2d(s->cb, (const float*)c.b, n, st));
@@ -556,15 +584,9 @@ int coarse_gmres(pff_solver* s, cudaStream_t st) {
   kw.m = s->prm.krylov_restart;
   kw.V = s->cV;
   kw.Z = s->cZ;
-  auto A = [&](const double* in, double* out) -> int { return coarse_spmv(s, mc, in, out, st); };
+  auto A = [&](const double* in, double* out) -> int { return h_spmv(s, lev, in, out, st); };
   auto M = [&](const double* in, double* out) -> int {
-    if (s->prm.coarse_solver == 2) {  // one h-multigrid V-cycle
-      HLevel& h0 = s->hl[0];
-      S_CK(cudaMemcpyAsync(h0.b, in, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
-      S_RC(hcycle(s, 0, st));
-      S_CK(cudaMemcpyAsync(out, h0.x, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
-      return PFF_OK;
-    }
+    if (s->prm.coarse_solver == 2) return hcycle_top(s, in, out, st);
     S_CK(launch_dscale<double>(out, in, s->cdiag, n, st));
     return PFF_OK;
   };
@@ -829,7 +851,12 @@ int pff_solver_vcycle(pff_solver* s, const double* r, double* z, void* stream) {
 
 int pff_solver_coarse_apply(pff_solver* s, const double* x, double* y, void* stream) {
   if (!s || !x || !y || !s->assembled) return sfail(PFF_ERR_INVALID, "pff_solver_coarse_apply: needs an assembled coarse level");
-  S_CK(launch_q1_spmv(s->lv.back().L->mesh, s->A, x, y, reinterpret_cast<cudaStream_t>(stream)));
+  StencilArgs a{};
+  a.mesh = s->lv.back().L->mesh;
+  a.A = s->A;
+  a.v = x;
+  a.y = y;
+  S_CK(launch_q1_stencil(kStProduct, false, false, a, reinterpret_cast<cudaStream_t>(stream)));
   return PFF_OK;
 }
 
@@ -847,7 +874,12 @@ int pff_solver_hlevel_info(const pff_solver* s, int level, int* dims, double* lm
 int pff_solver_hlevel_apply(pff_solver* s, int level, const double* x, double* y, void* stream) {
   if (!s || !x || !y || level < 0 || level >= (int)s->hl.size())
     return sfail(PFF_ERR_INVALID, "pff_solver_hlevel_apply: bad argument");
-  S_CK(launch_q1_spmv(s->hl[level].mesh, s->hl[level].A, x, y, reinterpret_cast<cudaStream_t>(stream)));
+  StencilArgs a{};
+  a.mesh = s->hl[level].mesh;
+  a.A = s->hl[level].A;
+  a.v = x;
+  a.y = y;
+  S_CK(launch_q1_stencil(kStProduct, false, false, a, reinterpret_cast<cudaStream_t>(stream)));
   return PFF_OK;
 }
 
@@ -856,7 +888,7 @@ int pff_solver_hcycle(pff_solver* s, const double* b, double* x, void* stream) {
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   HLevel& h0 = s->hl[0];
   S_CK(cudaMemcpyAsync(h0.b, b, sizeof(double) * h0.n, cudaMemcpyDeviceToDevice, st));
-  S_RC(hcycle(s, 0, st));
+  S_RC(hcycle_top(s, h0.b, h0.x, st));
   S_CK(cudaMemcpyAsync(x, h0.x, sizeof(double) * h0.n, cudaMemcpyDeviceToDevice, st));
   return PFF_OK;
 }

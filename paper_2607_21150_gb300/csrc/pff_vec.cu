@@ -368,6 +368,16 @@ __global__ void k_cheb_init(long long n, const T* __restrict__ b, const T* __res
     d[i] = ri * inv_theta;
   }
 }
+// init from x = 0: r = D^-1 b, d = r / theta
+template <typename T>
+__global__ void k_cheb_zero(long long n, const T* __restrict__ b, const T* __restrict__ diag, T* __restrict__ r,
+                            T* __restrict__ d, T inv_theta) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const T ri = b[i] / diag[i];
+    r[i] = ri;
+    d[i] = ri * inv_theta;
+  }
+}
 template <typename T>
 __global__ void k_cheb_step(long long n, T* __restrict__ x, T* __restrict__ d, T* __restrict__ r,
                             const T* __restrict__ Ad, const T* __restrict__ diag, T c_d, T c_r, int last) {
@@ -389,6 +399,16 @@ cudaError_t launch_cheb_init(long long n, const T* b, const T* Ax, const T* diag
   k_cheb_init<T><<<grid_for(n), kVecThreads, 0, st>>>(n, b, Ax, diag, r, d, (T)inv_theta); note_launch();
   return cudaGetLastError();
 }
+template <typename T>
+cudaError_t launch_cheb_zero(long long n, const T* b, const T* diag, T* r, T* d, double inv_theta, cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  k_cheb_zero<T><<<grid_for(n), kVecThreads, 0, st>>>(n, b, diag, r, d, (T)inv_theta); note_launch();
+  return cudaGetLastError();
+}
+template cudaError_t launch_cheb_zero<double>(long long, const double*, const double*, double*, double*, double,
+                                              cudaStream_t);
+template cudaError_t launch_cheb_zero<float>(long long, const float*, const float*, float*, float*, double,
+                                             cudaStream_t);
 template <typename T>
 cudaError_t launch_cheb_step(long long n, T* x, T* d, T* r, const T* Ad, const T* diag, double c_d, double c_r,
                              int last, cudaStream_t st) {
