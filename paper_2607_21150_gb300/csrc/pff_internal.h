@@ -275,19 +275,40 @@ template <typename T>
 cudaError_t launch_cheb_init(long long n, const T* b, const T* Ax, const T* diag, T* r, T* d,
                              double inv_theta, cudaStream_t st);
 template <typename T>
+cudaError_t launch_cheb_zero(long long n, const T* b, const T* diag, T* r, T* d, double inv_theta, cudaStream_t st);
+template <typename T>
 cudaError_t launch_cheb_step(long long n, T* x, T* d, T* r, const T* Ad, const T* diag,
                              double c_d, double c_r, int last, cudaStream_t st);
 
 
 // Krylov vectors and the assembled coarse operator (pff_krylov.cu)
 constexpr int kReduceBlocks = 152 * 4;
-// out[j] = V_j . w for j < k (vectors V_j at stride ldv), FP64 accumulation in a
-// fixed order; partial needs k * kReduceBlocks doubles.
+constexpr int kMaxDots = 64;
+// Scalars of one set of dot products (device, with a copy in page-locked host
+// memory whose seq is written last).
+struct DotScalars {
+  double dot[kMaxDots];
+  double ww2;   // the last dot, less the squares of the others (gs), not negative
+  double inv;   // 1 / sqrt(ww2), 0 where ww2 = 0
+  int second;   // the subtraction cancelled more than half: a second pass is due
+  unsigned long long seq;
+};
+struct LinCoef {
+  double c[kMaxDots];
+};
+// out->dot[j] = V_j . w for j < k <= 62 (vectors V_j at stride ldv), FP64
+// accumulation in a fixed order; partial needs k * kReduceBlocks doubles,
+// *arrived is 0 between calls (one call at a time).  host: device-visible
+// page-locked copy, seq its sequence number.
 template <typename TV, typename T>
-cudaError_t launch_mdot(const TV* V, long long ldv, int k, const T* w, long long n, double* partial, double* out,
+cudaError_t launch_mdot(const TV* V, long long ldv, int k, const T* w, long long n, double* partial, unsigned* arrived,
+                        int gs, const DotScalars* gate, DotScalars* out, DotScalars* host, unsigned long long seq,
                         cudaStream_t st);
-cudaError_t launch_maxpy(double* w, const double* V, long long ldv, int k, const double* h, double sign, long long n,
-                         cudaStream_t st);
+cudaError_t launch_gs_update(double* w, const double* V, long long ldv, int k, const DotScalars* sc,
+                             const DotScalars* gate, long long n, cudaStream_t st);
+cudaError_t launch_normalise(double* y, const double* x, const DotScalars* sc, long long n, cudaStream_t st);
+cudaError_t launch_lincomb(double* x, const double* Z, long long ldz, int k, const LinCoef& c, int add, long long n,
+                           cudaStream_t st);
 template <typename T>
 cudaError_t launch_axpby(T* y, const T* x, double a, double b, long long n, cudaStream_t st);
 template <typename T>
@@ -307,13 +328,15 @@ enum StencilMode { kStProduct, kStScaled, kStResidual, kStChebInit, kStChebStep 
 struct StencilArgs {
   MeshDev mesh;
   const void* A;
-  const double *v, *b, *diag;
+  const double *v, *b, *dinv;  // dinv = D^-1
   double *y, *r, *x;
   double cd, cr;
   int xset, last;
 };
 cudaError_t launch_q1_stencil(int mode, bool f32, bool transpose, const StencilArgs& a, cudaStream_t st);
-cudaError_t launch_q1_diag(const MeshDev& mc, const double* A, double* d, cudaStream_t st);
+cudaError_t launch_q1_dinv(const MeshDev& mc, const double* A, double* d, cudaStream_t st);
+cudaError_t launch_jacobi(long long n, const double* b, const double* dinv, double* r, double* d, double c,
+                          cudaStream_t st);
 // Sum-factorised element matrices (Ke: [nel][32][32] work space) and a
 // deterministic gather into the stencil storage.
 // lin32 not null: from the FP32 words (quad layout) in FP32 arithmetic (the
@@ -333,11 +356,8 @@ cudaError_t launch_hprolong_add(const MeshDev& mc, const MeshDev& mf, const doub
                                 const uint8_t* maskc, const uint8_t* maskf, cudaStream_t st);
 // ... and the coarse level's first smoothing vectors r = D^-1 r_c, d = inv_theta r.
 cudaError_t launch_hrestrict(const MeshDev& mc, const MeshDev& mf, const double* rf, double* rc,
-                             const uint8_t* maskc, const uint8_t* maskf, const double* diag, double inv_theta,
+                             const uint8_t* maskc, const uint8_t* maskf, const double* dinv, double inv_theta,
                              double* r, double* d, cudaStream_t st);
-// The same from a given b (vectors of n entries).
-template <typename T>
-cudaError_t launch_cheb_zero(long long n, const T* b, const T* diag, T* r, T* d, double inv_theta, cudaStream_t st);
 cudaError_t launch_sel_scale(double* y, const uint8_t* sel, double s, long long n, cudaStream_t st);
 cudaError_t launch_zero_masked(double* y, const uint8_t* mask, long long n, cudaStream_t st);
 

@@ -11,90 +11,171 @@ constexpr int kRedThreads = 256;
 constexpr int kRedBlocks = kReduceBlocks;
 
 // ---------------------------------------------------------------- reductions
-// partial[j * kRedBlocks + b] = block b's share of sum_i V_j[i] w[i], j < k.
-// Vectors are taken in chunks of CH so that w is read once per chunk (long
-// vectors: HBM traffic k + k / CH instead of 2 k vectors); short vectors live
-// in L2 and take CH = 1, which keeps fewer registers and barriers per pass.
-template <typename TV, typename T, int CH>
-__global__ void __launch_bounds__(kRedThreads) k_mdot_partial(const TV* __restrict__ V, long long ldv, int k,
-                                                              const T* __restrict__ w, long long n,
-                                                              double* __restrict__ partial) {
-  __shared__ double red[CH][kRedThreads / 32];
-  for (int j0 = 0; j0 < k; j0 += CH) {
-    double s[CH];
+// out[j] = sum_i V_j[i] w[i], j < k, in one launch: every block leaves its
+// share of each dot in partial, and the block that arrives last sums the shares
+// in a fixed order and, for the orthogonalisation of w = V_(k-1) (gs), derives
+// what the update needs: ||w||^2 after the projection, whether the projection
+// cancelled more than half of ||w||^2 (a second pass is then due), 1 / norm.
+// The scalars stay on the device for the update kernel and go to page-locked
+// host memory, sequence number last, for the host's Hessenberg matrix: no copy,
+// no second launch and no upload of the coefficients (they took 14.6 + 2.9 us
+// of kernels and two copies per orthogonalisation on 17^3 nodes).
+// Vectors are taken in chunks of eight so that w is read once per chunk.
+// gate: do nothing unless the gate scalars ask for a second pass.
+constexpr int kDotChunk = 8;
+template <typename TV, typename T>
+__global__ void __launch_bounds__(kRedThreads) k_mdot(const TV* __restrict__ V, long long ldv, int k,
+                                                      const T* __restrict__ w, long long n,
+                                                      double* __restrict__ partial, unsigned* __restrict__ arrived,
+                                                      int gs, const DotScalars* __restrict__ gate,
+                                                      DotScalars* __restrict__ out, volatile DotScalars* host,
+                                                      unsigned long long seq) {
+  if (gate && !gate->second) return;
+  __shared__ double red[kDotChunk][kRedThreads / 32];
+  __shared__ bool is_last;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nb = gridDim.x;
+  for (int j0 = 0; j0 < k; j0 += kDotChunk) {
+    double s[kDotChunk];
 #pragma unroll
-    for (int c = 0; c < CH; ++c) s[c] = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-      const double wi = (double)w[i];
+    for (int c = 0; c < kDotChunk; ++c) s[c] = 0.0;
+    const long long stride = (long long)nb * kRedThreads;
+    if (j0 + kDotChunk <= k) {
+#pragma unroll 2
+      for (long long i = blockIdx.x * (long long)kRedThreads + t; i < n; i += stride) {
+        const double wi = (double)w[i];
 #pragma unroll
-      for (int c = 0; c < CH; ++c)
-        if (j0 + c < k) s[c] += (double)V[(j0 + c) * ldv + i] * wi;
+        for (int c = 0; c < kDotChunk; ++c) s[c] += (double)V[(j0 + c) * ldv + i] * wi;
+      }
+    } else {
+#pragma unroll 2
+      for (long long i = blockIdx.x * (long long)kRedThreads + t; i < n; i += stride) {
+        const double wi = (double)w[i];
+#pragma unroll
+        for (int c = 0; c < kDotChunk; ++c)
+          if (j0 + c < k) s[c] += (double)V[(j0 + c) * ldv + i] * wi;
+      }
     }
 #pragma unroll
-    for (int c = 0; c < CH; ++c) {
-      double t = s[c];
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-      if ((threadIdx.x & 31) == 0) red[c][threadIdx.x >> 5] = t;
+    for (int c = 0; c < kDotChunk; ++c) {
+      double v = s[c];
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      if (lane == 0) red[c][warp] = v;
     }
     __syncthreads();
-    if (threadIdx.x < CH && j0 + (int)threadIdx.x < k) {
-      double t = 0.0;
-      for (int wp = 0; wp < kRedThreads / 32; ++wp) t += red[threadIdx.x][wp];
-      partial[(j0 + threadIdx.x) * kRedBlocks + blockIdx.x] = t;
+    if (t < kDotChunk && j0 + t < k) {
+      double v = 0.0;
+      for (int wp = 0; wp < kRedThreads / 32; ++wp) v += red[t][wp];
+      partial[(j0 + t) * kRedBlocks + blockIdx.x] = v;
     }
     __syncthreads();
   }
-}
-// out[j] = sum_b partial[j * kRedBlocks + b] (one block per j, fixed order).
-__global__ void k_mdot_final(const double* __restrict__ partial, int k, double* __restrict__ out) {
-  __shared__ double red[32];
-  const int j = blockIdx.x;
-  double s = 0.0;
-  for (int b = threadIdx.x; b < kRedBlocks; b += blockDim.x) s += partial[j * kRedBlocks + b];
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __threadfence();
   __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = (threadIdx.x < (int)(blockDim.x / 32)) ? red[threadIdx.x] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if (threadIdx.x == 0) out[j] = t;
+  if (t == 0) is_last = atomicAdd(arrived, 1u) == (unsigned)nb - 1;
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+  __shared__ double dot[kMaxDots];
+  for (int j = warp; j < k; j += kRedThreads / 32) {
+    double v = 0.0;
+    for (int b = lane; b < nb; b += 32) v += __ldcg(partial + j * kRedBlocks + b);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) {
+      dot[j] = v;
+      out->dot[j] = v;
+      host->dot[j] = v;
+      __threadfence_system();  // before thread 0 publishes the sequence number
+    }
   }
+  __syncthreads();
+  if (t != 0) return;
+  *arrived = 0u;
+  const double ww = dot[k - 1];
+  double ww2 = ww;
+  if (gs) {
+    double hsq = 0.0;
+    for (int j = 0; j + 1 < k; ++j) hsq += dot[j] * dot[j];
+    ww2 = ww - hsq;
+    ww2 = ww2 < 0.0 ? 0.0 : ww2;
+  }
+  const int second = gs && !gate && ww2 < 0.5 * ww;
+  out->ww2 = ww2;
+  out->inv = ww2 > 0.0 ? 1.0 / sqrt(ww2) : 0.0;
+  out->second = second;
+  host->ww2 = ww2;
+  host->second = second;
+  __threadfence_system();
+  host->seq = seq;
 }
 
 template <typename TV, typename T>
-cudaError_t launch_mdot(const TV* V, long long ldv, int k, const T* w, long long n, double* partial, double* out,
+cudaError_t launch_mdot(const TV* V, long long ldv, int k, const T* w, long long n, double* partial, unsigned* arrived,
+                        int gs, const DotScalars* gate, DotScalars* out, DotScalars* host, unsigned long long seq,
                         cudaStream_t st) {
   if (k <= 0) return cudaSuccess;
-  if (n >= (1LL << 22))
-    k_mdot_partial<TV, T, 8><<<kRedBlocks, kRedThreads, 0, st>>>(V, ldv, k, w, n, partial);
-  else
-    k_mdot_partial<TV, T, 1><<<kRedBlocks, kRedThreads, 0, st>>>(V, ldv, k, w, n, partial);
+  long long nb = (n + 4 * kRedThreads - 1) / (4 * kRedThreads);
+  nb = nb < 1 ? 1 : nb > kRedBlocks ? kRedBlocks : nb;
+  k_mdot<TV, T><<<(unsigned)nb, kRedThreads, 0, st>>>(V, ldv, k, w, n, partial, arrived, gs, gate, out, host, seq);
   note_launch();
-  k_mdot_final<<<k, 256, 0, st>>>(partial, k, out); note_launch();
   return cudaGetLastError();
 }
 template cudaError_t launch_mdot<double, double>(const double*, long long, int, const double*, long long, double*,
-                                                 double*, cudaStream_t);
-template cudaError_t launch_mdot<float, float>(const float*, long long, int, const float*, long long, double*,
-                                               double*, cudaStream_t);
+                                                 unsigned*, int, const DotScalars*, DotScalars*, DotScalars*,
+                                                 unsigned long long, cudaStream_t);
 
 // ---------------------------------------------------------------- vector updates
-// w -= sum_j h[j] V_j   (h on the device, k <= 64)
-__global__ void k_maxpy(double* __restrict__ w, const double* __restrict__ V, long long ldv, int k,
-                        const double* __restrict__ h, double sign, long long n) {
-  __shared__ double hs[64];
-  if (threadIdx.x < k) hs[threadIdx.x] = h[threadIdx.x];
+// Orthogonalisation step: w -= sum_j dot[j] V_j with the scalars of launch_mdot
+// (k <= 62), normalised unless a second pass follows.  gate as in launch_mdot.
+__global__ void __launch_bounds__(256) k_gs_update(double* __restrict__ w, const double* __restrict__ V, long long ldv,
+                                                   int k, const DotScalars* __restrict__ sc,
+                                                   const DotScalars* __restrict__ gate, long long n) {
+  if (gate && !gate->second) return;
+  __shared__ double hs[kMaxDots];
+  if (threadIdx.x < k) hs[threadIdx.x] = sc->dot[threadIdx.x];
+  const double scale = sc->second || sc->inv == 0.0 ? 1.0 : sc->inv;
   __syncthreads();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     double s = w[i];
-    for (int j = 0; j < k; ++j) s += sign * hs[j] * V[j * ldv + i];
-    w[i] = s;
+#pragma unroll 4
+    for (int j = 0; j < k; ++j) s -= hs[j] * V[j * ldv + i];
+    w[i] = s * scale;
   }
 }
-cudaError_t launch_maxpy(double* w, const double* V, long long ldv, int k, const double* h, double sign, long long n,
-                         cudaStream_t st) {
-  if (k <= 0 || n == 0) return cudaSuccess;
-  k_maxpy<<<kRedBlocks * 2, 256, 0, st>>>(w, V, ldv, k, h, sign, n); note_launch();
+static unsigned vec_blocks(long long n) {
+  const long long nb = (n + 255) / 256;
+  return (unsigned)(nb < kRedBlocks * 4 ? nb : kRedBlocks * 4);
+}
+cudaError_t launch_gs_update(double* w, const double* V, long long ldv, int k, const DotScalars* sc,
+                             const DotScalars* gate, long long n, cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  k_gs_update<<<vec_blocks(n), 256, 0, st>>>(w, V, ldv, k, sc, gate, n); note_launch();
+  return cudaGetLastError();
+}
+// y = x / norm with the norm's scalars (y may be x); the zero vector stays zero.
+__global__ void k_normalise(double* y, const double* x, const DotScalars* __restrict__ sc, long long n) {
+  const double inv = sc->inv;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    y[i] = x[i] * inv;
+}
+cudaError_t launch_normalise(double* y, const double* x, const DotScalars* sc, long long n, cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  k_normalise<<<vec_blocks(n), 256, 0, st>>>(y, x, sc, n); note_launch();
+  return cudaGetLastError();
+}
+// x = (add ? x : 0) + sum_j c[j] Z_j, the coefficients as kernel parameters.
+__global__ void __launch_bounds__(256) k_lincomb(double* __restrict__ x, const double* __restrict__ Z, long long ldz,
+                                                 int k, const LinCoef c, int add, long long n) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    double s = add ? x[i] : 0.0;
+#pragma unroll 4
+    for (int j = 0; j < k; ++j) s += c.c[j] * Z[j * ldz + i];
+    x[i] = s;
+  }
+}
+cudaError_t launch_lincomb(double* x, const double* Z, long long ldz, int k, const LinCoef& c, int add, long long n,
+                           cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  k_lincomb<<<vec_blocks(n), 256, 0, st>>>(x, Z, ldz, k, c, add, n); note_launch();
   return cudaGetLastError();
 }
 
@@ -206,7 +287,7 @@ __global__ void __launch_bounds__(kStThreads) k_q1_stencil(const StencilArgs a) 
   double b = 0.0, dg = 1.0, r = 0.0, v = 0.0, x = 0.0;
   if (owner) {
     if (MODE == kStResidual || MODE == kStChebInit) b = a.b[i];
-    if (MODE == kStScaled || MODE == kStChebInit || MODE == kStChebStep) dg = a.diag[i];
+    if (MODE == kStScaled || MODE == kStChebInit || MODE == kStChebStep) dg = a.dinv[i];
     if (MODE == kStChebStep) {
       r = a.r[i];
       v = a.v[i];
@@ -248,15 +329,15 @@ __global__ void __launch_bounds__(kStThreads) k_q1_stencil(const StencilArgs a) 
   for (int w = 0; w < kStRows; ++w) sum += red[w][row][lane];
   const double Av = st_sum(sum);
   if (MODE == kStProduct) a.y[i] = Av;
-  if (MODE == kStScaled) a.y[i] = Av / dg;
+  if (MODE == kStScaled) a.y[i] = Av * dg;
   if (MODE == kStResidual) a.y[i] = b - Av;
   if (MODE == kStChebInit) {
-    const double ri = (b - Av) / dg;
+    const double ri = (b - Av) * dg;
     a.r[i] = ri;
     a.y[i] = ri * a.cr;
   }
   if (MODE == kStChebStep) {
-    const double ri = r - Av / dg;
+    const double ri = r - Av * dg;
     const double di = a.cd * v + a.cr * ri;
     double xi = a.xset ? v : x + v;
     if (a.last) {
@@ -307,13 +388,30 @@ cudaError_t launch_zero_masked(double* y, const uint8_t* mask, long long n, cuda
   return cudaGetLastError();
 }
 
-__global__ void k_q1_diag(MeshDev mc, const double* __restrict__ A, double* __restrict__ d) {
+// Reciprocal diagonal (the smoothers multiply: an FP64 division is a chain of
+// dependent operations at the end of every product).
+__global__ void k_q1_dinv(MeshDev mc, const double* __restrict__ A, double* __restrict__ d) {
   const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (n >= mc.nn) return;
-  for (int f = 0; f < 4; ++f) d[f * mc.nn + n] = A[(long long)(13 * 16 + f * 4 + f) * mc.nn + n];
+  for (int f = 0; f < 4; ++f) d[f * mc.nn + n] = 1.0 / A[(long long)(13 * 16 + f * 4 + f) * mc.nn + n];
 }
-cudaError_t launch_q1_diag(const MeshDev& mc, const double* A, double* d, cudaStream_t st) {
-  k_q1_diag<<<(unsigned)((mc.nn + 255) / 256), 256, 0, st>>>(mc, A, d); note_launch();
+cudaError_t launch_q1_dinv(const MeshDev& mc, const double* A, double* d, cudaStream_t st) {
+  k_q1_dinv<<<(unsigned)((mc.nn + 255) / 256), 256, 0, st>>>(mc, A, d); note_launch();
+  return cudaGetLastError();
+}
+// r = dinv b (r may be null), d = c dinv b: Jacobi, and a smoother's first vectors.
+__global__ void k_jacobi(long long n, const double* __restrict__ b, const double* __restrict__ dinv,
+                         double* __restrict__ r, double* __restrict__ d, double c) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const double ri = b[i] * dinv[i];
+    if (r) r[i] = ri;
+    d[i] = ri * c;
+  }
+}
+cudaError_t launch_jacobi(long long n, const double* b, const double* dinv, double* r, double* d, double c,
+                          cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  k_jacobi<<<vec_blocks(n), 256, 0, st>>>(n, b, dinv, r, d, c); note_launch();
   return cudaGetLastError();
 }
 
@@ -622,7 +720,7 @@ __global__ void k_hprolong_add(MeshDev mc, MeshDev mf, const double* __restrict_
 // the coarse level's smoothing from x = 0: r = D^-1 r_c, d = r / theta.
 __global__ void k_hrestrict(MeshDev mc, MeshDev mf, const double* __restrict__ rf, double* __restrict__ rc,
                             const uint8_t* __restrict__ maskc, const uint8_t* __restrict__ maskf,
-                            const double* __restrict__ diag, double inv_theta, double* __restrict__ r,
+                            const double* __restrict__ dinv, double inv_theta, double* __restrict__ r,
                             double* __restrict__ d) {
   const long long G = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (G >= 4 * mc.nn) return;
@@ -644,7 +742,7 @@ __global__ void k_hrestrict(MeshDev mc, MeshDev mf, const double* __restrict__ r
   }
   if (maskc && maskc[G]) acc = 0.0;
   rc[G] = acc;
-  const double ri = acc / diag[G];
+  const double ri = acc * dinv[G];
   r[G] = ri;
   d[G] = ri * inv_theta;
 }
@@ -672,9 +770,9 @@ cudaError_t launch_hprolong_add(const MeshDev& mc, const MeshDev& mf, const doub
   return cudaGetLastError();
 }
 cudaError_t launch_hrestrict(const MeshDev& mc, const MeshDev& mf, const double* rf, double* rc,
-                             const uint8_t* maskc, const uint8_t* maskf, const double* diag, double inv_theta,
+                             const uint8_t* maskc, const uint8_t* maskf, const double* dinv, double inv_theta,
                              double* r, double* d, cudaStream_t st) {
-  k_hrestrict<<<(unsigned)((4 * mc.nn + 127) / 128), 128, 0, st>>>(mc, mf, rf, rc, maskc, maskf, diag, inv_theta, r, d);
+  k_hrestrict<<<(unsigned)((4 * mc.nn + 127) / 128), 128, 0, st>>>(mc, mf, rf, rc, maskc, maskf, dinv, inv_theta, r, d);
   note_launch();
   return cudaGetLastError();
 }

@@ -19,6 +19,7 @@
 //   seeded random-sign vector, re-estimated every eig_every Newton iterations
 //   (0: only on the first); smoothing interval [lo, hi] * lambda_max.
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -60,7 +61,7 @@ struct LevelWork {
 struct HLevel {
   MeshDev mesh;
   long long n = 0;
-  double *Ke = nullptr, *A = nullptr, *diag = nullptr;
+  double *Ke = nullptr, *A = nullptr, *dinv = nullptr;  // dinv: reciprocal diagonal
   float* A32 = nullptr;  // mixed solver: FP32 copy of A for the preconditioner's products
   const uint8_t* mask = nullptr;
   uint8_t* own_mask = nullptr;
@@ -68,6 +69,10 @@ struct HLevel {
   double lmax = 1.0;
   bool owns = false;
 };
+
+// Page-locked sets of dot scalars: six of the Krylov solves; the Arnoldi process
+// (not nested in one) uses two per step, up to 60 steps.
+constexpr int kHostSlots = 128;
 
 double now() {
   return std::chrono::duration<double>(std::chrono::steady_clock::now().time_since_epoch()).count();
@@ -80,7 +85,7 @@ struct pff_solver {
   pff_solver_params prm;
   std::vector<LevelWork> lv;
   bool assembled = false;
-  double *A = nullptr, *cdiag = nullptr, *cb = nullptr, *cx = nullptr, *cwork = nullptr;
+  double *A = nullptr, *cdinv = nullptr, *cb = nullptr, *cx = nullptr, *cwork = nullptr;
   float* A32 = nullptr;                 // mixed solver: FP32 copy of the coarse stencil
   double *cV = nullptr, *cZ = nullptr;  // coarse GMRES basis
   double* Ke = nullptr;                 // coarse element matrices [nel][32][32]
@@ -89,7 +94,11 @@ struct pff_solver {
   double clmax = 1.0;
   long long n = 0;
   double *V = nullptr, *Z = nullptr, *r = nullptr, *dz = nullptr, *zold = nullptr;
-  double *partial = nullptr, *dots = nullptr, *hdev = nullptr;
+  double* partial = nullptr;       // block shares of the dot products
+  unsigned* arrived = nullptr;     // blocks of a dot-product launch that have finished
+  DotScalars* sc = nullptr;        // six sets of dot scalars: outer Krylov (and Arnoldi), coarse Krylov
+  DotScalars *host = nullptr, *host_dev = nullptr;  // page-locked copies and their device address
+  unsigned long long seq = 0;
   double* pw64 = nullptr;  // power-iteration start vector (FP64, fine size)
   float* pw32 = nullptr;
   int transpose = 0;       // 1 while solving with J^T (adjoint)
@@ -99,21 +108,38 @@ struct pff_solver {
 
 namespace {
 
-int dev_dots(pff_solver* s, const double* V, long long ldv, int k, const double* w, long long n, double* host,
-             cudaStream_t st) {
-  S_CK((launch_mdot<double, double>(V, ldv, k, w, n, s->partial, s->dots, st)));
-  S_CK(cudaMemcpyAsync(host, s->dots, sizeof(double) * k, cudaMemcpyDeviceToHost, st));
-  S_CK(cudaStreamSynchronize(st));
+// Dot products out->dot[j] = V_j . w, j < k, with their host copy in slot
+// `slot` under a new sequence number (returned in *seq).
+int dots(pff_solver* s, const double* V, long long ldv, int k, const double* w, long long n, int gs,
+         const DotScalars* gate, DotScalars* out, int slot, unsigned long long* seq, cudaStream_t st) {
+  *seq = ++s->seq;
+  S_CK((launch_mdot<double, double>(V, ldv, k, w, n, s->partial, s->arrived, gs, gate, out, s->host_dev + slot, *seq, st)));
   return PFF_OK;
 }
 
-int norm_level(pff_solver* s, const LevelWork& w, const void* v, double* out, cudaStream_t st) {
-  if (w.prec == PFF_F64) S_CK((launch_mdot<double, double>((const double*)v, 0, 1, (const double*)v, w.n, s->partial, s->dots, st)));
-  else S_CK((launch_mdot<float, float>((const float*)v, 0, 1, (const float*)v, w.n, s->partial, s->dots, st)));
-  double h = 0.0;
-  S_CK(cudaMemcpyAsync(&h, s->dots, sizeof(double), cudaMemcpyDeviceToHost, st));
-  S_CK(cudaStreamSynchronize(st));
-  *out = std::sqrt(h);
+// Waits for the host copy of a set of dot products: polls the sequence number
+// that the kernel writes last, so that the work queued behind the products keeps
+// running; the stream is queried now and then, which also ends the wait on an
+// error.
+int wait_dots(pff_solver* s, int slot, unsigned long long seq, cudaStream_t st) {
+  const volatile DotScalars* h = s->host + slot;
+  for (unsigned it = 1; h->seq != seq; ++it) {
+    if (it % 2048) continue;
+    const cudaError_t e = cudaStreamQuery(st);
+    if (e == cudaErrorNotReady) continue;
+    if (e != cudaSuccess) return sfail(PFF_ERR_CUDA, std::string("dot products: ") + cudaGetErrorString(e));
+    if (h->seq != seq) return sfail(PFF_ERR_CUDA, "dot products: no result");
+  }
+  std::atomic_thread_fence(std::memory_order_acquire);
+  return PFF_OK;
+}
+
+// ||v||^2 on the host.
+int dev_norm2(pff_solver* s, const double* v, long long n, double* out, cudaStream_t st) {
+  unsigned long long seq;
+  S_RC(dots(s, v, 0, 1, v, n, 0, nullptr, s->sc, 0, &seq, st));
+  S_RC(wait_dots(s, 0, seq, st));
+  *out = s->host[0].dot[0];
   return PFF_OK;
 }
 
@@ -132,7 +158,7 @@ HLevel coarse_level(pff_solver* s) {
   h.n = s->lv.back().n;
   h.A = s->A;
   h.A32 = s->A32;
-  h.diag = s->cdiag;
+  h.dinv = s->cdinv;
   h.work = s->cwork;
   return h;
 }
@@ -182,7 +208,7 @@ int h_stencil(pff_solver* s, const HLevel& h, int mode, StencilArgs a, cudaStrea
   const bool f32 = h.A32 && !s->transpose;
   a.mesh = h.mesh;
   a.A = f32 ? (const void*)h.A32 : (const void*)h.A;
-  a.diag = h.diag;
+  a.dinv = h.dinv;
   S_CK(launch_q1_stencil(mode, f32, s->transpose != 0, a, st));
   return PFF_OK;
 }
@@ -196,7 +222,7 @@ int h_spmv(pff_solver* s, const HLevel& h, const double* x, double* y, cudaStrea
 // Chebyshev-Jacobi smoothing (Saad, Alg. 12.1) of A x = b on an assembled
 // level, degree - 1 products, each with its updates in one kernel.  from_zero:
 // x = 0 on entry (its contents are not read) and h.work already holds
-// r = D^-1 b and d = r / theta (launch_hrestrict or launch_cheb_zero).
+// r = D^-1 b and d = r / theta (launch_hrestrict or launch_jacobi).
 int h_cheb(pff_solver* s, HLevel& h, const double* b, double* x, int degree, double lmin, double lmax, bool from_zero,
            cudaStream_t st) {
   const long long n = h.n;
@@ -248,7 +274,7 @@ int coarse_cheb(pff_solver* s, cudaStream_t st) {
   if (c.prec == PFF_F64) S_CK(cudaMemcpyAsync(s->cb, c.b, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
   else S_CK(launch_f2d(s->cb, (const float*)c.b, n, st));
   const double lmax = s->clmax * s->prm.cheb_hi, lmin = s->clmax * s->prm.coarse_lo;
-  S_CK(launch_cheb_zero<double>(n, s->cb, s->cdiag, h.work, h.work + n, 2.0 / (lmax + lmin), st));
+  S_CK(launch_jacobi(n, s->cb, s->cdinv, h.work, h.work + n, 2.0 / (lmax + lmin), st));
   S_RC(h_cheb(s, h, s->cb, s->cx, s->prm.coarse_degree, lmin, lmax, true, st));
   if (c.prec == PFF_F64) S_CK(cudaMemcpyAsync(c.x, s->cx, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
   else S_CK(launch_d2f((float*)c.x, s->cx, n, st));
@@ -294,7 +320,7 @@ int hcycle(pff_solver* s, int l, const double* b, double* x, cudaStream_t st) {
   a.y = h.r;
   S_RC(h_stencil(s, h, kStResidual, a, st));
   HLevel& c = s->hl[l + 1];
-  S_CK(launch_hrestrict(c.mesh, h.mesh, h.r, c.b, c.mask, h.mask, c.diag, h_inv_theta(s, l + 1), c.work, c.work + c.n,
+  S_CK(launch_hrestrict(c.mesh, h.mesh, h.r, c.b, c.mask, h.mask, c.dinv, h_inv_theta(s, l + 1), c.work, c.work + c.n,
                         st));
   S_RC(hcycle(s, l + 1, c.b, c.x, st));
   S_CK(launch_hprolong_add(c.mesh, h.mesh, c.x, x, c.mask, h.mask, st));
@@ -304,7 +330,7 @@ int hcycle(pff_solver* s, int l, const double* b, double* x, cudaStream_t st) {
 // One V-cycle x = M_h^-1 b on h-level 0 (x and b distinct).
 int hcycle_top(pff_solver* s, const double* b, double* x, cudaStream_t st) {
   HLevel& h = s->hl[0];
-  S_CK(launch_cheb_zero<double>(h.n, b, h.diag, h.work, h.work + h.n, h_inv_theta(s, 0), st));
+  S_CK(launch_jacobi(h.n, b, h.dinv, h.work, h.work + h.n, h_inv_theta(s, 0), st));
   return hcycle(s, 0, b, x, st);
 }
 
@@ -339,40 +365,42 @@ double small_spectral_radius(const std::vector<double>& H, int k) {
 // w = D^-1 A v on FP64 vectors of length n.
 template <typename Op>
 int arnoldi_lmax(pff_solver* s, long long n, Op&& op, double* out, cudaStream_t st) {
+  // Nothing waits on the host between the steps: the second pass's kernels run
+  // or return at once by the first pass's scalars on the device, and the
+  // Hessenberg matrix is put together from the host copies at the end.
   const int k = std::min(s->prm.power_iters, s->prm.krylov_restart);
   double* V = s->V;  // (restart + 1) fine vectors >= (k + 1) level vectors
-  S_CK(cudaMemcpyAsync(V, s->pw64, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
-  double h0;
-  S_RC(dev_dots(s, V, 0, 1, V, n, &h0, st));
-  S_CK(launch_axpby<double>(V, V, 1.0 / std::sqrt(h0), 0.0, n, st));
-  std::vector<double> H((k + 1) * k, 0.0), h(k + 2);
-  int kk = k;
+  unsigned long long seq = 0;
+  std::vector<unsigned long long> seqs(2 * k + 1, 0);
+  S_RC(dots(s, s->pw64, 0, 1, s->pw64, n, 0, nullptr, s->sc, 0, &seq, st));
+  S_CK(launch_normalise(V, s->pw64, s->sc, n, st));
   for (int j = 0; j < k; ++j) {
-    double* vj = V + (long long)j * n;
     double* wv = V + (long long)(j + 1) * n;
-    S_RC(op(vj, wv));
+    S_RC(op(V + (long long)j * n, wv));
     // classical Gram-Schmidt with the second pass only when the first removed
     // more than half of ||w||^2 (the criterion of the outer FGMRES); the dots
     // include w . w itself (wv is V_{j+1})
+    for (int pass = 0; pass < 2; ++pass) {
+      const DotScalars* gate = pass ? s->sc : nullptr;
+      S_RC(dots(s, V, n, j + 2, wv, n, 1, gate, s->sc + pass, 1 + 2 * j + pass, &seqs[2 * j + pass], st));
+      S_CK(launch_gs_update(wv, V, n, j + 1, s->sc + pass, gate, n, st));
+    }
+  }
+  S_CK(cudaStreamSynchronize(st));
+  std::vector<double> H((k + 1) * k, 0.0);
+  int kk = k;
+  for (int j = 0; j < k; ++j) {
     double ww2 = 0.0;
     for (int pass = 0; pass < 2; ++pass) {
-      S_RC(dev_dots(s, V, n, j + 2, wv, n, h.data(), st));
-      const double ww = h[j + 1];
-      S_CK(cudaMemcpyAsync(s->hdev, h.data(), sizeof(double) * (j + 1), cudaMemcpyHostToDevice, st));
-      S_CK(launch_maxpy(wv, V, n, j + 1, s->hdev, -1.0, n, st));
-      double hsq = 0.0;
-      for (int i = 0; i <= j; ++i) {
-        H[i * k + j] += h[i];
-        hsq += h[i] * h[i];
-      }
-      ww2 = std::max(ww - hsq, 0.0);
-      if (ww2 >= 0.5 * ww) break;
+      const DotScalars& h = s->host[1 + 2 * j + pass];
+      if (h.seq != seqs[2 * j + pass]) break;  // no second pass
+      for (int i = 0; i <= j; ++i) H[i * k + j] += h.dot[i];
+      ww2 = h.ww2;
     }
     const double hn = std::sqrt(ww2);
     if (!std::isfinite(hn)) return sfail(PFF_ERR_DEVICE, "Arnoldi eigenvalue estimate: non-finite vector");
     H[(j + 1) * k + j] = hn;
     if (hn <= 1e-14 * std::fabs(H[j * k + j]) + 1e-300) { kk = j + 1; break; }
-    S_CK(launch_axpby<double>(wv, wv, 1.0 / hn, 0.0, n, st));
   }
   std::vector<double> Hk(kk * kk);
   for (int i = 0; i < kk; ++i)
@@ -417,7 +445,7 @@ int power_coarse(pff_solver* s, cudaStream_t st) {
   double* y = s->cb;
   S_CK(cudaMemcpyAsync(v, s->pw64, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
   double h;
-  S_RC(dev_dots(s, v, 0, 1, v, n, &h, st));
+  S_RC(dev_norm2(s, v, n, &h, st));
   S_CK(launch_axpby<double>(v, v, 1.0 / std::sqrt(h), 0.0, n, st));
   double lam = 1.0;
   for (int it = 0; it < s->prm.power_iters; ++it) {
@@ -425,7 +453,7 @@ int power_coarse(pff_solver* s, cudaStream_t st) {
     a.v = v;
     a.y = y;
     S_RC(h_stencil(s, lev, kStScaled, a, st));
-    S_RC(dev_dots(s, y, 0, 1, y, n, &h, st));
+    S_RC(dev_norm2(s, y, n, &h, st));
     lam = std::sqrt(h);
     if (!(lam > 0.0) || !std::isfinite(lam)) return sfail(PFF_ERR_DEVICE, "coarse power iteration failed");
     S_CK(launch_axpby<double>(v, y, 1.0 / lam, 0.0, n, st));
@@ -437,10 +465,14 @@ int power_coarse(pff_solver* s, cudaStream_t st) {
 // Flexible GMRES(m), right preconditioned (Saad, Alg. 9.6), FP64; classical
 // Gram-Schmidt with a second pass when the first one loses accuracy (the
 // adaptive CGS refinement of Sec. 5).  V: (m+1) n, Z: m n device doubles.
+// sc, slot: its three sets of dot scalars on the device and in host memory (an
+// inner solve runs between an outer one's and must not share them).
 struct Krylov {
   long long n = 0;
   int m = 0;
   double *V = nullptr, *Z = nullptr;
+  DotScalars* sc = nullptr;
+  int slot = 0;
 };
 
 template <typename ApplyA, typename ApplyM>
@@ -448,63 +480,74 @@ int gmres_flex(pff_solver* s, const Krylov& kw, ApplyA&& applyA, ApplyM&& applyM
                double rtol, int maxit, int* iters, double* relres, cudaStream_t st) {
   const long long n = kw.n;
   const int m = kw.m;
-  std::vector<double> H((m + 1) * m, 0.0), cs(m, 0.0), sn(m, 0.0), g(m + 1, 0.0), h(m + 2), y(m);
-  S_CK(cudaMemsetAsync(x, 0, sizeof(double) * n, st));
+  std::vector<double> H((m + 1) * m, 0.0), cs(m, 0.0), sn(m, 0.0), g(m + 1, 0.0);
+  const DotScalars* host = s->host + kw.slot;
   double beta0 = -1.0, res = 0.0;
   int total = 0;
   bool first = true;
   while (true) {
     double* v0 = kw.V;
-    if (first) {
-      S_CK(cudaMemcpyAsync(v0, b, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
-    } else {
+    if (!first) {
       S_RC(applyA(x, v0));
       S_CK(launch_bminus<double>(v0, b, n, st));
     }
-    double bb;
-    S_RC(dev_dots(s, v0, 0, 1, v0, n, &bb, st));
-    double beta = std::sqrt(bb);
-    if (beta0 < 0) beta0 = beta;
-    if (beta == 0.0 || beta0 == 0.0) { res = 0.0; break; }
-    res = beta;
-    if (beta <= rtol * beta0 || total >= maxit) break;
-    S_CK(launch_axpby<double>(v0, v0, 1.0 / beta, 0.0, n, st));
-    std::fill(g.begin(), g.end(), 0.0);
-    g[0] = beta;
+    // ||r|| and v0 = r / ||r|| on the device; the host learns the norm with the
+    // first Hessenberg column, except where it may end the iteration
+    const double* r0 = first ? b : v0;
+    unsigned long long seq_b = 0;
+    S_RC(dots(s, r0, 0, 1, r0, n, 0, nullptr, kw.sc, kw.slot, &seq_b, st));
+    double beta = 0.0;
+    bool known = false;
+    auto read_beta = [&]() -> int {
+      S_RC(wait_dots(s, kw.slot, seq_b, st));
+      beta = std::sqrt(host[0].dot[0]);
+      if (beta0 < 0) beta0 = beta;
+      known = true;
+      return PFF_OK;
+    };
+    if (!first || !(rtol < 1.0) || total >= maxit) {
+      S_RC(read_beta());
+      if (beta == 0.0 || beta0 == 0.0) { res = 0.0; break; }
+      res = beta;
+      if (beta <= rtol * beta0 || total >= maxit) break;
+    }
+    S_CK(launch_normalise(v0, r0, kw.sc, n, st));
     int jend = 0;
+    bool zero = false;
     for (int j = 0; j < m && total < maxit; ++j) {
       double* vj = kw.V + (long long)j * n;
       double* zj = kw.Z + (long long)j * n;
       double* w = kw.V + (long long)(j + 1) * n;
       S_RC(applyM(vj, zj));
       S_RC(applyA(zj, w));
-      S_RC(dev_dots(s, kw.V, n, j + 2, w, n, h.data(), st));
-      double ww = h[j + 1];
-      S_CK(cudaMemcpyAsync(s->hdev, h.data(), sizeof(double) * (j + 1), cudaMemcpyHostToDevice, st));
-      S_CK(launch_maxpy(w, kw.V, n, j + 1, s->hdev, -1.0, n, st));
-      double hsq = 0.0;
-      for (int i = 0; i <= j; ++i) hsq += h[i] * h[i];
-      std::vector<double> hcol(h.begin(), h.begin() + j + 1);
+      if (!known) {
+        S_RC(read_beta());
+        if (beta == 0.0) { zero = true; break; }
+      }
+      if (j == 0) {
+        std::fill(g.begin(), g.end(), 0.0);
+        g[0] = beta;
+      }
       // ||w||^2 after the projection is ww - hsq; a second pass only when the
       // first one removed more than half of ||w||^2 (cancellation has cost
       // accuracy: Daniel-Gragg-Kaufman-Stewart criterion), otherwise the
       // estimate is accurate to a few rounding errors and no further
       // reduction is needed
-      double ww2 = ww - hsq;
-      if (ww2 < 0.5 * ww) {
-        S_RC(dev_dots(s, kw.V, n, j + 2, w, n, h.data(), st));
-        ww2 = h[j + 1];
-        double h2sq = 0.0;
-        for (int i = 0; i <= j; ++i) h2sq += h[i] * h[i];
-        S_CK(cudaMemcpyAsync(s->hdev, h.data(), sizeof(double) * (j + 1), cudaMemcpyHostToDevice, st));
-        S_CK(launch_maxpy(w, kw.V, n, j + 1, s->hdev, -1.0, n, st));
-        for (int i = 0; i <= j; ++i) hcol[i] += h[i];
-        ww2 = std::max(ww2 - h2sq, 0.0);
+      unsigned long long seq;
+      S_RC(dots(s, kw.V, n, j + 2, w, n, 1, nullptr, kw.sc + 1, kw.slot + 1, &seq, st));
+      S_CK(launch_gs_update(w, kw.V, n, j + 1, kw.sc + 1, nullptr, n, st));
+      S_RC(wait_dots(s, kw.slot + 1, seq, st));
+      for (int i = 0; i <= j; ++i) H[i * m + j] = host[1].dot[i];
+      double ww2 = host[1].ww2;
+      if (host[1].second) {
+        S_RC(dots(s, kw.V, n, j + 2, w, n, 1, kw.sc + 1, kw.sc + 2, kw.slot + 2, &seq, st));
+        S_CK(launch_gs_update(w, kw.V, n, j + 1, kw.sc + 2, kw.sc + 1, n, st));
+        S_RC(wait_dots(s, kw.slot + 2, seq, st));
+        for (int i = 0; i <= j; ++i) H[i * m + j] += host[2].dot[i];
+        ww2 = host[2].ww2;
       }
-      double hn = std::sqrt(std::max(ww2, 0.0));
-      for (int i = 0; i <= j; ++i) H[i * m + j] = hcol[i];
+      const double hn = std::sqrt(ww2);
       H[(j + 1) * m + j] = hn;
-      if (hn > 0.0) S_CK(launch_axpby<double>(w, w, 1.0 / hn, 0.0, n, st));
       for (int i = 0; i < j; ++i) {
         double a = H[i * m + j], c = H[(i + 1) * m + j];
         H[i * m + j] = cs[i] * a + sn[i] * c;
@@ -523,17 +566,18 @@ int gmres_flex(pff_solver* s, const Krylov& kw, ApplyA&& applyA, ApplyM&& applyM
       res = std::fabs(g[j + 1]);
       if (res <= rtol * beta0 || hn == 0.0) break;
     }
+    if (zero) { res = 0.0; break; }
+    LinCoef y;
     for (int i = jend - 1; i >= 0; --i) {
       double sum = g[i];
-      for (int k = i + 1; k < jend; ++k) sum -= H[i * m + k] * y[k];
-      y[i] = sum / H[i * m + i];
+      for (int k = i + 1; k < jend; ++k) sum -= H[i * m + k] * y.c[k];
+      y.c[i] = sum / H[i * m + i];
     }
-    S_CK(cudaMemcpyAsync(s->hdev, y.data(), sizeof(double) * jend, cudaMemcpyHostToDevice, st));
-    S_CK(launch_maxpy(x, kw.Z, n, jend, s->hdev, 1.0, n, st));
-    S_CK(cudaStreamSynchronize(st));
+    S_CK(launch_lincomb(x, kw.Z, n, jend, y, first ? 0 : 1, n, st));
     first = false;
     if (res <= rtol * beta0 || total >= maxit) break;
   }
+  if (first) S_CK(cudaMemsetAsync(x, 0, sizeof(double) * n, st));  // zero right-hand side, or no iteration allowed
   *iters = total;
   *relres = beta0 > 0 ? res / beta0 : 0.0;
   return PFF_OK;
@@ -549,6 +593,8 @@ int fgmres(pff_solver* s, const double* b, double* x, double rtol, int maxit, in
   kw.m = s->prm.krylov_restart;
   kw.V = s->V;
   kw.Z = s->Z;
+  kw.sc = s->sc;
+  kw.slot = 0;
   const pff_prec outer = (pff_prec)s->prm.outer_prec;
   auto A = [&](const double* in, double* out) {
     if (s->transpose) return pff_jacobian_transpose_apply(F, outer, in, out, st);
@@ -584,10 +630,12 @@ int coarse_gmres(pff_solver* s, cudaStream_t st) {
   kw.m = s->prm.krylov_restart;
   kw.V = s->cV;
   kw.Z = s->cZ;
+  kw.sc = s->sc + 3;
+  kw.slot = 3;
   auto A = [&](const double* in, double* out) -> int { return h_spmv(s, lev, in, out, st); };
   auto M = [&](const double* in, double* out) -> int {
     if (s->prm.coarse_solver == 2) return hcycle_top(s, in, out, st);
-    S_CK(launch_dscale<double>(out, in, s->cdiag, n, st));
+    S_CK(launch_jacobi(n, in, s->cdinv, nullptr, out, 1.0, st));
     return PFF_OK;
   };
   int its = 0;
@@ -617,7 +665,7 @@ int setup(pff_solver* s, cudaStream_t st, bool eig = true) {
     S_CK(launch_q1_assemble_sf(c.L->mesh, op->Q, op->lin64, s->prm.mixed ? op->lin32 : nullptr, c.L->tab.B64,
                                c.L->tab.Dt64, c.L->mask, s->Ke, s->A,
                                op->geo != nullptr, st));
-    S_CK(launch_q1_diag(c.L->mesh, s->A, s->cdiag, st));
+    S_CK(launch_q1_dinv(c.L->mesh, s->A, s->cdinv, st));
     if (s->A32) S_CK(launch_d2f(s->A32, s->A, 27LL * 16 * c.L->mesh.nn, st));
     if (s->prm.coarse_solver == 0 && eig) S_RC(power_coarse(s, st));
     if (s->prm.coarse_solver == 2) {
@@ -627,7 +675,7 @@ int setup(pff_solver* s, cudaStream_t st, bool eig = true) {
         S_CK(launch_hmask(f.mesh, h.mesh, f.mask, h.own_mask, st));
         S_CK(launch_q1_coarsen(f.mesh, h.mesh, f.mask, f.Ke, h.Ke, s->prm.mixed != 0, st));
         S_CK(launch_q1_gather(h.mesh, h.Ke, h.mask, h.A, st));
-        S_CK(launch_q1_diag(h.mesh, h.A, h.diag, st));
+        S_CK(launch_q1_dinv(h.mesh, h.A, h.dinv, st));
         if (h.A32) S_CK(launch_d2f(h.A32, h.A, 27LL * 16 * h.mesh.nn, st));
       }
       if (eig)
@@ -645,14 +693,14 @@ void free_solver(pff_solver* s) {
   for (auto& w : s->lv) {
     cudaFree(w.diag); cudaFree(w.b); cudaFree(w.x); cudaFree(w.tmp); cudaFree(w.work);
   }
-  cudaFree(s->A); cudaFree(s->A32); cudaFree(s->cdiag); cudaFree(s->cb); cudaFree(s->cx); cudaFree(s->cwork);
+  cudaFree(s->A); cudaFree(s->A32); cudaFree(s->cdinv); cudaFree(s->cb); cudaFree(s->cx); cudaFree(s->cwork);
   cudaFree(s->cV); cudaFree(s->cZ); cudaFree(s->Ke);
   for (HLevel& h : s->hl) {
-    if (h.owns) { cudaFree(h.Ke); cudaFree(h.A); cudaFree(h.A32); cudaFree(h.diag); cudaFree(h.own_mask); }
+    if (h.owns) { cudaFree(h.Ke); cudaFree(h.A); cudaFree(h.A32); cudaFree(h.dinv); cudaFree(h.own_mask); }
     cudaFree(h.b); cudaFree(h.x); cudaFree(h.r); cudaFree(h.work);
   }
   cudaFree(s->V); cudaFree(s->Z); cudaFree(s->r); cudaFree(s->dz); cudaFree(s->zold);
-  cudaFree(s->partial); cudaFree(s->dots); cudaFree(s->hdev);
+  cudaFree(s->partial); cudaFree(s->arrived); cudaFree(s->sc); cudaFreeHost(s->host);
   cudaFree(s->pw64); cudaFree(s->pw32);
   cudaFree(s->a_in); cudaFree(s->pbuf); cudaFree(s->qa); cudaFree(s->ag); cudaFree(s->alam); cudaFree(s->av);
   cudaFree(s->gth);
@@ -734,7 +782,7 @@ int pff_create_solver(pff_op* op, int nlevels, pff_level* const* levels, const p
     const long long nc = s->lv.back().n;
     if (e == cudaSuccess) e = cudaMalloc(&s->A, sizeof(double) * 27 * 16 * (nc / 4));
     if (e == cudaSuccess && prm->mixed) e = cudaMalloc(&s->A32, sizeof(float) * 27 * 16 * (nc / 4));
-    if (e == cudaSuccess) e = cudaMalloc(&s->cdiag, sizeof(double) * nc);
+    if (e == cudaSuccess) e = cudaMalloc(&s->cdinv, sizeof(double) * nc);
     if (e == cudaSuccess) e = cudaMalloc(&s->cb, sizeof(double) * nc);
     if (e == cudaSuccess) e = cudaMalloc(&s->cx, sizeof(double) * nc);
     if (e == cudaSuccess) e = cudaMalloc(&s->cwork, sizeof(double) * 3 * nc);
@@ -751,7 +799,7 @@ int pff_create_solver(pff_op* op, int nlevels, pff_level* const* levels, const p
       h0.Ke = s->Ke;
       h0.A = s->A;
       h0.A32 = s->A32;
-      h0.diag = s->cdiag;
+      h0.dinv = s->cdinv;
       h0.mask = Lc->is_fine ? op->mask : Lc->mask;
       s->hl.push_back(h0);
       while (true) {
@@ -769,7 +817,7 @@ int pff_create_solver(pff_op* op, int nlevels, pff_level* const* levels, const p
         if (e == cudaSuccess) e = cudaMalloc(&h.Ke, sizeof(double) * 1024 * (size_t)h.mesh.nel);
         if (e == cudaSuccess) e = cudaMalloc(&h.A, sizeof(double) * 27 * 16 * (size_t)h.mesh.nn);
         if (e == cudaSuccess && prm->mixed) e = cudaMalloc(&h.A32, sizeof(float) * 27 * 16 * (size_t)h.mesh.nn);
-        if (e == cudaSuccess) e = cudaMalloc(&h.diag, sizeof(double) * h.n);
+        if (e == cudaSuccess) e = cudaMalloc(&h.dinv, sizeof(double) * h.n);
         if (e == cudaSuccess) e = cudaMalloc(&h.own_mask, h.n);
         h.mask = h.own_mask;
         s->hl.push_back(h);
@@ -790,8 +838,12 @@ int pff_create_solver(pff_op* op, int nlevels, pff_level* const* levels, const p
   if (e == cudaSuccess) e = cudaMalloc(&s->dz, sizeof(double) * s->n);
   if (e == cudaSuccess) e = cudaMalloc(&s->zold, sizeof(double) * s->n);
   if (e == cudaSuccess) e = cudaMalloc(&s->partial, sizeof(double) * 64 * kReduceBlocks);
-  if (e == cudaSuccess) e = cudaMalloc(&s->dots, sizeof(double) * 64);
-  if (e == cudaSuccess) e = cudaMalloc(&s->hdev, sizeof(double) * 64);
+  if (e == cudaSuccess) e = cudaMalloc(&s->arrived, sizeof(unsigned));
+  if (e == cudaSuccess) e = cudaMemset(s->arrived, 0, sizeof(unsigned));
+  if (e == cudaSuccess) e = cudaMalloc(&s->sc, sizeof(DotScalars) * 6);
+  if (e == cudaSuccess) e = cudaHostAlloc((void**)&s->host, sizeof(DotScalars) * kHostSlots, cudaHostAllocMapped);
+  if (e == cudaSuccess) std::memset(s->host, 0, sizeof(DotScalars) * kHostSlots);
+  if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&s->host_dev, s->host, 0);
   if (e == cudaSuccess) e = cudaMalloc(&s->pw64, sizeof(double) * s->n);
   if (e == cudaSuccess) e = cudaMalloc(&s->pw32, sizeof(float) * s->n);
   if (e == cudaSuccess) {
@@ -896,7 +948,10 @@ int pff_solver_hcycle(pff_solver* s, const double* b, double* x, void* stream) {
 int pff_solver_krylov(pff_solver* s, const double* b, double* x, double rtol, int maxit, int* iters, double* relres,
                       void* stream) {
   if (!s || !b || !x || !iters || !relres) return sfail(PFF_ERR_INVALID, "pff_solver_krylov: null argument");
-  return fgmres(s, b, x, rtol, maxit, iters, relres, reinterpret_cast<cudaStream_t>(stream));
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  S_RC(fgmres(s, b, x, rtol, maxit, iters, relres, st));
+  S_CK(cudaStreamSynchronize(st));
+  return PFF_OK;
 }
 
 int pff_newton_solve(pff_solver* s, double* z, pff_newton_stats* stats, void* stream) {
@@ -918,7 +973,7 @@ int pff_newton_solve(pff_solver* s, double* z, pff_newton_stats* stats, void* st
       }
     }
     double rr;
-    S_RC(dev_dots(s, s->r, 0, 1, s->r, n, &rr, st));
+    S_RC(dev_norm2(s, s->r, n, &rr, st));
     double rn = std::sqrt(rr);
     stats->t_residual += now() - t0;
     if (r0 < 0) r0 = rn;
@@ -962,7 +1017,7 @@ int pff_newton_solve(pff_solver* s, double* z, pff_newton_stats* stats, void* st
       int lst = 0;
       S_RC(pff_get_status(s->op, stream, &lst));
       double r2 = 0.0;
-      if (!lst) S_RC(dev_dots(s, s->r, 0, 1, s->r, n, &r2, st));
+      if (!lst) S_RC(dev_norm2(s, s->r, n, &r2, st));
       const double rt = std::sqrt(r2);
       if (!lst && std::isfinite(rt) && rt <= (1.0 - 1e-4 * alpha) * rn) { accepted = true; break; }
       if (!lst && std::isfinite(rt) && ls == s->prm.line_search_max) { accepted = true; break; }
