@@ -268,8 +268,8 @@ int ensure_prolong_table(pff_level* c, pff_level* f) {
 }  // namespace
 
 template <typename T>
-static int cheb_t(pff_level* L, int degree, double lmin, double lmax, const T* diag, const T* b, T* x, T* work,
-                  cudaStream_t st, bool w16 = false) {
+static int cheb_t(pff_level* L, bool w16, bool transpose, bool from_zero, int degree, double lmin, double lmax,
+                  const T* diag, const T* b, T* x, T* work, cudaStream_t st) {
   const long long n = 4 * L->mesh.nn;
   T* r = work;
   T* d = work + n;
@@ -277,18 +277,22 @@ static int cheb_t(pff_level* L, int degree, double lmin, double lmax, const T* d
   const double theta = 0.5 * (lmax + lmin), delta = 0.5 * (lmax - lmin);
   const double sigma = theta / delta;
   double rho = 1.0 / sigma;
-  int rc = apply_t<T>(L, x, Ad, 0, st, w16);
-  if (rc) return rc;
-  PFF_CK(launch_cheb_init<T>(n, b, Ad, diag, r, d, 1.0 / theta, st));
-  for (int k = 0; k < degree; ++k) {
-    if (k == degree - 1) {
-      PFF_CK(launch_cheb_step<T>(n, x, d, r, Ad, diag, 0.0, 0.0, 1, st));
-      break;
-    }
-    rc = apply_t<T>(L, d, Ad, 0, st, w16);
-    if (rc) return rc;
+  const uint8_t* mask = level_mask(L);
+  // the vector updates prepare Ad for the atomic scatter; the deterministic
+  // transpose writes every entry itself
+  const bool init = L->op->det && L->op->evec;
+  int rc;
+  if (!from_zero && (rc = apply_t<T>(L, x, Ad, transpose, st, w16))) return rc;
+  PFF_CK(launch_cheb_first<T>(n, b, from_zero ? nullptr : Ad, diag, mask, r, d, Ad, 1.0 / theta, st));
+  if (degree == 1) {
+    if (from_zero) PFF_CK(cudaMemcpyAsync(x, d, sizeof(T) * n, cudaMemcpyDeviceToDevice, st));
+    else PFF_CK(launch_axpby<T>(x, d, 1.0, 1.0, n, st));
+  }
+  for (int k = 0; k + 1 < degree; ++k) {
+    if ((rc = apply_t<T>(L, d, Ad, transpose, st, w16, 0, 0, init))) return rc;
     const double rho_new = 1.0 / (2.0 * sigma - rho);
-    PFF_CK(launch_cheb_step<T>(n, x, d, r, Ad, diag, rho_new * rho, 2.0 * rho_new / delta, 0, st));
+    PFF_CK(launch_cheb_next<T>(n, x, d, r, Ad, diag, mask, rho_new * rho, 2.0 * rho_new / delta, from_zero && k == 0,
+                               k + 2 == degree, st));
     rho = rho_new;
   }
   return PFF_OK;
@@ -301,6 +305,14 @@ int apply_blocks(pff_level* L, int prec, const void* x, void* y, int transpose, 
     return apply_t<float>(L, (const float*)x, (float*)y, transpose, st, prec == PFF_F32_BF16, blk0, nblk, false);
   if (prec == PFF_DF64) return apply_df(L, (const double*)x, (double*)y, transpose, st, blk0, nblk, false);
   return fail(PFF_ERR_INVALID, "unknown precision");
+}
+int smooth_level(pff_level* L, int prec, bool transpose, bool from_zero, int degree, double lmin, double lmax,
+                 const void* diag, const void* b, void* x, void* work, cudaStream_t st) {
+  if (prec == PFF_F64)
+    return cheb_t<double>(L, false, transpose, from_zero, degree, lmin, lmax, (const double*)diag, (const double*)b,
+                          (double*)x, (double*)work, st);
+  return cheb_t<float>(L, prec == PFF_F32_BF16, transpose, from_zero, degree, lmin, lmax, (const float*)diag,
+                       (const float*)b, (float*)x, (float*)work, st);
 }
 const uint8_t* level_rows_mask(const pff_level* L) { return level_mask(L); }
 int set_last_error(int code, const char* msg) { return fail(code, msg); }
@@ -852,11 +864,8 @@ int pff_chebyshev_smooth(pff_level* L, pff_prec prec, int degree, double lmin, d
   PFF_REQUIRE(L && diag && b && x && work, "pff_chebyshev_smooth: null argument");
   PFF_REQUIRE(degree >= 1 && degree <= 64, "pff_chebyshev_smooth: 1 <= degree <= 64");
   PFF_REQUIRE(lmax > lmin && lmin > 0.0, "pff_chebyshev_smooth: need 0 < lmin < lmax");
-  if (prec == PFF_F64)
-    return cheb_t<double>(L, degree, lmin, lmax, (const double*)diag, (const double*)b, (double*)x, (double*)work, S(stream));
-  if (prec == PFF_F32 || prec == PFF_F32_BF16)
-    return cheb_t<float>(L, degree, lmin, lmax, (const float*)diag, (const float*)b, (float*)x, (float*)work, S(stream),
-                         prec == PFF_F32_BF16);
+  if (prec == PFF_F64 || prec == PFF_F32 || prec == PFF_F32_BF16)
+    return smooth_level(L, prec, false, false, degree, lmin, lmax, diag, b, x, work, S(stream));
   return fail(PFF_ERR_INVALID, "pff_chebyshev_smooth: unknown precision");
 }
 

@@ -91,6 +91,11 @@ namespace pff {
 // the initialisation of y; prec PFF_F64, PFF_F32, PFF_DF64 or PFF_F32_BF16
 // (pff_abi.cpp).
 int apply_blocks(pff_level* L, int prec, const void* x, void* y, int transpose, int blk0, int nblk, cudaStream_t st);
+// Chebyshev smoothing of J x = b or (transpose) J^T x = b on a level (Saad, Alg.
+// 12.1); work: three level vectors.  from_zero: x is zero on entry and not read,
+// and the first product is left out (pff_abi.cpp).
+int smooth_level(pff_level* L, int prec, bool transpose, bool from_zero, int degree, double lmin, double lmax,
+                 const void* diag, const void* b, void* x, void* work, cudaStream_t st);
 // The Dirichlet mask of a level's rows (pff_abi.cpp).
 const uint8_t* level_rows_mask(const pff_level* L);
 // Releases the staging buffers, streams and events of pff_jacobian_apply_host (pff_hostio.cpp).

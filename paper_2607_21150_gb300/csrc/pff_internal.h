@@ -271,14 +271,13 @@ cudaError_t launch_prolong(const MeshDev& mc, const MeshDev& mf, const T* I1, co
 template <typename T>
 cudaError_t launch_restrict(const MeshDev& mc, const MeshDev& mf, const T* I1, const T* rf, T* rc,
                             const uint8_t* maskc, const uint8_t* maskf, cudaStream_t st, void* evec = nullptr);
+// Chebyshev updates between level actions (Ax null: x = 0; mask null: none).
 template <typename T>
-cudaError_t launch_cheb_init(long long n, const T* b, const T* Ax, const T* diag, T* r, T* d,
-                             double inv_theta, cudaStream_t st);
+cudaError_t launch_cheb_first(long long n, const T* b, const T* Ax, const T* diag, const uint8_t* mask, T* r, T* d,
+                              T* Ad, double inv_theta, cudaStream_t st);
 template <typename T>
-cudaError_t launch_cheb_zero(long long n, const T* b, const T* diag, T* r, T* d, double inv_theta, cudaStream_t st);
-template <typename T>
-cudaError_t launch_cheb_step(long long n, T* x, T* d, T* r, const T* Ad, const T* diag,
-                             double c_d, double c_r, int last, cudaStream_t st);
+cudaError_t launch_cheb_next(long long n, T* x, T* d, T* r, T* Ad, const T* diag, const uint8_t* mask, double c_d,
+                             double c_r, int xset, int last, cudaStream_t st);
 
 
 // Krylov vectors and the assembled coarse operator (pff_krylov.cu)

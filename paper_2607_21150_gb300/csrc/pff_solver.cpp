@@ -168,37 +168,10 @@ int level_apply(pff_solver* s, const LevelWork& w, const void* x, void* y, cudaS
   return pff_jacobian_apply(w.L, (pff_prec)w.prec, x, y, st);
 }
 
-// Chebyshev smoothing (Saad, Alg. 12.1) of J x = b or, in transposed mode,
-// J^T x = b (same eigenvalue bounds: D^-1 J^T and D^-1 J have the same spectrum).
-int cheb_level(pff_solver* s, LevelWork& w, int degree, double lmin, double lmax, cudaStream_t st) {
-  const long long n = w.n;
-  const double theta = 0.5 * (lmax + lmin), delta = 0.5 * (lmax - lmin), sigma = theta / delta;
-  double rho = 1.0 / sigma;
-  char* base = (char*)w.work;
-  void* r = base;
-  void* d = base + w.esz * n;
-  void* Ad = base + 2 * w.esz * n;
-  S_RC(level_apply(s, w, w.x, Ad, st));
-  if (w.prec == PFF_F64)
-    S_CK(launch_cheb_init<double>(n, (const double*)w.b, (const double*)Ad, (const double*)w.diag, (double*)r, (double*)d, 1.0 / theta, st));
-  else
-    S_CK(launch_cheb_init<float>(n, (const float*)w.b, (const float*)Ad, (const float*)w.diag, (float*)r, (float*)d, 1.0 / theta, st));
-  for (int k = 0; k < degree; ++k) {
-    const bool last = (k == degree - 1);
-    double cd = 0.0, cr = 0.0;
-    if (!last) {
-      S_RC(level_apply(s, w, d, Ad, st));
-      const double rho_new = 1.0 / (2.0 * sigma - rho);
-      cd = rho_new * rho;
-      cr = 2.0 * rho_new / delta;
-      rho = rho_new;
-    }
-    if (w.prec == PFF_F64)
-      S_CK(launch_cheb_step<double>(n, (double*)w.x, (double*)d, (double*)r, (const double*)Ad, (const double*)w.diag, cd, cr, last, st));
-    else
-      S_CK(launch_cheb_step<float>(n, (float*)w.x, (float*)d, (float*)r, (const float*)Ad, (const float*)w.diag, cd, cr, last, st));
-  }
-  return PFF_OK;
+// Chebyshev smoothing of J x = b or, in transposed mode, J^T x = b (same
+// eigenvalue bounds: D^-1 J^T and D^-1 J have the same spectrum).
+int cheb_level(pff_solver* s, LevelWork& w, bool from_zero, int degree, double lmin, double lmax, cudaStream_t st) {
+  return smooth_level(w.L, w.prec, s->transpose != 0, from_zero, degree, lmin, lmax, w.diag, w.b, w.x, w.work, st);
 }
 
 // Stencil product of an assembled level with the update that consumes it: the
@@ -285,10 +258,9 @@ int vcycle(pff_solver* s, int l, cudaStream_t st) {
   LevelWork& w = s->lv[l];
   const bool coarsest = (l + 1 == (int)s->lv.size());
   if (coarsest && s->assembled) return coarse_cheb(s, st);
-  S_CK(cudaMemsetAsync(w.x, 0, w.esz * w.n, st));
   const int deg = coarsest ? s->prm.coarse_degree : s->prm.cheb_degree;
   const double lo = coarsest ? s->prm.coarse_lo : s->prm.cheb_lo;
-  S_RC(cheb_level(s, w, deg, lo * w.lmax, s->prm.cheb_hi * w.lmax, st));
+  S_RC(cheb_level(s, w, true, deg, lo * w.lmax, s->prm.cheb_hi * w.lmax, st));
   if (coarsest) return PFF_OK;
   // residual, restriction, coarse correction, prolongation
   S_RC(level_apply(s, w, w.x, w.tmp, st));
@@ -299,7 +271,7 @@ int vcycle(pff_solver* s, int l, cudaStream_t st) {
   S_RC(vcycle(s, l + 1, st));
   S_RC(pff_prolong(c.L, w.L, (pff_prec)w.prec, c.x, w.tmp, st));
   S_RC(axpby_level(w, w.x, w.tmp, 1.0, 1.0, st));
-  S_RC(cheb_level(s, w, s->prm.cheb_degree, s->prm.cheb_lo * w.lmax, s->prm.cheb_hi * w.lmax, st));
+  S_RC(cheb_level(s, w, false, s->prm.cheb_degree, s->prm.cheb_lo * w.lmax, s->prm.cheb_hi * w.lmax, st));
   return PFF_OK;
 }
 

@@ -4,6 +4,8 @@
 // and the geometric factors of mapped meshes.
 #include <cuda_bf16.h>
 
+#include <initializer_list>
+
 #include "pff_df.cuh"
 #include "pff_internal.h"
 
@@ -355,67 +357,106 @@ cudaError_t launch_restrict(const MeshDev& mc, const MeshDev& mf, const T* I1, c
   return cudaGetLastError();
 }
 
-// Chebyshev iteration (Saad, Alg. 12.1) on D^-1 A:
-//   init:  r = D^-1 (b - A x),  d = r / theta
-//   step:  x += d;  r -= D^-1 A d;  d = c_d d + c_r r      (c_d = rho_k+1 rho_k, c_r = 2 rho_k+1 / delta)
-//   last:  x += d
-template <typename T>
-__global__ void k_cheb_init(long long n, const T* __restrict__ b, const T* __restrict__ Ax, const T* __restrict__ diag,
-                            T* __restrict__ r, T* __restrict__ d, T inv_theta) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    T ri = (b[i] - Ax[i]) / diag[i];
-    r[i] = ri;
-    d[i] = ri * inv_theta;
+// Chebyshev iteration (Saad, Alg. 12.1) on D^-1 A, between products:
+//   first: r = D^-1 (b - A x),  d = r / theta          (A x absent: x = 0)
+//   next:  x += d (xset: x = d);  r -= D^-1 A d;  d = c_d d + c_r r
+//          last: x += that d too, which ends the smoothing (r, d not written)
+// Both leave in Ad what the action expects there, its next input's prescribed
+// entries and zeros elsewhere, so that no pass of its own prepares it.  Bound by
+// HBM: a degree-3 smoothing moves 21 vectors instead of 30 (64 bit or 32 bit;
+// 40^3 Q4 FP32, 67 MB each: 383 -> 226 us with the clears).  V entries per thread, 16-byte
+// accesses where every pointer allows them.
+template <typename T, int V> struct alignas(sizeof(T) * V) VecOf { T v[V]; };
+
+template <typename T, int V>
+__global__ void __launch_bounds__(kVecThreads) k_cheb_first(long long n, const T* b, const T* Ax, const T* diag,
+                                                            const uint8_t* mask, T* r, T* d, T* Ad, T inv_theta) {
+  using W = VecOf<T, V>;
+  using M = VecOf<uint8_t, V>;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n / V; i += (long long)gridDim.x * blockDim.x) {
+    const W bi = reinterpret_cast<const W*>(b)[i], gi = reinterpret_cast<const W*>(diag)[i];
+    W ax, ri, di, ai;
+    M m;
+    if (Ax) ax = reinterpret_cast<const W*>(Ax)[i];
+    if (mask) m = reinterpret_cast<const M*>(mask)[i];
+#pragma unroll
+    for (int c = 0; c < V; ++c) {
+      ri.v[c] = (Ax ? bi.v[c] - ax.v[c] : bi.v[c]) / gi.v[c];
+      di.v[c] = ri.v[c] * inv_theta;
+      ai.v[c] = mask && m.v[c] ? di.v[c] : T(0);
+    }
+    reinterpret_cast<W*>(r)[i] = ri;
+    reinterpret_cast<W*>(d)[i] = di;
+    reinterpret_cast<W*>(Ad)[i] = ai;
   }
 }
-// init from x = 0: r = D^-1 b, d = r / theta
-template <typename T>
-__global__ void k_cheb_zero(long long n, const T* __restrict__ b, const T* __restrict__ diag, T* __restrict__ r,
-                            T* __restrict__ d, T inv_theta) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const T ri = b[i] / diag[i];
-    r[i] = ri;
-    d[i] = ri * inv_theta;
-  }
-}
-template <typename T>
-__global__ void k_cheb_step(long long n, T* __restrict__ x, T* __restrict__ d, T* __restrict__ r,
-                            const T* __restrict__ Ad, const T* __restrict__ diag, T c_d, T c_r, int last) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    T di = d[i];
-    x[i] += di;
-    if (!last) {
-      T ri = r[i] - Ad[i] / diag[i];
-      r[i] = ri;
-      d[i] = c_d * di + c_r * ri;
+template <typename T, int V, bool LAST>
+__global__ void __launch_bounds__(kVecThreads) k_cheb_next(long long n, T* x, T* d, T* r, T* Ad, const T* diag,
+                                                           const uint8_t* mask, T c_d, T c_r, int xset) {
+  using W = VecOf<T, V>;
+  using M = VecOf<uint8_t, V>;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n / V; i += (long long)gridDim.x * blockDim.x) {
+    W di = reinterpret_cast<const W*>(d)[i], ri = reinterpret_cast<const W*>(r)[i];
+    const W gi = reinterpret_cast<const W*>(diag)[i];
+    W ai = reinterpret_cast<const W*>(Ad)[i], xi;
+    M m;
+    if (!xset) xi = reinterpret_cast<const W*>(x)[i];
+    if (!LAST && mask) m = reinterpret_cast<const M*>(mask)[i];
+#pragma unroll
+    for (int c = 0; c < V; ++c) {
+      xi.v[c] = xset ? di.v[c] : xi.v[c] + di.v[c];
+      ri.v[c] -= ai.v[c] / gi.v[c];
+      di.v[c] = c_d * di.v[c] + c_r * ri.v[c];
+      if (LAST) xi.v[c] += di.v[c];
+      else ai.v[c] = mask && m.v[c] ? di.v[c] : T(0);
+    }
+    reinterpret_cast<W*>(x)[i] = xi;
+    if (!LAST) {
+      reinterpret_cast<W*>(r)[i] = ri;
+      reinterpret_cast<W*>(d)[i] = di;
+      reinterpret_cast<W*>(Ad)[i] = ai;
     }
   }
 }
-
+static bool aligned16(std::initializer_list<const void*> ps) {
+  uintptr_t u = 0;
+  for (const void* p : ps) u |= reinterpret_cast<uintptr_t>(p);
+  return u % 16 == 0;
+}
 template <typename T>
-cudaError_t launch_cheb_init(long long n, const T* b, const T* Ax, const T* diag, T* r, T* d, double inv_theta,
-                             cudaStream_t st) {
+cudaError_t launch_cheb_first(long long n, const T* b, const T* Ax, const T* diag, const uint8_t* mask, T* r, T* d,
+                              T* Ad, double inv_theta, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  k_cheb_init<T><<<grid_for(n), kVecThreads, 0, st>>>(n, b, Ax, diag, r, d, (T)inv_theta); note_launch();
+  constexpr int V = 16 / sizeof(T);
+  if (n % V == 0 && aligned16({b, Ax, diag, mask, r, d, Ad}))
+    k_cheb_first<T, V><<<grid_for(n / V), kVecThreads, 0, st>>>(n, b, Ax, diag, mask, r, d, Ad, (T)inv_theta);
+  else
+    k_cheb_first<T, 1><<<grid_for(n), kVecThreads, 0, st>>>(n, b, Ax, diag, mask, r, d, Ad, (T)inv_theta);
+  note_launch();
   return cudaGetLastError();
 }
 template <typename T>
-cudaError_t launch_cheb_zero(long long n, const T* b, const T* diag, T* r, T* d, double inv_theta, cudaStream_t st) {
+cudaError_t launch_cheb_next(long long n, T* x, T* d, T* r, T* Ad, const T* diag, const uint8_t* mask, double c_d,
+                             double c_r, int xset, int last, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  k_cheb_zero<T><<<grid_for(n), kVecThreads, 0, st>>>(n, b, diag, r, d, (T)inv_theta); note_launch();
+  constexpr int V = 16 / sizeof(T);
+  const bool wide = n % V == 0 && aligned16({x, d, r, Ad, diag, mask});
+  const unsigned nb = grid_for(wide ? n / V : n);
+  if (wide && last) k_cheb_next<T, V, true><<<nb, kVecThreads, 0, st>>>(n, x, d, r, Ad, diag, mask, (T)c_d, (T)c_r, xset);
+  else if (wide) k_cheb_next<T, V, false><<<nb, kVecThreads, 0, st>>>(n, x, d, r, Ad, diag, mask, (T)c_d, (T)c_r, xset);
+  else if (last) k_cheb_next<T, 1, true><<<nb, kVecThreads, 0, st>>>(n, x, d, r, Ad, diag, mask, (T)c_d, (T)c_r, xset);
+  else k_cheb_next<T, 1, false><<<nb, kVecThreads, 0, st>>>(n, x, d, r, Ad, diag, mask, (T)c_d, (T)c_r, xset);
+  note_launch();
   return cudaGetLastError();
 }
-template cudaError_t launch_cheb_zero<double>(long long, const double*, const double*, double*, double*, double,
-                                              cudaStream_t);
-template cudaError_t launch_cheb_zero<float>(long long, const float*, const float*, float*, float*, double,
-                                             cudaStream_t);
-template <typename T>
-cudaError_t launch_cheb_step(long long n, T* x, T* d, T* r, const T* Ad, const T* diag, double c_d, double c_r,
-                             int last, cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  k_cheb_step<T><<<grid_for(n), kVecThreads, 0, st>>>(n, x, d, r, Ad, diag, (T)c_d, (T)c_r, last); note_launch();
-  return cudaGetLastError();
-}
+template cudaError_t launch_cheb_first<double>(long long, const double*, const double*, const double*, const uint8_t*,
+                                               double*, double*, double*, double, cudaStream_t);
+template cudaError_t launch_cheb_first<float>(long long, const float*, const float*, const float*, const uint8_t*,
+                                              float*, float*, float*, double, cudaStream_t);
+template cudaError_t launch_cheb_next<double>(long long, double*, double*, double*, double*, const double*,
+                                              const uint8_t*, double, double, int, int, cudaStream_t);
+template cudaError_t launch_cheb_next<float>(long long, float*, float*, float*, float*, const float*, const uint8_t*,
+                                             double, double, int, int, cudaStream_t);
 
 
 // Stored linearisation from the tiled layout to the canonical order [67][N_q]
@@ -555,14 +596,6 @@ template cudaError_t launch_restrict<double>(const MeshDev&, const MeshDev&, con
                                              const uint8_t*, const uint8_t*, cudaStream_t, void*);
 template cudaError_t launch_restrict<float>(const MeshDev&, const MeshDev&, const float*, const float*, float*,
                                             const uint8_t*, const uint8_t*, cudaStream_t, void*);
-template cudaError_t launch_cheb_init<double>(long long, const double*, const double*, const double*, double*, double*,
-                                              double, cudaStream_t);
-template cudaError_t launch_cheb_init<float>(long long, const float*, const float*, const float*, float*, float*,
-                                             double, cudaStream_t);
-template cudaError_t launch_cheb_step<double>(long long, double*, double*, double*, const double*, const double*,
-                                              double, double, int, cudaStream_t);
-template cudaError_t launch_cheb_step<float>(long long, float*, float*, float*, const float*, const float*, double,
-                                             double, int, cudaStream_t);
 
 // Geometry of a mapped mesh at every quadrature point from the parent Jacobian
 // J = dX / dxi (rows 3 f + al of an eval of the nodal coordinates):
