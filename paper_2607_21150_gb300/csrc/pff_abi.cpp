@@ -247,22 +247,15 @@ int diag_t(pff_level* L, T* diag, cudaStream_t st) {
   return PFF_OK;
 }
 
-int ensure_prolong_table(pff_level* c, pff_level* f) {
-  if (c->I_pf == f->p) return PFF_OK;
-  cudaFree(c->I64); cudaFree(c->I32);
-  c->I64 = nullptr; c->I32 = nullptr;
-  int pc = c->p, pf = f->p;
+void ensure_prolong_table(pff_level* c, pff_level* f) {
+  if (c->I_pf == f->p) return;
+  const int pc = c->p, pf = f->p;
   std::vector<double> xc(pc + 1), xf(pf + 1);
   gll_nodes(pc, xc.data());
   gll_nodes(pf, xf.data());
-  std::vector<double> I((pf + 1) * (pc + 1));
   for (int a = 0; a <= pf; ++a)
-    for (int b = 0; b <= pc; ++b) I[a * (pc + 1) + b] = lagrange(xc.data(), pc + 1, b, xf[a]);
-  int rc;
-  if ((rc = upload(I, &c->I64))) return rc;
-  if ((rc = upload(I, &c->I32))) return rc;
+    for (int b = 0; b <= pc; ++b) c->I1[a * (pc + 1) + b] = lagrange(xc.data(), pc + 1, b, xf[a]);
   c->I_pf = pf;
-  return PFF_OK;
 }
 
 }  // namespace
@@ -313,6 +306,22 @@ int smooth_level(pff_level* L, int prec, bool transpose, bool from_zero, int deg
                           (double*)x, (double*)work, st);
   return cheb_t<float>(L, prec == PFF_F32_BF16, transpose, from_zero, degree, lmin, lmax, (const float*)diag,
                        (const float*)b, (float*)x, (float*)work, st);
+}
+int transfer_prolong(pff_level* c, pff_level* f, int prec, const void* xc, void* xf, bool add, cudaStream_t st) {
+  ensure_prolong_table(c, f);
+  const uint8_t *mc = level_mask(c), *mf = level_mask(f), *em = level_emask(f);
+  if (prec == PFF_F64) PFF_CK(launch_prolong<double>(c->mesh, f->mesh, c->I1, (const double*)xc, (double*)xf, mc, mf, em, add, st));
+  else if (prec == PFF_F32 || prec == PFF_F32_BF16) PFF_CK(launch_prolong<float>(c->mesh, f->mesh, c->I1, (const float*)xc, (float*)xf, mc, mf, em, add, st));
+  else return fail(PFF_ERR_INVALID, "pff_prolong: unknown precision");
+  return PFF_OK;
+}
+int transfer_restrict(pff_level* c, pff_level* f, int prec, const void* rf, const void* b, void* rc, cudaStream_t st) {
+  ensure_prolong_table(c, f);
+  const uint8_t *mc = level_mask(c), *mf = level_mask(f), *em = level_emask(f);
+  if (prec == PFF_F64) PFF_CK(launch_restrict<double>(c->mesh, f->mesh, c->I1, (const double*)rf, (const double*)b, (double*)rc, mc, mf, em, st));
+  else if (prec == PFF_F32 || prec == PFF_F32_BF16) PFF_CK(launch_restrict<float>(c->mesh, f->mesh, c->I1, (const float*)rf, (const float*)b, (float*)rc, mc, mf, em, st));
+  else return fail(PFF_ERR_INVALID, "pff_restrict: unknown precision");
+  return PFF_OK;
 }
 const uint8_t* level_rows_mask(const pff_level* L) { return level_mask(L); }
 int set_last_error(int code, const char* msg) { return fail(code, msg); }
@@ -782,7 +791,6 @@ int pff_destroy_level(pff_level* L) {
   free_tables(L->tab);
   cudaFree(L->mask);
   cudaFree(L->emask);
-  cudaFree(L->I64); cudaFree(L->I32);
   delete L;
   return PFF_OK;
 }
@@ -834,29 +842,14 @@ int pff_prolong(pff_level* c, pff_level* f, pff_prec prec, const void* xc, void*
   PFF_REQUIRE(c && f && xc && xf, "pff_prolong: null argument");
   PFF_REQUIRE(c->op == f->op && c->p < f->p, "pff_prolong: levels must share the operator, coarse p < fine p");
   PFF_REQUIRE(f->mesh.offsets == nullptr, "pff_prolong: structured restriction required");
-  int rc = ensure_prolong_table(c, f);
-  if (rc) return rc;
-  const uint8_t* mc = level_mask(c);
-  const uint8_t* mf = level_mask(f);
-  if (prec == PFF_F64) PFF_CK(launch_prolong<double>(c->mesh, f->mesh, c->I64, (const double*)xc, (double*)xf, mc, mf, S(stream)));
-  else if (prec == PFF_F32 || prec == PFF_F32_BF16) PFF_CK(launch_prolong<float>(c->mesh, f->mesh, c->I32, (const float*)xc, (float*)xf, mc, mf, S(stream)));
-  else return fail(PFF_ERR_INVALID, "pff_prolong: unknown precision");
-  return PFF_OK;
+  return transfer_prolong(c, f, prec, xc, xf, false, S(stream));
 }
 
 int pff_restrict(pff_level* c, pff_level* f, pff_prec prec, const void* rf, void* rc_, void* stream) {
   PFF_REQUIRE(c && f && rf && rc_, "pff_restrict: null argument");
   PFF_REQUIRE(c->op == f->op && c->p < f->p, "pff_restrict: levels must share the operator, coarse p < fine p");
   PFF_REQUIRE(f->mesh.offsets == nullptr, "pff_restrict: structured restriction required");
-  int rc = ensure_prolong_table(c, f);
-  if (rc) return rc;
-  const uint8_t* mc = level_mask(c);
-  const uint8_t* mf = level_mask(f);
-  void* ev = (c->op->det && c->op->evec) ? c->op->evec : nullptr;
-  if (prec == PFF_F64) PFF_CK(launch_restrict<double>(c->mesh, f->mesh, c->I64, (const double*)rf, (double*)rc_, mc, mf, S(stream), ev));
-  else if (prec == PFF_F32 || prec == PFF_F32_BF16) PFF_CK(launch_restrict<float>(c->mesh, f->mesh, c->I32, (const float*)rf, (float*)rc_, mc, mf, S(stream), ev));
-  else return fail(PFF_ERR_INVALID, "pff_restrict: unknown precision");
-  return PFF_OK;
+  return transfer_restrict(c, f, prec, rf, nullptr, rc_, S(stream));
 }
 
 int pff_chebyshev_smooth(pff_level* L, pff_prec prec, int degree, double lmin, double lmax, const void* diag,

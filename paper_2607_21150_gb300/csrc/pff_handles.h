@@ -81,8 +81,7 @@ struct pff_level {
   bool is_fine = false;
   // prolongation table towards the finer level with order I_pf
   int I_pf = -1;
-  double* I64 = nullptr;
-  float* I32 = nullptr;
+  double I1[pff::kMaxQ * pff::kMaxQ] = {};  // [I_pf + 1][p + 1]
 };
 
 
@@ -96,6 +95,10 @@ int apply_blocks(pff_level* L, int prec, const void* x, void* y, int transpose, 
 // and the first product is left out (pff_abi.cpp).
 int smooth_level(pff_level* L, int prec, bool transpose, bool from_zero, int degree, double lmin, double lmax,
                  const void* diag, const void* b, void* x, void* work, cudaStream_t st);
+// pff_prolong and pff_restrict with x_f += P x_c (add) and r_c = P^T (b - r_f)
+// (b not null) (pff_abi.cpp).
+int transfer_prolong(pff_level* c, pff_level* f, int prec, const void* xc, void* xf, bool add, cudaStream_t st);
+int transfer_restrict(pff_level* c, pff_level* f, int prec, const void* rf, const void* b, void* rc, cudaStream_t st);
 // The Dirichlet mask of a level's rows (pff_abi.cpp).
 const uint8_t* level_rows_mask(const pff_level* L);
 // Releases the staging buffers, streams and events of pff_jacobian_apply_host (pff_hostio.cpp).

@@ -264,13 +264,15 @@ cudaError_t launch_masked_field_sums(const double* v, const uint8_t* sel, long l
 cudaError_t launch_state_summary(const uint8_t* flags, const double* hist, long long nq, const double* phi,
                                  long long nn, double* out, cudaStream_t st);
 cudaError_t launch_untile(const double* lin, double* out, long long nq, int Q, cudaStream_t st);
+// p-transfers (pff_transfer.cu); I1: host table [p_f + 1][p_c + 1] of the coarse
+// basis at the fine nodes.  add: x_f += P x_c.  b not null: r_c = P^T (b - r_f).
 template <typename T>
-cudaError_t launch_prolong(const MeshDev& mc, const MeshDev& mf, const T* I1, const T* xc, T* xf,
-                           const uint8_t* maskc, const uint8_t* maskf, cudaStream_t st);
-// evec (deterministic mode): element values and a node gather instead of atomics.
+cudaError_t launch_prolong(const MeshDev& mc, const MeshDev& mf, const double* I1, const T* xc, T* xf,
+                           const uint8_t* maskc, const uint8_t* maskf, const uint8_t* emaskf, int add,
+                           cudaStream_t st);
 template <typename T>
-cudaError_t launch_restrict(const MeshDev& mc, const MeshDev& mf, const T* I1, const T* rf, T* rc,
-                            const uint8_t* maskc, const uint8_t* maskf, cudaStream_t st, void* evec = nullptr);
+cudaError_t launch_restrict(const MeshDev& mc, const MeshDev& mf, const double* I1, const T* rf, const T* b, T* rc,
+                            const uint8_t* maskc, const uint8_t* maskf, const uint8_t* emaskf, cudaStream_t st);
 // Chebyshev updates between level actions (Ax null: x = 0; mask null: none).
 template <typename T>
 cudaError_t launch_cheb_first(long long n, const T* b, const T* Ax, const T* diag, const uint8_t* mask, T* r, T* d,

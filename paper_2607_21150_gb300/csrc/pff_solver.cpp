@@ -143,12 +143,6 @@ int dev_norm2(pff_solver* s, const double* v, long long n, double* out, cudaStre
   return PFF_OK;
 }
 
-int axpby_level(const LevelWork& w, void* y, const void* x, double a, double b, cudaStream_t st) {
-  if (w.prec == PFF_F64) S_CK(launch_axpby<double>((double*)y, (const double*)x, a, b, w.n, st));
-  else S_CK(launch_axpby<float>((float*)y, (const float*)x, a, b, w.n, st));
-  return PFF_OK;
-}
-
 int coarse_gmres(pff_solver* s, cudaStream_t st);
 
 // The assembled coarse level in the form of an h-level.
@@ -264,13 +258,10 @@ int vcycle(pff_solver* s, int l, cudaStream_t st) {
   if (coarsest) return PFF_OK;
   // residual, restriction, coarse correction, prolongation
   S_RC(level_apply(s, w, w.x, w.tmp, st));
-  if (w.prec == PFF_F64) S_CK(launch_bminus<double>((double*)w.tmp, (const double*)w.b, w.n, st));
-  else S_CK(launch_bminus<float>((float*)w.tmp, (const float*)w.b, w.n, st));
   LevelWork& c = s->lv[l + 1];
-  S_RC(pff_restrict(c.L, w.L, (pff_prec)w.prec, w.tmp, c.b, st));
+  S_RC(transfer_restrict(c.L, w.L, w.prec, w.tmp, w.b, c.b, st));
   S_RC(vcycle(s, l + 1, st));
-  S_RC(pff_prolong(c.L, w.L, (pff_prec)w.prec, c.x, w.tmp, st));
-  S_RC(axpby_level(w, w.x, w.tmp, 1.0, 1.0, st));
+  S_RC(transfer_prolong(c.L, w.L, w.prec, c.x, w.x, true, st));
   S_RC(cheb_level(s, w, false, s->prm.cheb_degree, s->prm.cheb_lo * w.lmax, s->prm.cheb_hi * w.lmax, st));
   return PFF_OK;
 }

@@ -1,5 +1,5 @@
 // Vector kernels: Dirichlet initialisation, the FP32 (and double-float)
-// planes of the stored linearisation, the p-multigrid transfer operators, the
+// planes of the stored linearisation, the
 // Chebyshev smoother updates, the export of the linearisation, reaction sums
 // and the geometric factors of mapped meshes.
 #include <cuda_bf16.h>
@@ -240,123 +240,6 @@ cudaError_t launch_split_words(const double* a, float* hi, float* lo, uint16_t* 
   return cudaGetLastError();
 }
 
-// Prolongation x_f = P x_c, P[f, c] = coarse Lagrange basis at the fine GLL
-// node (I1[a][b], a fine, b coarse, per direction).  One thread per fine node;
-// the owning element is any element whose closure holds the node (the coarse
-// space is continuous, so every choice gives the same value).
-template <typename T>
-__global__ void k_prolong(MeshDev mc, MeshDev mf, const T* __restrict__ I1, const T* __restrict__ xc,
-                          T* __restrict__ xf, const uint8_t* __restrict__ maskc, const uint8_t* __restrict__ maskf) {
-  const int Pc = mc.p + 1, Pf = mf.p + 1;
-  const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (n >= mf.nn) return;
-  const int I = (int)(n % mf.nnx);
-  const int J = (int)((n / mf.nnx) % mf.nny);
-  const int K = (int)(n / ((long long)mf.nnx * mf.nny));
-  const int idx[3] = {I, J, K};
-  const int ne[3] = {mf.nx, mf.ny, mf.nz};
-  int el[3], loc[3];
-  for (int d = 0; d < 3; ++d) {
-    int e = idx[d] / mf.p;
-    if (e >= ne[d]) e = ne[d] - 1;
-    el[d] = e;
-    loc[d] = idx[d] - mf.p * e;
-  }
-  for (int f = 0; f < 4; ++f) {
-    long long gf = f * mf.nn + n;
-    if (maskf && maskf[gf]) { xf[gf] = T(0); continue; }
-    T s = T(0);
-    for (int c = 0; c < Pc; ++c) {
-      T wz = I1[loc[2] * Pc + c];
-      for (int b = 0; b < Pc; ++b) {
-        T wyz = wz * I1[loc[1] * Pc + b];
-        for (int a = 0; a < Pc; ++a) {
-          long long nc = (long long)(mc.p * el[0] + a) + (long long)mc.nnx * ((long long)(mc.p * el[1] + b) + (long long)mc.nny * (mc.p * el[2] + c));
-          long long gc = f * mc.nn + nc;
-          if (maskc && maskc[gc]) continue;
-          s += wyz * I1[loc[0] * Pc + a] * xc[gc];
-        }
-      }
-    }
-    xf[gf] = s;
-  }
-  (void)Pf;
-}
-
-template <typename T>
-cudaError_t launch_prolong(const MeshDev& mc, const MeshDev& mf, const T* I1, const T* xc, T* xf,
-                           const uint8_t* maskc, const uint8_t* maskf, cudaStream_t st) {
-  if (mf.nn == 0) return cudaSuccess;
-  unsigned nb = (unsigned)((mf.nn + 255) / 256);
-  k_prolong<T><<<nb, 256, 0, st>>>(mc, mf, I1, xc, xf, maskc, maskf); note_launch();
-  return cudaGetLastError();
-}
-
-// Restriction r_c = P^T r_f, element by element: every element adds
-// I1^T-weighted fine residuals divided by the fine node's multiplicity (the
-// number of elements sharing it), which sums to exactly P^T r_f.  One thread
-// per (element, coarse local node).
-template <typename T>
-__global__ void k_restrict(MeshDev mc, MeshDev mf, const T* __restrict__ I1, const T* __restrict__ rf,
-                           T* __restrict__ rc, const uint8_t* __restrict__ maskc, const uint8_t* __restrict__ maskf,
-                           T* __restrict__ evec) {
-  const int Pc = mc.p + 1, Pf = mf.p + 1;
-  const int Pc3 = Pc * Pc * Pc;
-  const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (tid >= (long long)mc.nel * Pc3) return;
-  const int e = (int)(tid / Pc3);
-  const int lb = (int)(tid % Pc3);
-  const int b0 = lb % Pc, b1 = (lb / Pc) % Pc, b2 = lb / (Pc * Pc);
-  const int ex = e % mf.nx, ey = (e / mf.nx) % mf.ny, ez = e / (mf.nx * mf.ny);
-  const long long nc = (long long)(mc.p * ex + b0) + (long long)mc.nnx * ((long long)(mc.p * ey + b1) + (long long)mc.nny * (mc.p * ez + b2));
-  T acc[4] = {T(0), T(0), T(0), T(0)};
-  for (int c = 0; c < Pf; ++c) {
-    const int K = mf.p * ez + c;
-    const T mz = (c == 0 && ez > 0) || (c == mf.p && ez < mf.nz - 1) ? T(0.5) : T(1);
-    const T wz = I1[c * Pc + b2] * mz;
-    for (int b = 0; b < Pf; ++b) {
-      const int J = mf.p * ey + b;
-      const T my = (b == 0 && ey > 0) || (b == mf.p && ey < mf.ny - 1) ? T(0.5) : T(1);
-      const T wyz = wz * I1[b * Pc + b1] * my;
-      for (int a = 0; a < Pf; ++a) {
-        const int I = mf.p * ex + a;
-        const T mx = (a == 0 && ex > 0) || (a == mf.p && ex < mf.nx - 1) ? T(0.5) : T(1);
-        const T w = wyz * I1[a * Pc + b0] * mx;
-        const long long nf = I + (long long)mf.nnx * (J + (long long)mf.nny * K);
-        for (int f = 0; f < 4; ++f) {
-          long long gf = f * mf.nn + nf;
-          if (maskf && maskf[gf]) continue;
-          acc[f] += w * rf[gf];
-        }
-      }
-    }
-  }
-  if (evec) {  // deterministic: element values, summed per coarse node by k_node_gather
-    for (int f = 0; f < 4; ++f) evec[((long long)e * 4 + f) * Pc3 + lb] = acc[f];
-    return;
-  }
-  for (int f = 0; f < 4; ++f) {
-    long long gc = f * mc.nn + nc;
-    if (maskc && maskc[gc]) continue;
-    atomicAdd(rc + gc, acc[f]);
-  }
-}
-
-template <typename T>
-cudaError_t launch_restrict(const MeshDev& mc, const MeshDev& mf, const T* I1, const T* rf, T* rc,
-                            const uint8_t* maskc, const uint8_t* maskf, cudaStream_t st, void* evec) {
-  long long n = (long long)mc.nel * (mc.p + 1) * (mc.p + 1) * (mc.p + 1);
-  if (!evec) {
-    cudaError_t err = cudaMemsetAsync(rc, 0, sizeof(T) * 4 * mc.nn, st);
-    if (err != cudaSuccess) return err;
-  }
-  if (n == 0) return cudaSuccess;
-  k_restrict<T><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(mc, mf, I1, rf, rc, maskc, maskf, (T*)evec);
-  note_launch();
-  if (evec) return launch_node_gather(sizeof(T) == 8 ? 0 : 1, mc, evec, maskc, 3, nullptr, nullptr, rc, 0, mc.nn, st);
-  return cudaGetLastError();
-}
-
 // Chebyshev iteration (Saad, Alg. 12.1) on D^-1 A, between products:
 //   first: r = D^-1 (b - A x),  d = r / theta          (A x absent: x = 0)
 //   next:  x += d (xset: x = d);  r -= D^-1 A d;  d = c_d d + c_r r
@@ -588,14 +471,6 @@ cudaError_t launch_state_summary(const uint8_t* flags, const double* hist, long 
   return cudaGetLastError();
 }
 
-template cudaError_t launch_prolong<double>(const MeshDev&, const MeshDev&, const double*, const double*, double*,
-                                            const uint8_t*, const uint8_t*, cudaStream_t);
-template cudaError_t launch_prolong<float>(const MeshDev&, const MeshDev&, const float*, const float*, float*,
-                                           const uint8_t*, const uint8_t*, cudaStream_t);
-template cudaError_t launch_restrict<double>(const MeshDev&, const MeshDev&, const double*, const double*, double*,
-                                             const uint8_t*, const uint8_t*, cudaStream_t, void*);
-template cudaError_t launch_restrict<float>(const MeshDev&, const MeshDev&, const float*, const float*, float*,
-                                            const uint8_t*, const uint8_t*, cudaStream_t, void*);
 
 // Geometry of a mapped mesh at every quadrature point from the parent Jacobian
 // J = dX / dxi (rows 3 f + al of an eval of the nodal coordinates):
