@@ -63,8 +63,15 @@ int make_tables(int p, int Q, Tables& t) {
     }
   for (int i = 0; i < Q; ++i)
     for (int k = 0; k < Q; ++k) Dc[i * Q + k] = lagrange_deriv(xq.data(), Q, k, xq[i]);
-  for (int i = 0; i < Q * P; ++i) t.hB32[i] = (float)B[i];
-  for (int i = 0; i < Q * Q; ++i) t.hDc32[i] = (float)Dc[i];
+  for (int i = 0; i < Q * P; ++i) {
+    t.hB32[i] = (float)B[i];
+    t.hB[i] = B[i];
+    t.hDt[i] = Dt[i];
+  }
+  for (int i = 0; i < Q * Q; ++i) {
+    t.hDc32[i] = (float)Dc[i];
+    t.hDc[i] = Dc[i];
+  }
   int rc;
   if ((rc = upload(B, &t.B64))) return rc;
   if ((rc = upload(B, &t.B32))) return rc;
@@ -104,12 +111,12 @@ cudaError_t elem_dispatch(int Q, int P, int mode, const ElemArgs<T>& a, cudaStre
   return cudaErrorInvalidValue;
 }
 template <typename T>
-cudaError_t diag_dispatch(int Q, int P, const ElemArgs<T>& a, cudaStream_t st) {
+cudaError_t diag_dispatch(int Q, int P, const ElemArgs<T>& a, const Tables& t, cudaStream_t st) {
   switch (Q) {
-    case 2: return launch_diag_q2<T>(P, a, st);
-    case 3: return launch_diag_q3<T>(P, a, st);
-    case 4: return launch_diag_q4<T>(P, a, st);
-    case 5: return launch_diag_q5<T>(P, a, st);
+    case 2: return launch_diag_q2<T>(P, a, t.hB, t.hDt, st);
+    case 3: return launch_diag_q3<T>(P, a, t.hB, t.hDt, st);
+    case 4: return launch_diag_q4<T>(P, a, t.hB, t.hDt, st);
+    case 5: return launch_diag_q5<T>(P, a, t.hB, t.hDt, st);
   }
   return cudaErrorInvalidValue;
 }
@@ -240,7 +247,7 @@ int diag_t(pff_level* L, T* diag, cudaStream_t st) {
   ElemArgs<T> a = level_args<T>(L);
   a.y = diag;
   if (det) a.evec = op->evec;
-  PFF_CK(diag_dispatch<T>(op->Q, L->p + 1, a, st));
+  PFF_CK(diag_dispatch<T>(op->Q, L->p + 1, a, L->tab, st));
   if (det)
     PFF_CK(launch_node_gather(sizeof(T) == 8 ? 0 : 1, L->mesh, op->evec, level_mask(L), 2, nullptr, nullptr, diag, 0,
                               L->mesh.nn, st));

@@ -800,123 +800,184 @@ k_elem(const ElemArgs<T> a) {
 
 // Diagonal of the element operators: for each field f and node a,
 //   sum_q sum_{alpha,beta} D_{f alpha, f beta}(q) d_alpha N_a d_beta N_a
-// (+ the value term of the phase field), sum-factorised per (alpha, beta)
-// pair with the 1D products B*B, B*D, D*D.
+// (+ the value term of the phase field), sum-factorised with the 1D products
+// BB, BD, DD of the basis and its derivative (kinds 0, 1, 2 per direction).
+//
+// The (alpha, beta) terms of a field meet as early as their kinds allow: the
+// six (kx, ky, kz) = 200, 110, 101, 020, 011, 002 leave the z contraction
+// separately (the value term, 000, joins 002 there), the y contraction sums
+// them by kx into three, the x contraction into one.  A field takes three
+// barriers, and its words (whole quads in FP32) are requested while the former
+// field is contracted.  Term by term, as before, a block passed 66 barriers and
+// waited for each term's words: 290 us at 24x24x72 Q3 FP32, 113 us now (the
+// quads that hold the words are 456 MB, 68 us at the copy rate).
+constexpr int kDiagTerms = 6;
+// Words of field f at the thread's points, one value per term (f = 3: term 5
+// gets the value word besides, in v).
+template <int Q, typename T>
+__device__ __forceinline__ void diag_words(const ElemArgs<T>& a, int f, int t, bool valid, T w[kDiagTerms][Q], T v[Q]) {
+  constexpr long long EB = elems_per_block(Q), run = (long long)Q * Q * EB, stride = run * Q;
+  const T* lin = a.lin + (a.blk0 + blockIdx.x) * (long long)kLinWords * stride;
+#pragma unroll
+  for (int k = 0; k < Q; ++k) {
+#pragma unroll
+    for (int m = 0; m < kDiagTerms; ++m) w[m][k] = T(0);
+    v[k] = T(0);
+  }
+  if (!valid) return;
+  // first derivative pairs (alpha, beta) of the terms: 00, 01, 02, 11, 12, 22
+  if (f < 3) {
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+      if constexpr (sizeof(T) == 4) {
+        // the six words lie in three quads; f is uniform, so are the selections
+        const float* p = lin + (long long)k * 4 * run + 4 * t;
+        const int q0 = f == 0 ? 0 : f == 1 ? 6 : 9;   // quads of words (f0, f0 .. f2)
+        const int q1 = f == 0 ? 2 : f == 1 ? 7 : 10;
+        const int q2 = f == 0 ? 4 : f == 1 ? 8 : 11;
+        const float4 A = ld_lin4<false>(p + q0 * 4 * stride), B = ld_lin4<false>(p + q1 * 4 * stride),
+                     C = ld_lin4<false>(p + q2 * 4 * stride);
+        if (f == 0) {         // words 0, 1, 2, 9, 10, 17
+          w[0][k] = A.x; w[1][k] = A.y; w[2][k] = A.z; w[3][k] = B.y; w[4][k] = B.z; w[5][k] = C.y;
+        } else if (f == 1) {  // words 24, 25, 26, 30, 31, 35
+          w[0][k] = A.x; w[1][k] = A.y; w[2][k] = A.z; w[3][k] = B.z; w[4][k] = B.w; w[5][k] = C.w;
+        } else {              // words 39, 40, 41, 42, 43, 44
+          w[0][k] = A.w; w[1][k] = B.x; w[2][k] = B.y; w[3][k] = B.z; w[4][k] = B.w; w[5][k] = C.x;
+        }
+      } else {
+        const T* p = lin + (long long)k * run + t;
+        int m = 0;
+#pragma unroll
+        for (int al = 0; al < 3; ++al)
+#pragma unroll
+          for (int be = al; be < 3; ++be) w[m++][k] = ldg(p + (long long)sym9(3 * f + al, 3 * f + be) * stride);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+      w[1][k] *= T(2); w[2][k] *= T(2); w[4][k] *= T(2);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+      auto word = [&](int wd) {
+        return ldg(lin + (sizeof(T) == 4 ? lin32_word(wd, k, t, stride, run) : (long long)wd * stride + (long long)k * run + t));
+      };
+      w[0][k] = word(kWK); w[3][k] = word(kWK + 1); w[5][k] = word(kWK + 2); v[k] = word(kWD);
+      if (a.kx) {  // mapped mesh: 2 K_al,be d_al N d_be N
+        w[1][k] = T(2) * word(kWKX); w[2][k] = T(2) * word(kWKX + 1); w[4][k] = T(2) * word(kWKX + 2);
+      }
+    }
+  }
+}
+// The 1D products [kind][q][node] as kernel parameters (constant-bank operands;
+// from shared memory they took a load per two multiply-adds: 153 us at the size
+// above, 113 us now), rounded once from the FP64 products.
+template <typename T, int P, int Q> struct DiagMats { T m[3 * Q * P]; };
+template <int P, int Q> __host__ __device__ constexpr int diag_smem_words() {
+  return kDiagTerms * P * Q * Q + 3 * P * P * Q;
+}
+
 template <int P, int Q, typename T>
-__global__ void __launch_bounds__(Q * Q * elems_per_block(Q))
-k_diag(const ElemArgs<T> a) {
+__global__ void __launch_bounds__(Q * Q * elems_per_block(Q), 2)
+k_diag(const ElemArgs<T> a, const DiagMats<T, P, Q> mats) {
   constexpr int EB = elems_per_block(Q);
-  constexpr int Q2 = Q * Q, Q3 = Q * Q * Q, P3 = P * P * P;
+  constexpr int Q2 = Q * Q, P3 = P * P * P;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sm = reinterpret_cast<T*>(smem_raw);
   const int t = threadIdx.x;
   const int el = t / Q2, ij = t % Q2;
-  const int i = ij % Q, j = ij / Q;
   const int e = (a.blk0 + blockIdx.x) * EB + el;
   const bool valid = e < a.mesh.nel;
-  T* M = sm;  // [3][Q][P]: BB, BD, DD
-  for (int idx = t; idx < Q * P; idx += blockDim.x) {
-    T b = a.B[idx], d = a.Dt[idx];
-    M[idx] = b * b;
-    M[Q * P + idx] = b * d;
-    M[2 * Q * P + idx] = d * d;
-  }
-  T* base = sm + mat_smem_words<P, Q>() + el * elem_smem_words<Q>();
-  T* bufA = base;           // Q^3
-  T* bufB = base + Q3;      // Q^3
-  T* acc = base + 2 * Q3;   // [4][P3]
-  for (int idx = ij; idx < 4 * P3; idx += Q2) acc[idx] = T(0);
-  __syncthreads();
-  const long long blk_words = (long long)kLinWords * Q3 * EB;
-  const long long stride = (long long)Q3 * EB;
-  // term list: (field, word, dim-kinds mask, weight)
-  // u fields: pairs alpha <= beta; phase field: value term and 3 gradient terms
-  const int nterms = a.kx ? 25 : 22;
+  T* Zb = sm + el * diag_smem_words<P, Q>();  // [term][c][j][i], then [c][b][a]
+  T* Yb = Zb + kDiagTerms * P * Q2;                                     // [kx][c][b][i]
+  const bool masked = a.mask && valid && (!a.emask || a.emask[e]);
+  const long long nn = a.mesh.nn;
+  // kinds of the terms 00, 01, 02, 11, 12, 22
+  constexpr int KX[kDiagTerms] = {2, 1, 1, 0, 0, 0}, KY[kDiagTerms] = {0, 1, 0, 2, 1, 0}, KZ[kDiagTerms] = {0, 0, 1, 0, 1, 2};
+  T w[kDiagTerms][Q], v[Q];
+  diag_words<Q, T>(a, 0, t, valid, w, v);
 #pragma unroll 1
-  for (int term = 0; term < nterms; ++term) {
-    int f, word, kx, ky, kz;
-    T wgt = T(1);
-    if (term < 18) {
-      f = term / 6;
-      int pr = term % 6;
-      const int al_of[6] = {0, 1, 2, 0, 0, 1};
-      const int be_of[6] = {0, 1, 2, 1, 2, 2};
-      int al = al_of[pr], be = be_of[pr];
-      word = sym9(3 * f + al, 3 * f + be);
-      if (al != be) wgt = T(2);
-      int kd[3];
+  for (int f = 0; f < 4; ++f) {
 #pragma unroll
-      for (int d = 0; d < 3; ++d) kd[d] = (d == al) + (d == be);  // 0: BB, 1: BD, 2: DD
-      kx = kd[0]; ky = kd[1]; kz = kd[2];
-    } else {
-      f = 3;
-      if (term == 18) { word = kWD; kx = ky = kz = 0; }
-      else if (term < 22) {
-        int al = term - 19;
-        word = kWK + al;
-        kx = (al == 0) ? 2 : 0; ky = (al == 1) ? 2 : 0; kz = (al == 2) ? 2 : 0;
-      } else {  // off-diagonal phase-gradient pair (al, be): 2 K_al,be d_al N d_be N
-        const int pr = term - 22;               // 01, 02, 12
-        const int al = (pr == 2) ? 1 : 0, be = (pr == 0) ? 1 : 2;
-        word = kWKX + pr;
-        wgt = T(2);
-        kx = (al == 0) + (be == 0); ky = (al == 1) + (be == 1); kz = (al == 2) + (be == 2);
+    for (int c = 0; c < P; ++c)
+#pragma unroll
+      for (int m = 0; m < kDiagTerms; ++m) {
+        T s = T(0);
+#pragma unroll
+        for (int k = 0; k < Q; ++k) s += mats.m[(KZ[m] * Q + k) * P + c] * w[m][k];
+        if (m == 5) {
+          T u = T(0);
+#pragma unroll
+          for (int k = 0; k < Q; ++k) u += mats.m[k * P + c] * v[k];
+          s += u;
+        }
+        Zb[(m * P + c) * Q2 + ij] = s;
+      }
+    __syncthreads();
+    if (f < 3) diag_words<Q, T>(a, f + 1, t, valid, w, v);
+    for (int idx = ij; idx < P * Q; idx += Q2) {  // y: lines (c, i)
+      const int i = idx % Q, c = idx / Q;
+      T s[3][P];
+#pragma unroll
+      for (int g = 0; g < 3; ++g)
+#pragma unroll
+        for (int bb = 0; bb < P; ++bb) s[g][bb] = T(0);
+#pragma unroll
+      for (int m = 0; m < kDiagTerms; ++m) {
+        T u[P];  // each term's sum by itself (short chains keep FP32's error at the former level)
+#pragma unroll
+        for (int bb = 0; bb < P; ++bb) u[bb] = T(0);
+#pragma unroll
+        for (int j = 0; j < Q; ++j) {
+          const T z = Zb[(m * P + c) * Q2 + j * Q + i];
+#pragma unroll
+          for (int bb = 0; bb < P; ++bb) u[bb] += mats.m[(KY[m] * Q + j) * P + bb] * z;
+        }
+#pragma unroll
+        for (int bb = 0; bb < P; ++bb) s[KX[m]][bb] += u[bb];
+      }
+#pragma unroll
+      for (int g = 0; g < 3; ++g)
+#pragma unroll
+        for (int bb = 0; bb < P; ++bb) Yb[((g * P + c) * P + bb) * Q + i] = s[g][bb];
+    }
+    __syncthreads();
+    for (int idx = ij; idx < P * P; idx += Q2) {  // x: lines (c, b)
+      T s[P];
+#pragma unroll
+      for (int aa = 0; aa < P; ++aa) s[aa] = T(0);
+#pragma unroll
+      for (int g = 0; g < 3; ++g) {
+        T u[P];
+#pragma unroll
+        for (int aa = 0; aa < P; ++aa) u[aa] = T(0);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+          const T y = Yb[(g * P * P + idx) * Q + i];
+#pragma unroll
+          for (int aa = 0; aa < P; ++aa) u[aa] += mats.m[(g * Q + i) * P + aa] * y;
+        }
+#pragma unroll
+        for (int aa = 0; aa < P; ++aa) s[aa] += u[aa];
+      }
+#pragma unroll
+      for (int aa = 0; aa < P; ++aa) Zb[idx * P + aa] = s[aa];
+    }
+    __syncthreads();
+    if (valid) {
+      if (a.evec) {  // deterministic: element-local values, summed per node by k_node_gather
+        T* ev = static_cast<T*>(a.evec) + ((long long)e * 4 + f) * P3;
+        for (int idx = ij; idx < P3; idx += Q2) ev[idx] = Zb[idx];
+      } else {
+        for (int idx = ij; idx < P3; idx += Q2) {
+          const long long g = f * nn + node_of<P, Q>(a.mesh, e, idx % P, (idx / P) % P, idx / (P * P));
+          if (masked && a.mask[g]) continue;
+          atomicAdd(a.y + g, Zb[idx]);
+        }
       }
     }
-    const T* Mx = M + kx * Q * P;
-    const T* My = M + ky * Q * P;
-    const T* Mz = M + kz * Q * P;
-    // coefficients on the column (i, j, :) -> z contraction in registers
-    T col[Q];
-#pragma unroll
-    for (int k = 0; k < Q; ++k) {
-      const long long off = (a.blk0 + blockIdx.x) * blk_words + (sizeof(T) == 4 ? lin32_word(word, k, t, stride, Q2 * EB)
-                                                                    : (long long)word * stride + (long long)k * Q2 * EB + t);
-      col[k] = valid ? ldg(a.lin + off) * wgt : T(0);
-    }
-#pragma unroll
-    for (int c = 0; c < P; ++c) {
-      T s = T(0);
-#pragma unroll
-      for (int k = 0; k < Q; ++k) s += Mz[k * P + c] * col[k];
-      bufA[c * Q2 + j * Q + i] = s;
-    }
-    __syncthreads();
-    for (int idx = ij; idx < P * P * Q; idx += Q2) {
-      int ii = idx % Q, bb = (idx / Q) % P, c = idx / (P * Q);
-      T s = T(0);
-#pragma unroll
-      for (int jj = 0; jj < Q; ++jj) s += My[jj * P + bb] * bufA[c * Q2 + jj * Q + ii];
-      bufB[idx] = s;
-    }
-    __syncthreads();
-    for (int idx = ij; idx < P3; idx += Q2) {
-      int aa = idx % P, r = idx / P;
-      T s = T(0);
-#pragma unroll
-      for (int ii = 0; ii < Q; ++ii) s += Mx[ii * P + aa] * bufB[r * Q + ii];
-      acc[f * P3 + idx] += s;
-    }
-    __syncthreads();
-  }
-  if (!valid) return;
-  if (a.evec) {  // deterministic: element-local values, summed per node by k_node_gather
-    T* ev = static_cast<T*>(a.evec) + (long long)e * 4 * P3;
-    for (int idx = ij; idx < P3; idx += Q2)
-#pragma unroll
-      for (int f = 0; f < 4; ++f) ev[f * P3 + idx] = acc[f * P3 + idx];
-    return;
-  }
-  const long long nn = a.mesh.nn;
-  for (int idx = ij; idx < P3; idx += Q2) {
-    int aa = idx % P, bb = (idx / P) % P, cc = idx / (P * P);
-    long long n = node_of<P, Q>(a.mesh, e, aa, bb, cc);
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      long long g = f * nn + n;
-      if (a.mask && a.mask[g]) continue;
-      atomicAdd(a.y + g, acc[f * P3 + idx]);
-    }
+    __syncthreads();  // the next field's terms overwrite Zb
   }
 }
 
@@ -963,14 +1024,20 @@ cudaError_t launch_elem_pq(int mode, const ElemArgs<T>& a, cudaStream_t st) {
 }
 
 template <int P, int Q, typename T>
-cudaError_t launch_diag_pq(const ElemArgs<T>& a, cudaStream_t st) {
+cudaError_t launch_diag_pq(const ElemArgs<T>& a, const double* B, const double* D, cudaStream_t st) {
+  DiagMats<T, P, Q> mats;
+  for (int i = 0; i < Q * P; ++i) {
+    mats.m[i] = (T)(B[i] * B[i]);
+    mats.m[Q * P + i] = (T)(B[i] * D[i]);
+    mats.m[2 * Q * P + i] = (T)(D[i] * D[i]);
+  }
   constexpr int EB = elems_per_block(Q);
   int nblk = (a.mesh.nel + EB - 1) / EB;
   if (nblk == 0) return cudaSuccess;
-  size_t smem = sizeof(T) * (size_t)(mat_smem_words<P, Q>() + EB * elem_smem_words<Q>());
+  size_t smem = sizeof(T) * (size_t)(EB * diag_smem_words<P, Q>());
   auto k = k_diag<P, Q, T>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k<<<nblk, Q * Q * EB, smem, st>>>(a); note_launch();
+  k<<<nblk, Q * Q * EB, smem, st>>>(a, mats); note_launch();
   return cudaGetLastError();
 }
 

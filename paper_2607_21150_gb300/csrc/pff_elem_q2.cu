@@ -11,16 +11,16 @@ cudaError_t launch_elem_q2(int P, int mode, const ElemArgs<T>& a, cudaStream_t s
   }
 }
 template <typename T>
-cudaError_t launch_diag_q2(int P, const ElemArgs<T>& a, cudaStream_t st) {
+cudaError_t launch_diag_q2(int P, const ElemArgs<T>& a, const double* B, const double* D, cudaStream_t st) {
   switch (P) {
-    case 2: return launch_diag_pq<2, 2, T>(a, st);
+    case 2: return launch_diag_pq<2, 2, T>(a, B, D, st);
     default: return cudaErrorInvalidValue;
   }
 }
 template cudaError_t launch_elem_q2<double>(int, int, const ElemArgs<double>&, cudaStream_t);
 template cudaError_t launch_elem_q2<float>(int, int, const ElemArgs<float>&, cudaStream_t);
 template cudaError_t launch_elem_q2<df64>(int, int, const ElemArgs<df64>&, cudaStream_t);
-template cudaError_t launch_diag_q2<double>(int, const ElemArgs<double>&, cudaStream_t);
-template cudaError_t launch_diag_q2<float>(int, const ElemArgs<float>&, cudaStream_t);
+template cudaError_t launch_diag_q2<double>(int, const ElemArgs<double>&, const double*, const double*, cudaStream_t);
+template cudaError_t launch_diag_q2<float>(int, const ElemArgs<float>&, const double*, const double*, cudaStream_t);
 
 }  // namespace pff

@@ -13,18 +13,18 @@ cudaError_t launch_elem_q4(int P, int mode, const ElemArgs<T>& a, cudaStream_t s
   }
 }
 template <typename T>
-cudaError_t launch_diag_q4(int P, const ElemArgs<T>& a, cudaStream_t st) {
+cudaError_t launch_diag_q4(int P, const ElemArgs<T>& a, const double* B, const double* D, cudaStream_t st) {
   switch (P) {
-    case 2: return launch_diag_pq<2, 4, T>(a, st);
-    case 3: return launch_diag_pq<3, 4, T>(a, st);
-    case 4: return launch_diag_pq<4, 4, T>(a, st);
+    case 2: return launch_diag_pq<2, 4, T>(a, B, D, st);
+    case 3: return launch_diag_pq<3, 4, T>(a, B, D, st);
+    case 4: return launch_diag_pq<4, 4, T>(a, B, D, st);
     default: return cudaErrorInvalidValue;
   }
 }
 template cudaError_t launch_elem_q4<double>(int, int, const ElemArgs<double>&, cudaStream_t);
 template cudaError_t launch_elem_q4<float>(int, int, const ElemArgs<float>&, cudaStream_t);
 template cudaError_t launch_elem_q4<df64>(int, int, const ElemArgs<df64>&, cudaStream_t);
-template cudaError_t launch_diag_q4<double>(int, const ElemArgs<double>&, cudaStream_t);
-template cudaError_t launch_diag_q4<float>(int, const ElemArgs<float>&, cudaStream_t);
+template cudaError_t launch_diag_q4<double>(int, const ElemArgs<double>&, const double*, const double*, cudaStream_t);
+template cudaError_t launch_diag_q4<float>(int, const ElemArgs<float>&, const double*, const double*, cudaStream_t);
 
 }  // namespace pff

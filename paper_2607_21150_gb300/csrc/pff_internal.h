@@ -220,10 +220,12 @@ struct ElemArgs {
 };
 
 // One translation unit per quadrature size Q (pff_elem_q<Q>.cu); each covers
-// every basis size P <= Q in both precisions.
+// every basis size P <= Q in both precisions.  launch_diag: B, D = host tables
+// [Q][P] of the basis and its derivative.
 #define PFF_DECLARE_ELEM_Q(QQ)                                                                  \
   template <typename T> cudaError_t launch_elem_q##QQ(int P, int mode, const ElemArgs<T>& a, cudaStream_t st); \
-  template <typename T> cudaError_t launch_diag_q##QQ(int P, const ElemArgs<T>& a, cudaStream_t st);
+  template <typename T> cudaError_t launch_diag_q##QQ(int P, const ElemArgs<T>& a, const double* B, const double* D, \
+                                                      cudaStream_t st);
 PFF_DECLARE_ELEM_Q(2)
 PFF_DECLARE_ELEM_Q(3)
 PFF_DECLARE_ELEM_Q(4)
