@@ -68,10 +68,8 @@ int make_tables(int p, int Q, Tables& t) {
     t.hB[i] = B[i];
     t.hDt[i] = Dt[i];
   }
-  for (int i = 0; i < Q * Q; ++i) {
-    t.hDc32[i] = (float)Dc[i];
-    t.hDc[i] = Dc[i];
-  }
+  for (int i = 0; i < Q * Q; ++i) t.hDc32[i] = (float)Dc[i];
+  t.fix = fix_table(P, Q, B.data(), Dc.data());
   int rc;
   if ((rc = upload(B, &t.B64))) return rc;
   if ((rc = upload(B, &t.B32))) return rc;
@@ -160,6 +158,7 @@ ElemArgs<T> level_args(const pff_level* L) {
   a.Dc = tabDc<T>(L->tab);
   a.Dt = tabDt<T>(L->tab);
   a.lin = linOf<T>(L->op);
+  a.fix = L->tab.fix;
   a.nq = L->op->nq;
   a.kx = L->op->geo != nullptr;
   for (int d = 0; d < 3; ++d) a.s[d] = L->op->geom.s[d];
@@ -676,6 +675,7 @@ int pff_op_set_geometry(pff_op* op, const double* X, void* stream) {
   a.B = op->tab.B64;
   a.Dc = op->tab.Dc64;
   a.Dt = op->tab.Dt64;
+  a.fix = op->tab.fix;
   a.scratch = op->io;
   a.nq = nq;
   for (int d = 0; d < 3; ++d) a.s[d] = 1.0;
@@ -709,6 +709,7 @@ int pff_residual(pff_op* op, const double* z, double* r, void* stream) {
   a.B = op->tab.B64;
   a.Dc = op->tab.Dc64;
   a.Dt = op->tab.Dt64;
+  a.fix = op->tab.fix;
   a.scratch = op->io;
   a.nq = op->nq;
   a.geo = op->geo;
@@ -767,6 +768,7 @@ int pff_reaction(pff_op* op, const uint8_t* sel, double* out4, void* stream) {
   a.B = op->tab.B64;
   a.Dc = op->tab.Dc64;
   a.Dt = op->tab.Dt64;
+  a.fix = op->tab.fix;
   a.scratch = op->io;
   a.nq = op->nq;
   PFF_CK(elem_dispatch<double>(op->Q, op->p + 1, kBack, a, st));

@@ -3,7 +3,9 @@
 // Gauss-Lobatto-Legendre nodes by the Newton iteration on x P_p(x) - P_{p-1}(x)
 // started from Chebyshev-Gauss-Lobatto points; Gauss-Legendre points by Newton
 // on P_Q; Lagrange polynomials in barycentric form.
+#include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "pff_internal.h"
@@ -97,6 +99,44 @@ double lagrange_deriv(const double* nodes, int n, int a, double t) {
   for (int b = 0; b < n; ++b)
     if (b != a) s += 1.0 / (t - nodes[b]);
   return lagrange(nodes, n, a, t) * s;
+}
+
+FixTab fix_table(int P, int Q, const double* B, const double* Dc) {
+  FixTab t;
+  std::memset(&t, 0, sizeof(t));
+  double rowB = 0.0, colB = 0.0, colD = 0.0, maxD = 0.0;
+  for (int q = 0; q < Q; ++q) {
+    double b = 0.0, c = 0.0;
+    for (int p = 0; p < P; ++p) b += std::fabs(B[q * P + p]);
+    for (int k = 0; k < Q; ++k) {
+      c += std::fabs(Dc[k * Q + q]);
+      maxD = std::max(maxD, std::fabs(Dc[q * Q + k]));
+    }
+    rowB = std::max(rowB, b);
+    colD = std::max(colD, c);
+  }
+  for (int p = 0; p < P; ++p) {
+    double b = 0.0;
+    for (int q = 0; q < Q; ++q) b += std::fabs(B[q * P + p]);
+    colB = std::max(colB, b);
+  }
+  // |D 2^sD| <= 2^60; a derivative comes out divided by 2^(60 - sD)
+  t.sD = 60 - std::max(0, (int)std::ceil(std::log2(maxD)));
+  const double dd = std::ldexp(1.0, 60 - t.sD);
+  auto halves = [](double v, int s, int* h, int* l) {
+    const long long b = std::llrint(std::ldexp(v, s));
+    *h = (int)((b + (1LL << 29)) >> 30);
+    *l = (int)(b - ((long long)*h << 30));
+  };
+  for (int k = 0; k < Q * P; ++k) halves(B[k], 60, t.Bh + k, t.Bl + k);
+  for (int k = 0; k < Q * Q; ++k) halves(Dc[k], t.sD, t.Dh + k, t.Dl + k);
+  // no stage's input passes 2^61 (its halves fit 32 bits and the sums 64): forward
+  // after three interpolations, transposed before the last of them; the three
+  // derivative sums of a column are below 2 2^eD times the largest output
+  t.wf = (int)std::floor(60.9 - 3.0 * std::log2(std::max(1.0, rowB)));
+  t.eD = (int)std::floor(std::log2(3.0 * colD));
+  t.wb = (int)std::floor(60.95 - std::log2(std::ldexp(3.0 * colD, -t.eD)) - 2.0 * std::log2(std::max(1.0, colB)));
+  return t;
 }
 
 }  // namespace pff

@@ -612,7 +612,7 @@ __device__ __forceinline__ void set_column_at(T (&y)[Q], int k, T v) {
 // single resident block the barriers of the slice loop leave the SM idle.
 template <typename T> constexpr int elem_min_blocks() { return sizeof(T) == 4 ? 3 : 2; }
 
-template <int P, int Q, typename T, int MODE>
+template <int P, int Q, typename T>
 __global__ void __launch_bounds__(Q * Q * elems_per_block(Q), elem_min_blocks<T>())
 k_elem(const ElemArgs<T> a) {
   constexpr int EB = elems_per_block(Q);
@@ -630,7 +630,7 @@ k_elem(const ElemArgs<T> a) {
   T* Dcs = Bs + Q * P;
   for (int idx = t; idx < Q * P; idx += blockDim.x) Bs[idx] = from_store<T>(a.B[idx]);
   for (int idx = t; idx < Q * Q; idx += blockDim.x) Dcs[idx] = from_store<T>(a.Dc[idx]);
-  constexpr bool kSplit = elem_split<T>() && MODE == kApply;
+  constexpr bool kSplit = elem_split<T>();
   T* base = sm + mat_smem_words<P, Q>() + el * elem_smem_words_t<Q, T>();
   // split form: bufB first (read by every slice's gradients), then bufA which
   // extends to the 8 x Q^3 derivative outputs of the pointwise stage
@@ -640,44 +640,7 @@ k_elem(const ElemArgs<T> a) {
   if constexpr (kSplit)
     for (int k = 0; k < kPrefetchAhead; ++k) prefetch_slice<Q, T>(a, k, t);
 
-  if constexpr (MODE == kApply || MODE == kEval) forward<P, Q, T>(a, s, e, valid, ij);
-
-  if constexpr (MODE == kEval) {
-    if (valid) {
-      T sd[3];  // d xi / dX of the box
-#pragma unroll
-      for (int al = 0; al < 3; ++al) sd[al] = from_store<T>(a.s[al]);
-#pragma unroll 1
-      for (int k = 0; k < Q; ++k) {
-        T g[4][3], phi;
-        grad_at<P, Q, T>(s, i, j, k, g, phi);
-        long long q = (long long)e * Q3 + k * Q2 + j * Q + i;
-        if (a.geo) {  // mapped mesh: reference gradient = parent gradient x d xi / dX
-          T G[3][3];
-#pragma unroll
-          for (int al = 0; al < 3; ++al)
-#pragma unroll
-            for (int A = 0; A < 3; ++A) G[al][A] = from_store<T>(a.geo[(3 * al + A) * a.nq + q]);
-#pragma unroll
-          for (int f = 0; f < 4; ++f)
-#pragma unroll
-            for (int A = 0; A < 3; ++A) {
-              const T v = madd(madd(mul(g[f][0], G[0][A]), g[f][1], G[1][A]), g[f][2], G[2][A]);
-              a.scratch[((f < 3) ? 3 * f + A : 10 + A) * a.nq + q] = to_vec(v);
-            }
-        } else {
-#pragma unroll
-          for (int f = 0; f < 3; ++f)
-#pragma unroll
-            for (int al = 0; al < 3; ++al) a.scratch[(3 * f + al) * a.nq + q] = to_vec(mul(g[f][al], sd[al]));
-#pragma unroll
-          for (int al = 0; al < 3; ++al) a.scratch[(10 + al) * a.nq + q] = to_vec(mul(g[3][al], sd[al]));
-        }
-        a.scratch[9 * a.nq + q] = to_vec(phi);
-      }
-    }
-    return;
-  }
+  forward<P, Q, T>(a, s, e, valid, ij);
 
   T Y[4][Q];
 #pragma unroll
@@ -729,46 +692,25 @@ k_elem(const ElemArgs<T> a) {
     backward<P, Q, T>(a, s, e, valid, ij, Y);
     return;
   }
-  // The double-float action keeps this loop rolled: its pointwise map takes
-  // about ten times the instructions of the FP64 one, and five unrolled
-  // slices, each with both orientations of the map, overflow the instruction
-  // cache.  Y[f][k] is then selected and written back by column_at /
-  // set_column_at; o0 joins Y[3][k] after the barrier, in the same order of
-  // operations as the FP64 loop.
-  constexpr bool kRollSlices = sizeof(T) != sizeof(typename ElemTypes<T>::L);
-#pragma unroll(kRollSlices ? 1 : Q)
+  // The slice loop stays rolled: the pointwise map takes about ten times the
+  // instructions of an FP64 one, and five unrolled slices, each with both
+  // orientations of the map, overflow the instruction cache.  Y[f][k] is then
+  // selected and written back by column_at / set_column_at.
+#pragma unroll 1
   for (int k = 0; k < Q; ++k) {
-    T o[4][3], o0 = zero<T>();
-    if constexpr (MODE == kApply) {
-      T g[4][3], phi;
-      grad_at<P, Q, T>(s, i, j, k, g, phi);
-      if (valid) {
-        jac_at<Q, T>(a, k, t, g, phi, o, o0);
-      } else {
+    T g[4][3], phi, o[4][3], o0 = zero<T>();
+    grad_at<P, Q, T>(s, i, j, k, g, phi);
+    if (valid) {
+      jac_at<Q, T>(a, k, t, g, phi, o, o0);
+    } else {
 #pragma unroll
-        for (int f = 0; f < 4; ++f) o[f][0] = o[f][1] = o[f][2] = zero<T>();
-      }
-    } else {  // kBack: integrands from the pointwise kernel
-      if (valid) {
-        long long q = (long long)e * Q3 + k * Q2 + j * Q + i;
-#pragma unroll
-        for (int f = 0; f < 3; ++f)
-#pragma unroll
-          for (int al = 0; al < 3; ++al) o[f][al] = from_store<T>(a.scratch[(3 * f + al) * a.nq + q]);
-        o0 = from_store<T>(a.scratch[9 * a.nq + q]);
-#pragma unroll
-        for (int al = 0; al < 3; ++al) o[3][al] = from_store<T>(a.scratch[(10 + al) * a.nq + q]);
-      } else {
-#pragma unroll
-        for (int f = 0; f < 4; ++f) o[f][0] = o[f][1] = o[f][2] = zero<T>();
-      }
+      for (int f = 0; f < 4; ++f) o[f][0] = o[f][1] = o[f][2] = zero<T>();
     }
     // transposed z-derivative (own column) and the value term
 #pragma unroll
     for (int f = 0; f < 4; ++f)
 #pragma unroll
       for (int kk = 0; kk < Q; ++kk) Y[f][kk] = madd(Y[f][kk], s.Dc[k * Q + kk], o[f][2]);
-    if constexpr (!kRollSlices) Y[3][k] = add(Y[3][k], o0);
     // x- and y-derivative outputs of this slice through shared memory
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
@@ -778,20 +720,14 @@ k_elem(const ElemArgs<T> a) {
     __syncthreads();
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-      T acc;
-      if constexpr (kRollSlices) {
-        acc = column_at<Q>(Y[f], k);
-        if (f == 3) acc = add(acc, o0);
-      } else {
-        acc = Y[f][k];
-      }
+      T acc = column_at<Q>(Y[f], k);
+      if (f == 3) acc = add(acc, o0);
 #pragma unroll
       for (int m = 0; m < Q; ++m) {
         acc = madd(acc, s.Dc[m * Q + i], s.slice[(2 * f) * Q2 + j * Q + m]);
         acc = madd(acc, s.Dc[m * Q + j], s.slice[(2 * f + 1) * Q2 + m * Q + i]);
       }
-      if constexpr (kRollSlices) set_column_at<Q>(Y[f], k, acc);
-      else Y[f][k] = acc;
+      set_column_at<Q>(Y[f], k, acc);
     }
     __syncthreads();
   }
@@ -983,44 +919,34 @@ k_diag(const ElemArgs<T> a, const DiagMats<T, P, Q> mats) {
 
 }  // namespace pff
 
+#include "pff_elem_fix.cuh"
 #include "pff_elem_pipe.cuh"
 
 namespace pff {
 
+// FP64: fixed-point contractions, every mode.  FP32 arithmetic and double-float:
+// the action only, FP32 in the persistent kernel where its slots fit.
 template <int P, int Q, typename T>
 cudaError_t launch_elem_pq(int mode, const ElemArgs<T>& a, cudaStream_t st) {
   constexpr int EB = elems_per_block(Q);
   int nblk = a.nblk > 0 ? a.nblk : (a.mesh.nel + EB - 1) / EB;
   if (nblk == 0) return cudaSuccess;
-  if constexpr (sizeof(T) == 4 && sizeof(typename ElemTypes<T>::L) == 4) {  // FP32 arithmetic: persistent kernel
-    if (a.lin16 && mode != kApply) return cudaErrorInvalidValue;
-    if (mode == kApply) {
+  if constexpr (sizeof(typename ElemTypes<T>::L) == 8) {
+    if (mode == kApply) return launch_elem_fix<P, Q, kApply>(a, nblk, st);
+    if (mode == kEval) return launch_elem_fix<P, Q, kEval>(a, nblk, st);
+    return launch_elem_fix<P, Q, kBack>(a, nblk, st);
+  } else {
+    if (mode != kApply) return cudaErrorInvalidValue;
+    if constexpr (sizeof(T) == 4) {
       cudaError_t err = cudaSuccess;
       if (launch_level_pipe<P, Q>(a, nblk, st, &err)) return err;
     }
+    const size_t smem = sizeof(T) * (size_t)(mat_smem_words<P, Q>() + EB * elem_smem_words_t<Q, T>());
+    auto k = k_elem<P, Q, T>;
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k<<<nblk, Q * Q * EB, smem, st>>>(a); note_launch();
+    return cudaGetLastError();
   }
-  size_t smem = sizeof(T) * (size_t)(mat_smem_words<P, Q>() + EB * elem_smem_words<Q>());
-  dim3 block(Q * Q * EB);
-  if (mode == kApply) smem = sizeof(T) * (size_t)(mat_smem_words<P, Q>() + EB * elem_smem_words_t<Q, T>());
-  if constexpr (sizeof(T) != sizeof(typename ElemTypes<T>::L)) {  // double-float: the action only
-    if (mode != kApply) return cudaErrorInvalidValue;
-    auto k = k_elem<P, Q, T, kApply>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<nblk, block, smem, st>>>(a); note_launch();
-  } else if (mode == kApply) {
-    auto k = k_elem<P, Q, T, kApply>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<nblk, block, smem, st>>>(a); note_launch();
-  } else if (mode == kEval) {
-    auto k = k_elem<P, Q, T, kEval>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<nblk, block, smem, st>>>(a); note_launch();
-  } else {
-    auto k = k_elem<P, Q, T, kBack>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<nblk, block, smem, st>>>(a); note_launch();
-  }
-  return cudaGetLastError();
 }
 
 template <int P, int Q, typename T>

@@ -33,7 +33,8 @@ struct Tables {  // per-level device copies of the 1D matrices, both precisions
   double *B64 = nullptr, *Dc64 = nullptr, *Dt64 = nullptr;
   float *B32 = nullptr, *Dc32 = nullptr, *Dt32 = nullptr;
   float hB32[pff::kMaxQ * pff::kMaxQ] = {}, hDc32[pff::kMaxQ * pff::kMaxQ] = {};  // host copies (kernel parameters)
-  double hB[pff::kMaxQ * pff::kMaxQ] = {}, hDt[pff::kMaxQ * pff::kMaxQ] = {}, hDc[pff::kMaxQ * pff::kMaxQ] = {};
+  double hB[pff::kMaxQ * pff::kMaxQ] = {}, hDt[pff::kMaxQ * pff::kMaxQ] = {};
+  pff::FixTab fix = {};  // the same for the FP64 kernels' fixed-point contractions
 };
 
 struct pff_op {

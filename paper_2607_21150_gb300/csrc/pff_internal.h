@@ -184,6 +184,17 @@ struct __align__(8) df64 {
 template <typename T> struct ElemTypes { using V = T; using L = T; using M = T; };
 template <> struct ElemTypes<df64> { using V = double; using L = float; using M = double; };
 
+// 1D matrices of the FP64 kernels' fixed-point contractions (pff_elem_fix.cuh):
+// B [Q][P] in units of 2^-60 and Dc [Q][Q] in units of 2^-sD, each entry in two
+// halves h 2^30 + l.  wf: bits kept below the largest entry of a field in an
+// element; wb: bits below 2^eD times the largest output, the power of two below
+// the bound of the transposed derivative sums; such that no stage's input passes 2^61.
+struct FixTab {
+  int Bh[kMaxQ * kMaxQ], Bl[kMaxQ * kMaxQ], Dh[kMaxQ * kMaxQ], Dl[kMaxQ * kMaxQ];
+  int sD, wf, wb, eD;
+};
+FixTab fix_table(int P, int Q, const double* B, const double* Dc);  // pff_basis.cpp
+
 template <typename T>
 struct ElemArgs {
   using V = typename ElemTypes<T>::V;
@@ -217,6 +228,7 @@ struct ElemArgs {
   // parameters, read as constant-bank operands where the index is fixed at compile time
   float cB[kMaxQ * kMaxQ];
   float cDc[kMaxQ * kMaxQ];
+  FixTab fix;             // FP64 kernels
 };
 
 // One translation unit per quadrature size Q (pff_elem_q<Q>.cu); each covers

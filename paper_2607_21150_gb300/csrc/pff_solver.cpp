@@ -1018,6 +1018,7 @@ ElemArgs<double> fine_args(pff_op* op) {
   a.B = op->tab.B64;
   a.Dc = op->tab.Dc64;
   a.Dt = op->tab.Dt64;
+  a.fix = op->tab.fix;
   a.lin = op->lin64;
   a.nq = op->nq;
   a.geo = op->geo;
