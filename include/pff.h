@@ -65,11 +65,10 @@ extern "C" {
 #define PFF_STATUS_RETURN 16     /* hardening return map: local Newton hit its cap (50) */
 #define PFF_STATUS_PIPE 32       /* FP32-arithmetic level action (PFF_F32 or PFF_F32_BF16 words): a wait for staged words gave up (result invalid) */
 
-/* PFF_DF64: FP64 vectors, the Jacobian action's contractions carried in
- * double-float arithmetic (pairs of FP32 words on the FP32 pipes, error about
- * 2^-47 of the magnitudes per operation instead of 2^-53) and the stored
- * linearisation read from its hi/lo FP32 planes (pff_op_enable_df).  Accepted
- * by pff_jacobian_apply and pff_jacobian_transpose_apply only.
+/* PFF_DF64: FP64 vectors, an accuracy of at least double-float (about 2^-47 of the
+ * magnitudes per operation) asked for; served by the FP64 action, which takes less
+ * time than pairs of floats did.  Needs pff_op_enable_df; accepted by
+ * pff_jacobian_apply, pff_jacobian_transpose_apply and pff_jacobian_apply_host only.
  * PFF_F32_BF16: FP32 vectors and arithmetic, the stored linearisation read as
  * BF16 words (8 significant bits, relative rounding error <= 2^-9 per word;
  * pff_op_enable_bf16): the p-multigrid level precision that halves the word
@@ -154,13 +153,10 @@ int pff_destroy_restriction(pff_restr* restr);
 int pff_create_operator(pff_ctx* ctx, pff_basis* fine, pff_restr* restr, pff_op** op);
 int pff_destroy_operator(pff_op* op);
 /* Also keep an FP32 copy of the stored linearisation (written by pff_residual),
- * needed by PFF_F32 applies.  Disabling frees it (and the PFF_DF64 planes). */
+ * needed by PFF_F32 applies.  Disabling frees it and ends PFF_DF64 too. */
 int pff_op_enable_f32(pff_op* op, int enable);
-/* Keep the stored linearisation also as two FP32 planes hi = fl32(w),
- * lo = fl32(w - hi) (written by pff_residual; 8 more bytes per word than FP64
- * alone), needed by PFF_DF64 applies.  The hi plane doubles as the FP32 copy,
- * so enabling also enables FP32.  Disabling stops the lo updates and keeps the
- * memory until pff_op_enable_f32(op, 0). */
+/* Allow PFF_DF64 applies.  Enabling also enables FP32 (pff_op_enable_f32);
+ * pff_op_enable_f32(op, 0) disables both. */
 int pff_op_enable_df(pff_op* op, int enable);
 /* Keep the stored linearisation also as BF16 words (72 per point, 144 bytes;
  * written by pff_residual, round to nearest even from FP64), needed by

@@ -1,12 +1,10 @@
-// Double-float arithmetic for the element kernels.  A value is the unevaluated
-// sum hi + lo of two floats; products and sums are formed with error-free FP32
-// transformations: Knuth's two-sum (s + e = a + b exactly) and the FMA-based
-// exact product (p + e = a * b exactly, e = fma(a, b, -p)).  On GB300 the FP32
-// pipes are 61 times wider than the FP64 pipe, so a contraction carried this
-// way can outrun FP64 although it takes about a dozen FP32 instructions per
-// multiply-add (the Q4 Jacobian action: 8.94 ms against 20.1 ms at 64^3), at
-// an error of about 2^-47 of the magnitudes involved per operation (FP64:
-// 2^-53).
+// Double-float arithmetic for the tangent of the pointwise update.  A value is the
+// unevaluated sum hi + lo of two floats; products and sums are formed with
+// error-free FP32 transformations: Knuth's two-sum (s + e = a + b exactly) and the
+// FMA-based exact product (p + e = a * b exactly, e = fma(a, b, -p)).  On GB300 the
+// FP32 pipes are 61 times wider than the FP64 pipe, so products carried this way
+// outrun FP64 although they take about a dozen FP32 instructions per multiply-add,
+// at an error of about 2^-47 of the magnitudes involved per operation.
 //
 // Accumulators stay unnormalised inside a contraction (|lo| may grow to a few
 // ulps of hi); two-sum is exact for any pair of floats, so only the final
@@ -87,34 +85,6 @@ __device__ __forceinline__ df64 df_split(double x) {
     const unsigned two_k = (unsigned)el << 23;
     l = __fsub_rn(__uint_as_float(two_k | ((lw >> 6) & 0x7fffffu)), __uint_as_float(two_k));
     if (sgn) l = -l;
-  }
-  return df_make(h, l);
-}
-// The same with hi = x rounded to the nearest float (ties to even), as the
-// FP32 planes of the stored words need: lo carries |x - hi| <= ulp(hi) / 2 to
-// 23 bits (|x - hi - lo| < 2^-46 |x|).  Zero and FP64 subnormals give zero;
-// |x| < 2^-126 and |x| >= 2^128 go through the conversion instructions.
-__device__ __forceinline__ df64 df_split_rn(double x) {
-  const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
-  const unsigned sgn = hw & 0x80000000u;
-  const int e = (int)((hw >> 20) & 0x7ffu);
-  if (e == 0) return df_make(0.0f, 0.0f);
-  const int ef = e - 896;
-  if (ef <= 0 || ef >= 254) {
-    const float h = __double2float_rn(x);
-    return df_make(h, __double2float_rn(x - (double)h));
-  }
-  const unsigned m23 = ((hw & 0xfffffu) << 3) | (lw >> 29);
-  const unsigned rem = lw & 0x1fffffffu;  // the 29 bits below hi's significand
-  const unsigned inc = (rem > 0x10000000u || (rem == 0x10000000u && (m23 & 1u))) ? 1u : 0u;
-  const float h = __uint_as_float((sgn | ((unsigned)ef << 23) | m23) + inc);  // a carry moves into the exponent
-  const unsigned m = inc ? 0x20000000u - rem : rem;  // |x - hi| in units of 2^(e - 1075)
-  const int el = e - 919;
-  float l = 0.0f;
-  if (el > 0) {
-    const unsigned two_k = (unsigned)el << 23;
-    l = __fsub_rn(__uint_as_float(two_k | ((m >> 6) & 0x7fffffu)), __uint_as_float(two_k));
-    if ((sgn != 0u) != (inc != 0u)) l = -l;
   }
   return df_make(h, l);
 }

@@ -12,9 +12,8 @@
 // the FP32 planes group words 0..63 of a point by four (lin32_word), so that
 // one 128-bit load fetches four words.
 //
-// The arithmetic type T is double, float or df64 (double-float pairs on the
-// FP32 pipes, FP64 vectors in and out); every multiply-add goes through
-// madd/mul/add so that one source serves all three.
+// The action in FP32 arithmetic is here and in pff_elem_pipe.cuh, every FP64
+// kernel in pff_elem_fix.cuh.
 #pragma once
 #include "pff_df.cuh"
 #include "pff_internal.h"
@@ -22,59 +21,11 @@
 namespace pff {
 
 template <typename T> __device__ __forceinline__ T ldg(const T* p) { return __ldg(p); }
-// Loads of the stored linearisation: the read-only path for the FP64 and FP32
-// actions, streaming loads (evict-first) for the two planes of the
-// double-float action (64^3 Q4: 16.0 -> 10.3 ms; the FP32 action measured
-// 2.9 ms with the read-only path, 3.0 ms with streaming loads).
-template <bool STREAM> __device__ __forceinline__ float ld_lin1(const float* p) { return STREAM ? __ldcs(p) : __ldg(p); }
-template <bool STREAM> __device__ __forceinline__ float4 ld_lin4(const float* p) {
-  return STREAM ? __ldcs(reinterpret_cast<const float4*>(p)) : __ldg(reinterpret_cast<const float4*>(p));
-}
+// four consecutive words of the FP32 quad layout; p is 16-byte aligned
+__device__ __forceinline__ float4 ld_quad(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
 
 __device__ __forceinline__ double madd(double c, double a, double b) { return fma(a, b, c); }
 __device__ __forceinline__ float madd(float c, float a, float b) { return fmaf(a, b, c); }
-__device__ __forceinline__ df64 madd(df64 c, df64 a, df64 b) { return df_madd(c, a, b); }
-__device__ __forceinline__ double mul(double a, double b) { return a * b; }
-__device__ __forceinline__ float mul(float a, float b) { return a * b; }
-__device__ __forceinline__ df64 mul(df64 a, df64 b) { return df_mul(a, b); }
-__device__ __forceinline__ double add(double a, double b) { return a + b; }
-__device__ __forceinline__ float add(float a, float b) { return a + b; }
-__device__ __forceinline__ df64 add(df64 a, df64 b) { return df_add(a, b); }
-
-template <typename T> __device__ __forceinline__ T zero() { return T(0); }
-template <> __device__ __forceinline__ df64 zero<df64>() { return df_make(0.0f, 0.0f); }
-// storage value (vector entry or basis matrix) -> arithmetic type; FP64 ->
-// double-float by integer operations (the conversion instructions run at the
-// FP64 rate on GB300)
-template <typename T, typename S> __device__ __forceinline__ T from_store(S x) { return (T)x; }
-template <> __device__ __forceinline__ df64 from_store<df64, double>(double x) { return df_split(x); }
-// arithmetic type -> vector entry
-__device__ __forceinline__ double to_vec(double v) { return v; }
-__device__ __forceinline__ float to_vec(float v) { return v; }
-__device__ __forceinline__ double to_vec(df64 v) { return df_join(v); }
-// stored linearisation word (df64: hi plane at p, lo plane at p + lo)
-template <typename T>
-__device__ __forceinline__ T ld_lin(const typename ElemTypes<T>::L* p, long long lo) {
-  if constexpr (sizeof(T) == sizeof(typename ElemTypes<T>::L)) {
-    return ldg(p);
-  } else {
-    return df_make(ld_lin1<true>(p), ld_lin1<true>(p + lo));
-  }
-}
-
-// four consecutive words of the FP32 quad layout (df64: hi plane at p, lo
-// plane at p + lo); p is 16-byte aligned
-template <typename T>
-__device__ __forceinline__ void ld_quad(const float* p, long long lo, T w[4]) {
-  if constexpr (sizeof(T) == 4) {
-    const float4 h = ld_lin4<false>(p);
-    w[0] = h.x; w[1] = h.y; w[2] = h.z; w[3] = h.w;
-  } else {
-    const float4 h = ld_lin4<true>(p);
-    const float4 l = ld_lin4<true>(p + lo);
-    w[0] = df_make(h.x, l.x); w[1] = df_make(h.y, l.y); w[2] = df_make(h.z, l.z); w[3] = df_make(h.w, l.w);
-  }
-}
 
 template <int P, int Q>
 __device__ __forceinline__ long long node_of(const MeshDev& m, int e, int a, int b, int c) {
@@ -86,25 +37,17 @@ __device__ __forceinline__ long long node_of(const MeshDev& m, int e, int a, int
   return (long long)(m.p * ex + a) + (long long)m.nnx * ((long long)(m.p * ey + b) + (long long)m.nny * (m.p * ez + c));
 }
 
-// Shared-memory layout per element: two ping-pong buffers of 4 fields x Q^3
-// values and a slice buffer of 8 x Q^2 values (x- and y-derivative outputs of
-// the four fields at one k).  The FP32 action ("split" form) instead keeps the
-// x- and y-derivative outputs of all Q slices, 8 x Q^3 values starting at the
-// second buffer, so that its pointwise stage runs without barriers.
-template <int Q> __host__ __device__ constexpr int elem_smem_words() { return 8 * Q * Q * Q + 8 * Q * Q; }
-template <typename T> __host__ __device__ constexpr bool elem_split() { return sizeof(T) == 4; }
-template <int Q, typename T> __host__ __device__ constexpr int elem_smem_words_t() {
-  return elem_split<T>() ? 12 * Q * Q * Q : elem_smem_words<Q>();
-}
+// Shared-memory layout per element of k_elem: the values at the Gauss points
+// (4 Q^3), then a ping-pong buffer that extends to the x- and y-derivative outputs
+// of all slices (8 Q^3), so that the pointwise stage runs without barriers.
+template <int Q> __host__ __device__ constexpr int elem_smem_words() { return 12 * Q * Q * Q; }
 
 template <int P, int Q, typename T>
 struct ElemSmem {
   T* bufA;  // [4][Q^3]
   T* bufB;  // [4][Q^3]
-  T* slice; // [8][Q^2]
   const T* B;
   const T* Dc;
-  const T* Dt;
 };
 
 // Gather x into bufA [4][c][b][a] (masked entries zero).
@@ -125,12 +68,12 @@ __device__ __forceinline__ void gather(const ElemArgs<T>& a, T* bufA, int e, boo
     long long n = valid ? node_of<P, Q>(a.mesh, e, aa, bb, cc) : 0;
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-      T v = zero<T>();
+      T v = T(0);
       if (valid) {
         long long g = f * nn + n;
         const auto xv = ldg(a.x + g);
         const bool fixed = masked && ldg(a.mask + g);
-        if (!fixed) v = from_store<T>(xv);
+        if (!fixed) v = (T)(xv);
       }
       bufA[f * Q3 + idx] = v;
     }
@@ -149,7 +92,7 @@ __device__ __forceinline__ void forward(const ElemArgs<T>& a, const ElemSmem<P, 
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
       const T* in = s.bufA + f * Q3 + r * P;
-      T acc = zero<T>();
+      T acc = T(0);
 #pragma unroll
       for (int k = 0; k < P; ++k) acc = madd(acc, s.B[i * P + k], in[k]);
       s.bufB[f * Q3 + idx] = acc;
@@ -162,7 +105,7 @@ __device__ __forceinline__ void forward(const ElemArgs<T>& a, const ElemSmem<P, 
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
       const T* in = s.bufB + f * Q3 + c * (P * Q) + i;
-      T acc = zero<T>();
+      T acc = T(0);
 #pragma unroll
       for (int k = 0; k < P; ++k) acc = madd(acc, s.B[j * P + k], in[k * Q]);
       s.bufA[f * Q3 + idx] = acc;
@@ -179,7 +122,7 @@ __device__ __forceinline__ void forward(const ElemArgs<T>& a, const ElemSmem<P, 
       for (int c = 0; c < P; ++c) col[c] = s.bufA[f * Q3 + c * Q2 + j * Q + i];
 #pragma unroll
       for (int k = 0; k < Q; ++k) {
-        T acc = zero<T>();
+        T acc = T(0);
 #pragma unroll
         for (int c = 0; c < P; ++c) acc = madd(acc, s.B[k * P + c], col[c]);
         s.bufB[f * Q3 + k * Q2 + j * Q + i] = acc;
@@ -218,7 +161,7 @@ __device__ __forceinline__ void fwd_lines(const ElemArgs<T>& a, T* bufA, T* bufB
     T* out = bufB + f * Q3 + cb * Q;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-      T acc = zero<T>();
+      T acc = T(0);
 #pragma unroll
       for (int aa = 0; aa < P; ++aa) acc = madd(acc, basis_b(a, i * P + aa), v[aa]);
       out[i] = acc;
@@ -237,7 +180,7 @@ __device__ __forceinline__ void fwd_lines(const ElemArgs<T>& a, T* bufA, T* bufB
     T* out = bufA + f * Q3 + c * Q2 + i;
 #pragma unroll
     for (int j = 0; j < Q; ++j) {
-      T acc = zero<T>();
+      T acc = T(0);
 #pragma unroll
       for (int b = 0; b < P; ++b) acc = madd(acc, basis_b(a, j * P + b), v[b]);
       out[j * Q] = acc;
@@ -251,7 +194,7 @@ __device__ __forceinline__ void fwd_lines(const ElemArgs<T>& a, T* bufA, T* bufB
     for (int c = 0; c < P; ++c) v[c] = bufA[f * Q3 + c * Q2 + ij];
 #pragma unroll
     for (int k = 0; k < Q; ++k) {
-      T acc = zero<T>();
+      T acc = T(0);
 #pragma unroll
       for (int c = 0; c < P; ++c) acc = madd(acc, basis_b(a, k * P + c), v[c]);
       bufB[f * Q3 + k * Q2 + ij] = acc;
@@ -273,7 +216,7 @@ __device__ __forceinline__ void bwd_lines(const ElemArgs<T>& a, T* bufA, T* bufB
   for (int f = 0; f < 4; ++f)
 #pragma unroll
     for (int c = 0; c < P; ++c) {
-      T acc = zero<T>();
+      T acc = T(0);
 #pragma unroll
       for (int k = 0; k < Q; ++k) acc = madd(acc, basis_b(a, k * P + c), Y[f][k]);
       bufA[f * Q3 + c * Q2 + ij] = acc;
@@ -291,7 +234,7 @@ __device__ __forceinline__ void bwd_lines(const ElemArgs<T>& a, T* bufA, T* bufB
     T* out = bufB + f * Q3 + c * (P * Q) + i;
 #pragma unroll
     for (int b = 0; b < P; ++b) {
-      T acc = zero<T>();
+      T acc = T(0);
 #pragma unroll
       for (int j = 0; j < Q; ++j) acc = madd(acc, basis_b(a, j * P + b), v[j]);
       out[b * Q] = acc;
@@ -310,7 +253,7 @@ __device__ __forceinline__ void bwd_lines(const ElemArgs<T>& a, T* bufA, T* bufB
     T* out = bufA + f * Q3 + cb * P;
 #pragma unroll
     for (int aa = 0; aa < P; ++aa) {
-      T acc = zero<T>();
+      T acc = T(0);
 #pragma unroll
       for (int i = 0; i < Q; ++i) acc = madd(acc, basis_b(a, i * P + aa), v[i]);
       out[aa] = acc;
@@ -319,11 +262,10 @@ __device__ __forceinline__ void bwd_lines(const ElemArgs<T>& a, T* bufA, T* bufB
   __syncthreads();
   if (!valid) return;
   if (a.evec) {  // deterministic transpose: element-local values, summed per node by k_node_gather
-    using V = typename ElemTypes<T>::V;
-    V* ev = static_cast<V*>(a.evec) + (long long)e * 4 * P3;
+    T* ev = static_cast<T*>(a.evec) + (long long)e * 4 * P3;
     for (int idx = ij; idx < P3; idx += Q2)
 #pragma unroll
-      for (int f = 0; f < 4; ++f) ev[f * P3 + idx] = to_vec(bufA[f * Q3 + idx]);
+      for (int f = 0; f < 4; ++f) ev[f * P3 + idx] = (bufA[f * Q3 + idx]);
     return;
   }
   const long long nn = a.mesh.nn;
@@ -338,7 +280,7 @@ __device__ __forceinline__ void bwd_lines(const ElemArgs<T>& a, T* bufA, T* bufB
     for (int f = 0; f < 4; ++f) {
       const long long g = f * nn + n;
       if (masked && __ldg(a.mask + g)) continue;
-      atomicAdd(a.y + g, to_vec(bufA[f * Q3 + idx]));
+      atomicAdd(a.y + g, (bufA[f * Q3 + idx]));
     }
   }
 }
@@ -350,7 +292,7 @@ __device__ __forceinline__ void grad_at(const ElemSmem<P, Q, T>& s, int i, int j
 #pragma unroll
   for (int f = 0; f < 4; ++f) {
     const T* V = s.bufB + f * Q3;
-    T gx = zero<T>(), gy = zero<T>(), gz = zero<T>();
+    T gx = T(0), gy = T(0), gz = T(0);
 #pragma unroll
     for (int m = 0; m < Q; ++m) {
       gx = madd(gx, s.Dc[i * Q + m], V[k * Q2 + j * Q + m]);
@@ -374,7 +316,7 @@ __device__ __forceinline__ void backward(const ElemArgs<T>& a, const ElemSmem<P,
   for (int f = 0; f < 4; ++f)
 #pragma unroll
     for (int c = 0; c < P; ++c) {
-      T acc = zero<T>();
+      T acc = T(0);
 #pragma unroll
       for (int k = 0; k < Q; ++k) acc = madd(acc, s.B[k * P + c], Y[f][k]);
       s.bufA[f * Q3 + c * Q2 + j * Q + i] = acc;
@@ -386,7 +328,7 @@ __device__ __forceinline__ void backward(const ElemArgs<T>& a, const ElemSmem<P,
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
       const T* in = s.bufA + f * Q3 + c * Q2 + ii;
-      T acc = zero<T>();
+      T acc = T(0);
 #pragma unroll
       for (int jj = 0; jj < Q; ++jj) acc = madd(acc, s.B[jj * P + bb], in[jj * Q]);
       s.bufB[f * Q3 + idx] = acc;
@@ -399,7 +341,7 @@ __device__ __forceinline__ void backward(const ElemArgs<T>& a, const ElemSmem<P,
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
       const T* in = s.bufB + f * Q3 + r * Q;
-      T acc = zero<T>();
+      T acc = T(0);
 #pragma unroll
       for (int ii = 0; ii < Q; ++ii) acc = madd(acc, s.B[ii * P + aa], in[ii]);
       s.bufA[f * Q3 + idx] = acc;
@@ -408,11 +350,10 @@ __device__ __forceinline__ void backward(const ElemArgs<T>& a, const ElemSmem<P,
   __syncthreads();
   if (!valid) return;
   if (a.evec) {  // deterministic transpose: element-local values, summed per node by k_node_gather
-    using V = typename ElemTypes<T>::V;
-    V* ev = static_cast<V*>(a.evec) + (long long)e * 4 * P3;
+    T* ev = static_cast<T*>(a.evec) + (long long)e * 4 * P3;
     for (int idx = ij; idx < P3; idx += Q2)
 #pragma unroll
-      for (int f = 0; f < 4; ++f) ev[f * P3 + idx] = to_vec(s.bufA[f * Q3 + idx]);
+      for (int f = 0; f < 4; ++f) ev[f * P3 + idx] = (s.bufA[f * Q3 + idx]);
     return;
   }
   const long long nn = a.mesh.nn;
@@ -427,86 +368,85 @@ __device__ __forceinline__ void backward(const ElemArgs<T>& a, const ElemSmem<P,
     for (int f = 0; f < 4; ++f) {
       long long g = f * nn + n;
       if (masked && ldg(a.mask + g)) continue;
-      atomicAdd(a.y + g, to_vec(s.bufA[f * Q3 + idx]));
+      atomicAdd(a.y + g, (s.bufA[f * Q3 + idx]));
     }
   }
 }
 
-// Pointwise linear map of the Jacobian with the stored words (already scaled
+// Pointwise linear map of the Jacobian with the stored FP64 words (already scaled
 // by the quadrature weight and the parent-to-reference factors).
-template <typename T>
-__device__ __forceinline__ void jac_point(const typename ElemTypes<T>::L* lin, const typename ElemTypes<T>::L* linP,
-                                          const typename ElemTypes<T>::L* linC, long long stride, long long lo,
-                                          int kx, const T g[4][3], T phi, T o[4][3], T& o0) {
-  T gu[9];
+__device__ __forceinline__ void jac_point(const double* lin, const double* linP, const double* linC, long long stride,
+                                          int kx, const double g[4][3], double phi, double o[4][3], double& o0) {
+  double gu[9];
 #pragma unroll
   for (int f = 0; f < 3; ++f)
 #pragma unroll
     for (int al = 0; al < 3; ++al) gu[3 * f + al] = g[f][al];
-  T ou[9];
+  double ou[9];
 #pragma unroll
-  for (int m = 0; m < 9; ++m) ou[m] = mul(ld_lin<T>(linP + m * stride, lo), phi);
+  for (int m = 0; m < 9; ++m) ou[m] = ldg(linP + m * stride) * phi;
   // symmetric 9x9 block
 #pragma unroll
   for (int m = 0; m < 9; ++m) {
 #pragma unroll
     for (int n = m; n < 9; ++n) {
-      T A = ld_lin<T>(lin + (long long)sym9(m, n) * stride, lo);
+      const double A = ldg(lin + (long long)sym9(m, n) * stride);
       ou[m] = madd(ou[m], A, gu[n]);
       if (n != m) ou[n] = madd(ou[n], A, gu[m]);
     }
   }
-  T s0 = mul(ld_lin<T>(lin + kWD * stride, lo), phi);
+  double s0 = ldg(lin + kWD * stride) * phi;
 #pragma unroll
-  for (int m = 0; m < 9; ++m) s0 = madd(s0, ld_lin<T>(linC + m * stride, lo), gu[m]);
+  for (int m = 0; m < 9; ++m) s0 = madd(s0, ldg(linC + m * stride), gu[m]);
   o0 = s0;
 #pragma unroll
   for (int f = 0; f < 3; ++f)
 #pragma unroll
     for (int al = 0; al < 3; ++al) o[f][al] = ou[3 * f + al];
 #pragma unroll
-  for (int al = 0; al < 3; ++al) o[3][al] = mul(ld_lin<T>(lin + (kWK + al) * stride, lo), g[3][al]);
+  for (int al = 0; al < 3; ++al) o[3][al] = ldg(lin + (kWK + al) * stride) * g[3][al];
   if (kx) {  // mapped mesh: symmetric off-diagonal coefficients 01, 02, 12
-    const T k01 = ld_lin<T>(lin + (kWKX + 0) * stride, lo);
-    const T k02 = ld_lin<T>(lin + (kWKX + 1) * stride, lo);
-    const T k12 = ld_lin<T>(lin + (kWKX + 2) * stride, lo);
+    const double k01 = ldg(lin + (kWKX + 0) * stride);
+    const double k02 = ldg(lin + (kWKX + 1) * stride);
+    const double k12 = ldg(lin + (kWKX + 2) * stride);
     o[3][0] = madd(madd(o[3][0], k01, g[3][1]), k02, g[3][2]);
     o[3][1] = madd(madd(o[3][1], k01, g[3][0]), k12, g[3][2]);
     o[3][2] = madd(madd(o[3][2], k02, g[3][0]), k12, g[3][1]);
   }
 }
 
-// The same map reading the FP32 planes in the quad layout: q = the point's
-// first quad (quads at stride qs), tl = its word 64 (tail words at stride ts).
-// Every quad is used as it arrives, in word order: the 9x9 block, dP/dphi and
+// The same map reading the FP32 plane in the quad layout: q = the point's first
+// quad (quads at stride qs), tl = its word 64 (tail words at stride ts).  Every
+// quad is used as it arrives, in word order: the 9x9 block, dP/dphi and
 // d(s_phi L)/dF (their roles swapped for the transpose, TR), d(s_phi L)/dphi.
-template <typename T, bool TR>
-__device__ __forceinline__ void jac_point_q(const float* q, long long qs, const float* tl, long long ts, long long lo,
-                                            int kx, const T g[4][3], T phi, T o[4][3], T& o0) {
-  T gu[9];
+template <bool TR>
+__device__ __forceinline__ void jac_point_q(const float* q, long long qs, const float* tl, long long ts, int kx,
+                                            const float g[4][3], float phi, float o[4][3], float& o0) {
+  float gu[9];
 #pragma unroll
   for (int f = 0; f < 3; ++f)
 #pragma unroll
     for (int al = 0; al < 3; ++al) gu[3 * f + al] = g[f][al];
-  T ou[9], s0 = zero<T>();
+  float ou[9], s0 = 0.0f;
 #pragma unroll
-  for (int m = 0; m < 9; ++m) ou[m] = zero<T>();
-  T cur[4];
+  for (int m = 0; m < 9; ++m) ou[m] = 0.0f;
+  float4 quad;
+  auto word = [&](int wd) {
+    if ((wd & 3) == 0) quad = ld_quad(q + (wd >> 2) * qs);
+    return (wd & 3) == 0 ? quad.x : (wd & 3) == 1 ? quad.y : (wd & 3) == 2 ? quad.z : quad.w;
+  };
 #pragma unroll
   for (int m = 0; m < 9; ++m) {  // upper triangle of the symmetric 9x9 block, row-major
 #pragma unroll
     for (int n = m; n < 9; ++n) {
-      const int wd = sym9(m, n);
-      if ((wd & 3) == 0) ld_quad<T>(q + (wd >> 2) * qs, lo, cur);
-      const T w = cur[wd & 3];
+      const float w = word(sym9(m, n));
       ou[m] = madd(ou[m], w, gu[n]);
       if (n != m) ou[n] = madd(ou[n], w, gu[m]);
     }
   }
 #pragma unroll
   for (int wd = kWP; wd < kLinQuadWords; ++wd) {  // the quad of word 44 is loaded
-    if ((wd & 3) == 0) ld_quad<T>(q + (wd >> 2) * qs, lo, cur);
-    const T w = cur[wd & 3];
+    const float w = word(wd);
     if (wd < kWC) {
       if (TR) s0 = madd(s0, w, gu[wd - kWP]);
       else ou[wd - kWP] = madd(ou[wd - kWP], w, phi);
@@ -523,32 +463,12 @@ __device__ __forceinline__ void jac_point_q(const float* q, long long qs, const 
 #pragma unroll
     for (int al = 0; al < 3; ++al) o[f][al] = ou[3 * f + al];
 #pragma unroll
-  for (int al = 0; al < 3; ++al) o[3][al] = mul(ld_lin<T>(tl + al * ts, lo), g[3][al]);
+  for (int al = 0; al < 3; ++al) o[3][al] = ldg(tl + al * ts) * g[3][al];
   if (kx) {  // mapped mesh: symmetric off-diagonal coefficients 01, 02, 12
-    const T k01 = ld_lin<T>(tl + 3 * ts, lo);
-    const T k02 = ld_lin<T>(tl + 4 * ts, lo);
-    const T k12 = ld_lin<T>(tl + 5 * ts, lo);
+    const float k01 = ldg(tl + 3 * ts), k02 = ldg(tl + 4 * ts), k12 = ldg(tl + 5 * ts);
     o[3][0] = madd(madd(o[3][0], k01, g[3][1]), k02, g[3][2]);
     o[3][1] = madd(madd(o[3][1], k01, g[3][0]), k12, g[3][2]);
     o[3][2] = madd(madd(o[3][2], k02, g[3][0]), k12, g[3][1]);
-  }
-}
-
-// Jacobian map at point (slice k, thread t) of this block: FP64 planar words
-// or the FP32 quad layout.
-template <int Q, typename T>
-__device__ __forceinline__ void jac_at(const ElemArgs<T>& a, int k, int t, const T g[4][3], T phi, T o[4][3], T& o0) {
-  constexpr long long EB = elems_per_block(Q);
-  constexpr long long run = (long long)Q * Q * EB, stride = run * Q;
-  const long long blk = (a.blk0 + blockIdx.x) * (long long)kLinWords * stride;
-  if constexpr (sizeof(typename ElemTypes<T>::L) == 4) {
-    const float* q = a.lin + blk + lin32_word(0, k, t, stride, run);
-    const float* tl = a.lin + blk + lin32_word(kLinQuadWords, k, t, stride, run);
-    if (a.transpose) jac_point_q<T, true>(q, 4 * stride, tl, stride, a.lo, a.kx, g, phi, o, o0);
-    else jac_point_q<T, false>(q, 4 * stride, tl, stride, a.lo, a.kx, g, phi, o, o0);
-  } else {
-    const long long off = blk + (long long)k * run + t;
-    jac_point<T>(a.lin + off, a.linP + off, a.linC + off, stride, a.lo, a.kx, g, phi, o, o0);
   }
 }
 
@@ -557,10 +477,8 @@ __device__ __forceinline__ void jac_at(const ElemArgs<T>& a, int k, int t, const
 // the next three (six on mapped meshes) the run of one tail word (Q^2 EB words),
 // each with one bulk prefetch, so the next slice streams from HBM while this
 // one computes (64^3 Q4: 3.76 -> 3.48 ms; two or three slices ahead measured
-// slower).  The double-float action does not prefetch: with the same requests
-// for both of its planes it took 14.2 ms instead of 10.4 ms.  Tail runs
-// start on 8-byte boundaries; the request is widened to 16-byte boundaries and
-// clipped to the plane.
+// slower).  Tail runs start on 8-byte boundaries; the request is widened to
+// 16-byte boundaries and clipped to the plane.
 constexpr int kPrefetchAhead = 1;  // slices requested ahead of the one computed
 __device__ __forceinline__ void prefetch_run(uintptr_t base, long long first, long long run, long long plane) {
   const uintptr_t lo = (base + 4 * first) & ~uintptr_t(15);
@@ -572,166 +490,98 @@ __device__ __forceinline__ void prefetch_run(uintptr_t base, long long first, lo
       "{\n\t.reg .u64 ga;\n\tcvta.to.global.u64 ga, %0;\n\tcp.async.bulk.prefetch.L2.global [ga], %1;\n\t}"
       :: "l"(lo), "r"((unsigned)(hi - lo)) : "memory");
 }
-template <int Q, typename T>
-__device__ __forceinline__ void prefetch_slice(const ElemArgs<T>& a, int k, int t) {
-  if constexpr (sizeof(T) == 4) {
-    constexpr int EB = elems_per_block(Q);
-    constexpr long long run = (long long)Q * Q * EB;   // words of one (word, slice) run
-    constexpr int NQ = kLinQuadWords / 4;
-    if (t >= NQ + (a.kx ? kLinWords - kLinQuadWords : kWKX - kLinQuadWords) || k >= Q) return;
-    const long long nblk = (a.mesh.nel + EB - 1) / EB;
-    const long long plane = nblk * kLinWords * Q * Q * Q * EB;
-    const long long blk = (a.blk0 + blockIdx.x) * kLinWords * Q * run;
-    const uintptr_t base = reinterpret_cast<uintptr_t>(a.lin);
-    if (t < NQ) prefetch_run(base, blk + lin32_word(4 * t, k, 0, Q * run, run), 4 * run, plane);
-    else prefetch_run(base, blk + lin32_word(kLinQuadWords + t - NQ, k, 0, Q * run, run), run, plane);
-  }
+template <int Q>
+__device__ __forceinline__ void prefetch_slice(const ElemArgs<float>& a, int k, int t) {
+  constexpr int EB = elems_per_block(Q);
+  constexpr long long run = (long long)Q * Q * EB;   // words of one (word, slice) run
+  constexpr int NQ = kLinQuadWords / 4;
+  if (t >= NQ + (a.kx ? kLinWords - kLinQuadWords : kWKX - kLinQuadWords) || k >= Q) return;
+  const long long nblk = (a.mesh.nel + EB - 1) / EB;
+  const long long plane = nblk * kLinWords * Q * Q * Q * EB;
+  const long long blk = (a.blk0 + blockIdx.x) * kLinWords * Q * run;
+  const uintptr_t base = reinterpret_cast<uintptr_t>(a.lin);
+  if (t < NQ) prefetch_run(base, blk + lin32_word(4 * t, k, 0, Q * run, run), 4 * run, plane);
+  else prefetch_run(base, blk + lin32_word(kLinQuadWords + t - NQ, k, 0, Q * run, run), run, plane);
 }
 
-// Entry k of a thread's column accumulators when k is not a compile-time
-// constant: selects over the unrolled entries, so the column stays in
-// registers.
-template <int Q, typename T>
-__device__ __forceinline__ T column_at(const T (&y)[Q], int k) {
-  T v = y[0];
-#pragma unroll
-  for (int kk = 1; kk < Q; ++kk)
-    if (kk == k) v = y[kk];
-  return v;
-}
-template <int Q, typename T>
-__device__ __forceinline__ void set_column_at(T (&y)[Q], int k, T v) {
-#pragma unroll
-  for (int kk = 0; kk < Q; ++kk)
-    if (kk == k) y[kk] = v;
-}
-
-// Resident blocks per SM the register allocation is held to (Q = 5: 250
-// threads per block, 97 KB of shared memory at 8-byte words): two for FP64 and
-// double-float (<= 128 registers), three for FP32 (<= 85 registers).  With a
-// single resident block the barriers of the slice loop leave the SM idle.
-template <typename T> constexpr int elem_min_blocks() { return sizeof(T) == 4 ? 3 : 2; }
-
-template <int P, int Q, typename T>
-__global__ void __launch_bounds__(Q * Q * elems_per_block(Q), elem_min_blocks<T>())
-k_elem(const ElemArgs<T> a) {
+// FP32-word action without the persistent kernel's shared-memory ring (mapped
+// meshes at Q = 5, whose two slots leave no room for a second block): three
+// resident blocks per SM (<= 85 registers), no barriers in the pointwise stage.
+template <int P, int Q>
+__global__ void __launch_bounds__(Q * Q * elems_per_block(Q), 3)
+k_elem(const ElemArgs<float> a) {
   constexpr int EB = elems_per_block(Q);
   constexpr int Q2 = Q * Q, Q3 = Q * Q * Q;
+  constexpr long long run = (long long)Q2 * EB, stride = run * Q;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* sm = reinterpret_cast<T*>(smem_raw);
+  float* sm = reinterpret_cast<float*>(smem_raw);
   const int t = threadIdx.x;
   const int el = t / Q2, ij = t % Q2;
   const int i = ij % Q, j = ij / Q;
   const int e = (a.blk0 + blockIdx.x) * EB + el;
   const bool valid = e < a.mesh.nel;
 
-  T* mats = sm;
-  T* Bs = mats;
-  T* Dcs = Bs + Q * P;
-  for (int idx = t; idx < Q * P; idx += blockDim.x) Bs[idx] = from_store<T>(a.B[idx]);
-  for (int idx = t; idx < Q * Q; idx += blockDim.x) Dcs[idx] = from_store<T>(a.Dc[idx]);
-  constexpr bool kSplit = elem_split<T>();
-  T* base = sm + mat_smem_words<P, Q>() + el * elem_smem_words_t<Q, T>();
-  // split form: bufB first (read by every slice's gradients), then bufA which
-  // extends to the 8 x Q^3 derivative outputs of the pointwise stage
-  ElemSmem<P, Q, T> s = kSplit ? ElemSmem<P, Q, T>{base + 4 * Q3, base, nullptr, Bs, Dcs, nullptr}
-                               : ElemSmem<P, Q, T>{base, base + 4 * Q3, base + 8 * Q3, Bs, Dcs, nullptr};
+  float* Bs = sm;
+  float* Dcs = Bs + Q * P;
+  for (int idx = t; idx < Q * P; idx += blockDim.x) Bs[idx] = a.B[idx];
+  for (int idx = t; idx < Q * Q; idx += blockDim.x) Dcs[idx] = a.Dc[idx];
+  float* base = sm + mat_smem_words<P, Q>() + el * elem_smem_words<Q>();
+  // bufB first (read by every slice's gradients), then bufA which extends to the
+  // 8 x Q^3 derivative outputs of the pointwise stage
+  const ElemSmem<P, Q, float> s{base + 4 * Q3, base, Bs, Dcs};
   __syncthreads();
-  if constexpr (kSplit)
-    for (int k = 0; k < kPrefetchAhead; ++k) prefetch_slice<Q, T>(a, k, t);
+  for (int k = 0; k < kPrefetchAhead; ++k) prefetch_slice<Q>(a, k, t);
+  forward<P, Q, float>(a, s, e, valid, ij);
 
-  forward<P, Q, T>(a, s, e, valid, ij);
-
-  T Y[4][Q];
+  float Y[4][Q];
 #pragma unroll
   for (int f = 0; f < 4; ++f)
 #pragma unroll
-    for (int k = 0; k < Q; ++k) Y[f][k] = zero<T>();
-
-  if constexpr (kSplit) {
-    // pointwise stage of all slices without barriers: z-derivative and value
-    // terms into the registers of the own column, x- and y-derivative outputs
-    // to shared memory
-    T* oxy = s.bufA;  // [8][Q^3]
+    for (int k = 0; k < Q; ++k) Y[f][k] = 0.0f;
+  // pointwise stage of all slices: z-derivative and value terms into the
+  // registers of the own column, x- and y-derivative outputs to shared memory
+  const float* blk = a.lin + (a.blk0 + blockIdx.x) * (long long)kLinWords * stride;
+  float* oxy = s.bufA;  // [8][Q^3]
 #pragma unroll
-    for (int k = 0; k < Q; ++k) {
-      T g[4][3], phi, o[4][3], o0 = zero<T>();
-      prefetch_slice<Q, T>(a, k + kPrefetchAhead, t);
-      grad_at<P, Q, T>(s, i, j, k, g, phi);
-      if (valid) {
-        jac_at<Q, T>(a, k, t, g, phi, o, o0);
-      } else {
-#pragma unroll
-        for (int f = 0; f < 4; ++f) o[f][0] = o[f][1] = o[f][2] = zero<T>();
-      }
-#pragma unroll
-      for (int f = 0; f < 4; ++f) {
-#pragma unroll
-        for (int kk = 0; kk < Q; ++kk) Y[f][kk] = madd(Y[f][kk], s.Dc[k * Q + kk], o[f][2]);
-        oxy[(2 * f) * Q3 + k * Q2 + ij] = o[f][0];
-        oxy[(2 * f + 1) * Q3 + k * Q2 + ij] = o[f][1];
-      }
-      Y[3][k] = add(Y[3][k], o0);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < Q; ++k)
-#pragma unroll
-      for (int f = 0; f < 4; ++f) {
-        const T* ox = oxy + (2 * f) * Q3 + k * Q2;
-        const T* oy = oxy + (2 * f + 1) * Q3 + k * Q2;
-        T acc = Y[f][k];
-#pragma unroll
-        for (int m = 0; m < Q; ++m) {
-          acc = madd(acc, s.Dc[m * Q + i], ox[j * Q + m]);
-          acc = madd(acc, s.Dc[m * Q + j], oy[m * Q + i]);
-        }
-        Y[f][k] = acc;
-      }
-    __syncthreads();  // the derivative outputs are read; backward reuses the buffers
-    backward<P, Q, T>(a, s, e, valid, ij, Y);
-    return;
-  }
-  // The slice loop stays rolled: the pointwise map takes about ten times the
-  // instructions of an FP64 one, and five unrolled slices, each with both
-  // orientations of the map, overflow the instruction cache.  Y[f][k] is then
-  // selected and written back by column_at / set_column_at.
-#pragma unroll 1
   for (int k = 0; k < Q; ++k) {
-    T g[4][3], phi, o[4][3], o0 = zero<T>();
-    grad_at<P, Q, T>(s, i, j, k, g, phi);
+    float g[4][3], phi, o[4][3], o0 = 0.0f;
+    prefetch_slice<Q>(a, k + kPrefetchAhead, t);
+    grad_at<P, Q, float>(s, i, j, k, g, phi);
     if (valid) {
-      jac_at<Q, T>(a, k, t, g, phi, o, o0);
+      const float* q = blk + lin32_word(0, k, t, stride, run);
+      const float* tl = blk + lin32_word(kLinQuadWords, k, t, stride, run);
+      if (a.transpose) jac_point_q<true>(q, 4 * stride, tl, stride, a.kx, g, phi, o, o0);
+      else jac_point_q<false>(q, 4 * stride, tl, stride, a.kx, g, phi, o, o0);
     } else {
 #pragma unroll
-      for (int f = 0; f < 4; ++f) o[f][0] = o[f][1] = o[f][2] = zero<T>();
+      for (int f = 0; f < 4; ++f) o[f][0] = o[f][1] = o[f][2] = 0.0f;
     }
-    // transposed z-derivative (own column) and the value term
 #pragma unroll
-    for (int f = 0; f < 4; ++f)
+    for (int f = 0; f < 4; ++f) {
 #pragma unroll
       for (int kk = 0; kk < Q; ++kk) Y[f][kk] = madd(Y[f][kk], s.Dc[k * Q + kk], o[f][2]);
-    // x- and y-derivative outputs of this slice through shared memory
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      s.slice[(2 * f) * Q2 + ij] = o[f][0];
-      s.slice[(2 * f + 1) * Q2 + ij] = o[f][1];
+      oxy[(2 * f) * Q3 + k * Q2 + ij] = o[f][0];
+      oxy[(2 * f + 1) * Q3 + k * Q2 + ij] = o[f][1];
     }
-    __syncthreads();
+    Y[3][k] += o0;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < Q; ++k)
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-      T acc = column_at<Q>(Y[f], k);
-      if (f == 3) acc = add(acc, o0);
+      const float* ox = oxy + (2 * f) * Q3 + k * Q2;
+      const float* oy = oxy + (2 * f + 1) * Q3 + k * Q2;
+      float acc = Y[f][k];
 #pragma unroll
       for (int m = 0; m < Q; ++m) {
-        acc = madd(acc, s.Dc[m * Q + i], s.slice[(2 * f) * Q2 + j * Q + m]);
-        acc = madd(acc, s.Dc[m * Q + j], s.slice[(2 * f + 1) * Q2 + m * Q + i]);
+        acc = madd(acc, s.Dc[m * Q + i], ox[j * Q + m]);
+        acc = madd(acc, s.Dc[m * Q + j], oy[m * Q + i]);
       }
-      set_column_at<Q>(Y[f], k, acc);
+      Y[f][k] = acc;
     }
-    __syncthreads();
-  }
-  backward<P, Q, T>(a, s, e, valid, ij, Y);
+  __syncthreads();  // the derivative outputs are read; backward reuses the buffers
+  backward<P, Q, float>(a, s, e, valid, ij, Y);
 }
 
 // Diagonal of the element operators: for each field f and node a,
@@ -771,8 +621,8 @@ __device__ __forceinline__ void diag_words(const ElemArgs<T>& a, int f, int t, b
         const int q0 = f == 0 ? 0 : f == 1 ? 6 : 9;   // quads of words (f0, f0 .. f2)
         const int q1 = f == 0 ? 2 : f == 1 ? 7 : 10;
         const int q2 = f == 0 ? 4 : f == 1 ? 8 : 11;
-        const float4 A = ld_lin4<false>(p + q0 * 4 * stride), B = ld_lin4<false>(p + q1 * 4 * stride),
-                     C = ld_lin4<false>(p + q2 * 4 * stride);
+        const float4 A = ld_quad(p + q0 * 4 * stride), B = ld_quad(p + q1 * 4 * stride),
+                     C = ld_quad(p + q2 * 4 * stride);
         if (f == 0) {         // words 0, 1, 2, 9, 10, 17
           w[0][k] = A.x; w[1][k] = A.y; w[2][k] = A.z; w[3][k] = B.y; w[4][k] = B.z; w[5][k] = C.y;
         } else if (f == 1) {  // words 24, 25, 26, 30, 31, 35
@@ -924,28 +774,29 @@ k_diag(const ElemArgs<T> a, const DiagMats<T, P, Q> mats) {
 
 namespace pff {
 
-// FP64: fixed-point contractions, every mode.  FP32 arithmetic and double-float:
-// the action only, FP32 in the persistent kernel where its slots fit.
+// FP64: fixed-point contractions, every mode.  FP32 arithmetic: the action only,
+// in the persistent kernel where its slots fit.
 template <int P, int Q, typename T>
 cudaError_t launch_elem_pq(int mode, const ElemArgs<T>& a, cudaStream_t st) {
   constexpr int EB = elems_per_block(Q);
   int nblk = a.nblk > 0 ? a.nblk : (a.mesh.nel + EB - 1) / EB;
   if (nblk == 0) return cudaSuccess;
-  if constexpr (sizeof(typename ElemTypes<T>::L) == 8) {
+  if constexpr (sizeof(T) == 8) {
     if (mode == kApply) return launch_elem_fix<P, Q, kApply>(a, nblk, st);
     if (mode == kEval) return launch_elem_fix<P, Q, kEval>(a, nblk, st);
     return launch_elem_fix<P, Q, kBack>(a, nblk, st);
   } else {
     if (mode != kApply) return cudaErrorInvalidValue;
-    if constexpr (sizeof(T) == 4) {
-      cudaError_t err = cudaSuccess;
-      if (launch_level_pipe<P, Q>(a, nblk, st, &err)) return err;
+    cudaError_t err = cudaSuccess;
+    if (launch_level_pipe<P, Q>(a, nblk, st, &err)) return err;
+    if constexpr (!pipe_fits<P, Q, false, true>()) {
+      const size_t smem = sizeof(float) * (size_t)(mat_smem_words<P, Q>() + EB * elem_smem_words<Q>());
+      auto k = k_elem<P, Q>;
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      k<<<nblk, Q * Q * EB, smem, st>>>(a); note_launch();
+      return cudaGetLastError();
     }
-    const size_t smem = sizeof(T) * (size_t)(mat_smem_words<P, Q>() + EB * elem_smem_words_t<Q, T>());
-    auto k = k_elem<P, Q, T>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<nblk, Q * Q * EB, smem, st>>>(a); note_launch();
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
   }
 }
 

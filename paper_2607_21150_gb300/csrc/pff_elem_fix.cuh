@@ -253,7 +253,7 @@ k_elem_fix(const ElemArgs<double> a) {
         if constexpr (MODE == kApply) {
           constexpr long long run = (long long)Q2 * EB, stride = run * Q;
           const long long off = grp * kLinWords * stride + (pt / Q2) * run + (sub * EBS + el) * Q2 + pt % Q2;
-          jac_point<double>(a.lin + off, a.linP + off, a.linC + off, stride, a.lo, a.kx, g, phi, o, v0);
+          jac_point(a.lin + off, a.linP + off, a.linC + off, stride, a.kx, g, phi, o, v0);
         } else {  // integrands from the pointwise kernel
 #pragma unroll
           for (int f = 0; f < 4; ++f)

@@ -383,7 +383,7 @@ k_level_pipe(const ElemArgs<float> a) {
   for (int idx = t; idx < Q * P; idx += blockDim.x) Bs[idx] = a.cB[idx];
   for (int idx = t; idx < Q * Q; idx += blockDim.x) Dcs[idx] = a.cDc[idx];
   float* base = sm + mat_smem_words<P, Q>() + el * pipe_elem_stride<Q>();
-  const ElemSmem<P, Q, float> s{base + 4 * Q3, base, nullptr, Bs, Dcs, nullptr};
+  const ElemSmem<P, Q, float> s{base + 4 * Q3, base, Bs, Dcs};
   float* sbuf = s.bufA;  // [2][8][Q^2] during the slice loop
   if (t == 0) {
     mbar_init(bar, 1);

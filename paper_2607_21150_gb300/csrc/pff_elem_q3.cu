@@ -1,4 +1,4 @@
-// Element kernels for Q = 3 Gauss points per direction, every P <= Q, FP64, FP32 and double-float (action only).
+// Element kernels for Q = 3 Gauss points per direction, every P <= Q in FP64 and FP32.
 #include "pff_elem.cuh"
 
 namespace pff {
@@ -21,7 +21,6 @@ cudaError_t launch_diag_q3(int P, const ElemArgs<T>& a, const double* B, const d
 }
 template cudaError_t launch_elem_q3<double>(int, int, const ElemArgs<double>&, cudaStream_t);
 template cudaError_t launch_elem_q3<float>(int, int, const ElemArgs<float>&, cudaStream_t);
-template cudaError_t launch_elem_q3<df64>(int, int, const ElemArgs<df64>&, cudaStream_t);
 template cudaError_t launch_diag_q3<double>(int, const ElemArgs<double>&, const double*, const double*, cudaStream_t);
 template cudaError_t launch_diag_q3<float>(int, const ElemArgs<float>&, const double*, const double*, cudaStream_t);
 

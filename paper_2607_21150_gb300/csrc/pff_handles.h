@@ -50,7 +50,7 @@ struct pff_op {
   uint8_t* phase = nullptr;
   uint8_t* flags = nullptr;
   double* lin64 = nullptr;
-  float* lin32 = nullptr;     // FP32 copy; with df = 1 the hi plane [0, lin_len) and lo plane [lin_len, 2 lin_len)
+  float* lin32 = nullptr;     // FP32 copy (lin32_word layout)
   long long lin_len = 0;
   double* io = nullptr;
   uint8_t* mask = nullptr;
@@ -58,8 +58,7 @@ struct pff_op {
   double* dvals = nullptr;
   int* status = nullptr;
   int f32 = 0;
-  int df = 0;                 // maintain the double-float planes of the stored linearisation
-  int lin32_planes = 0;       // FP32 planes allocated at lin32 (0, 1 or 2)
+  int df = 0;                 // PFF_DF64 actions allowed (pff_op_enable_df)
   int det = 0;                // deterministic transpose (pff_op_set_deterministic)
   void* evec = nullptr;       // its element values, [nel][4][P^3] doubles of the fine order
   uint16_t* lin16 = nullptr;  // BF16 words (lin16_word layout), written by pff_residual when bf16 = 1

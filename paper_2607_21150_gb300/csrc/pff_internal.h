@@ -15,7 +15,7 @@ constexpr int kLinWords = 70;     // stored pointwise linearisation words per qu
 // All words are in the parent frame (w_q det J and d xi / dX folded in).
 constexpr int kWA = 0, kWP = 45, kWC = 54, kWD = 63, kWK = 64, kWKX = 67;
 constexpr int kLinWordsExport = 67;  // words returned by pff_get_linearization
-// FP32 planes (level actions, double-float hi/lo): words [0, 64) interleaved by
+// FP32 plane (level actions): words [0, 64) interleaved by
 // four, so that one 128-bit load fetches four words of one point; words
 // [64, 70) as in the FP64 layout.  Offset of word w of slice k, thread t within
 // a block's region (q3eb = Q^3 EB words per word plane, q2eb = Q^2 EB per slice):
@@ -24,7 +24,7 @@ __host__ __device__ constexpr long long lin32_word(int w, int k, int t, long lon
   return w < kLinQuadWords ? (long long)(w >> 2) * 4 * q3eb + (long long)k * 4 * q2eb + 4LL * t + (w & 3)
                            : (long long)w * q3eb + (long long)k * q2eb + t;
 }
-// Floats allocated past the FP32 planes: the persistent level kernel copies
+// Floats allocated past the FP32 plane: the persistent level kernel copies
 // each tail-word run widened to 16-byte boundaries, up to 12 bytes past it.
 constexpr long long kLin32Pad = 16;
 
@@ -167,7 +167,7 @@ struct AdjArgs {
 };
 cudaError_t launch_adjoint_point(const AdjArgs& a, cudaStream_t st);
 
-// Element-kernel launches (pff_elem*.cu).  T = double, float or df64.
+// Element-kernel launches (pff_elem*.cu).  T = double or float.
 enum ElemMode { kApply = 0, kEval = 1, kBack = 2 };
 
 // Double-float value hi + lo (two FP32 words, about 48 significant bits); the
@@ -176,13 +176,6 @@ enum ElemMode { kApply = 0, kEval = 1, kBack = 2 };
 struct __align__(8) df64 {
   float hi, lo;
 };
-
-// Storage types of an element kernel computing in T: vectors V, stored
-// linearisation L, 1D basis matrices M.  The double-float kernel reads and
-// writes FP64 vectors, the stored linearisation as two FP32 planes (hi, then
-// lo at a fixed offset) and converts the FP64 basis matrices on entry.
-template <typename T> struct ElemTypes { using V = T; using L = T; using M = T; };
-template <> struct ElemTypes<df64> { using V = double; using L = float; using M = double; };
 
 // 1D matrices of the FP64 kernels' fixed-point contractions (pff_elem_fix.cuh):
 // B [Q][P] in units of 2^-60 and Dc [Q][Q] in units of 2^-sD, each entry in two
@@ -197,30 +190,26 @@ FixTab fix_table(int P, int Q, const double* B, const double* Dc);  // pff_basis
 
 template <typename T>
 struct ElemArgs {
-  using V = typename ElemTypes<T>::V;
-  using L = typename ElemTypes<T>::L;
-  using M = typename ElemTypes<T>::M;
   MeshDev mesh;
-  const V* x;             // [4][nn] input (apply) / unused
-  V* y;                   // [4][nn] output (scatter-add)
+  const T* x;             // [4][nn] input (apply) / unused
+  T* y;                   // [4][nn] output (scatter-add)
   const uint8_t* mask;    // [4][nn] Dirichlet mask or nullptr
-  const M* B;             // [Q][P] interpolation to Gauss points
-  const M* Dc;            // [Q][Q] collocated derivative at Gauss points
-  const M* Dt;            // [Q][P] derivative of the basis at Gauss points (diagonal)
-  const L* lin;           // tiled stored linearisation (apply / diagonal)
-  const L* linP;          // words multiplying dphi in the u rows (dP/dphi or, transposed, dL/dF)
-  const L* linC;          // words multiplying grad u in the phi row
+  const T* B;             // [Q][P] interpolation to Gauss points
+  const T* Dc;            // [Q][Q] collocated derivative at Gauss points
+  const T* Dt;            // [Q][P] derivative of the basis at Gauss points (diagonal)
+  const T* lin;           // tiled stored linearisation (apply / diagonal)
+  const T* linP;          // words multiplying dphi in the u rows (dP/dphi or, transposed, dL/dF)
+  const T* linC;          // words multiplying grad u in the phi row
   double* scratch;        // [13][nq] (eval / back)
   double s[3];            // d xi / d X (eval, box)
   const double* geo;      // mapped mesh (eval): [10][nq] d xi / dX per point; null = box
   long long nq;
   int transpose;
   int kx;                 // 1: add the off-diagonal phase-gradient words (mapped meshes)
-  long long lo;           // df64: offset (in words) from the hi plane to the lo plane
   const uint16_t* lin16;  // FP32 action only: read the BF16 words (lin16_word layout) instead of lin
   int* status;            // device status word (BF16-word action: bit 32 when a staging wait gave up)
   const uint8_t* emask;   // [nel] 1 = the element has masked nodes (null: check the mask everywhere)
-  void* evec;             // deterministic transpose: element values [nel][4][P^3] (type V) instead of atomics
+  void* evec;             // deterministic transpose: element values [nel][4][P^3] (type T) instead of atomics
   int blk0;               // first element block of the launch (actions; 0 = from the first)
   int ctas;               // FP32-arithmetic actions: resident blocks of the persistent kernel (0 = one per element block)
   int nblk;               // element blocks of the launch (actions; 0 = all blocks from blk0 = 0)
@@ -266,11 +255,9 @@ cudaError_t launch_elem_mask(const MeshDev& m, const uint8_t* mask, uint8_t* ema
 // y = mask ? x : 0 on nodes [n0, n1) of each field (prec 0: FP64, 1: FP32).
 cudaError_t launch_init_rows(int prec, void* y, const void* x, const uint8_t* mask, long long nn, long long n0,
                              long long n1, cudaStream_t st);
-// Level copies of the FP64 words a in one pass, each optional: FP32 planes hi
-// (round to nearest even) and lo = a - hi (lin32_word layout), BF16 words b16
-// (round to nearest even, lin16_word layout).
-cudaError_t launch_split_words(const double* a, float* hi, float* lo, uint16_t* b16, long long nblk, int Q,
-                               cudaStream_t st);
+// Level copies of the FP64 words a in one pass, each optional: FP32 plane
+// (lin32_word layout) and BF16 words (lin16_word layout), rounded to nearest even.
+cudaError_t launch_level_words(const double* a, float* w32, uint16_t* b16, long long nblk, int Q, cudaStream_t st);
 cudaError_t launch_apply_dirichlet(double* z, const double* ubar, const uint8_t* mask, long long n, cudaStream_t st);
 cudaError_t launch_masked_field_sums(const double* v, const uint8_t* sel, long long nn, double* out, cudaStream_t st);
 // out[8]: flag counts (yield, history active, theta >= 0), phi max / min, nodes

@@ -1,5 +1,5 @@
-// Vector kernels: Dirichlet initialisation, the FP32 (and double-float)
-// planes of the stored linearisation, the
+// Vector kernels: Dirichlet initialisation, the FP32 and BF16 copies of the
+// stored linearisation, the
 // Chebyshev smoother updates, the export of the linearisation, reaction sums
 // and the geometric factors of mapped meshes.
 #include <cuda_bf16.h>
@@ -161,19 +161,30 @@ __device__ __forceinline__ unsigned bf16_rne(double x) {
   return sgn | (top + inc);  // a carry moves into the exponent
 }
 
-// The level copies of the stored linearisation in one pass over the FP64
-// words: the FP32 planes (lin32_word layout; hi = fl32(a), round to nearest
-// even, and lo = a - hi to 23 bits, df_split_rn) and the BF16 words
-// (lin16_word layout; words 70 and 71 zero), each optional.  All conversions
-// are integer operations, so that the pass runs at HBM speed rather than at
-// the FP64 rate of the conversion instructions.  One thread per octet of a
-// point's words [0, 64) (eight coalesced FP64 reads; two 128-bit writes per
-// FP32 plane, one for the BF16 octet), then one per tail plane of four words.
-// Writing these copies from the pointwise kernel instead measured slower
-// (64^3 Q4 residual 154 -> 176 ms): its scattered narrow stores cost more than
-// this pass.
-__global__ void k_split_words(const double* __restrict__ a, float* __restrict__ hi, float* __restrict__ lo,
-                              uint16_t* __restrict__ b16, long long nblk, long long q3eb) {
+// FP32 word of x, round to nearest even, by integer operations (zero and FP64
+// subnormals give zero; |x| outside the normal FP32 range goes through the
+// conversion instruction).
+__device__ __forceinline__ float f32_rne(double x) {
+  const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
+  const int e = (int)((hw >> 20) & 0x7ffu), ef = e - 896;
+  if (e == 0) return 0.0f;
+  if (ef <= 0 || ef >= 254) return __double2float_rn(x);
+  const unsigned m23 = ((hw & 0xfffffu) << 3) | (lw >> 29), rem = lw & 0x1fffffffu;
+  const unsigned inc = (rem > 0x10000000u || (rem == 0x10000000u && (m23 & 1u))) ? 1u : 0u;
+  return __uint_as_float(((hw & 0x80000000u) | ((unsigned)ef << 23) | m23) + inc);  // a carry moves into the exponent
+}
+
+// The level copies of the stored linearisation in one pass over the FP64 words:
+// the FP32 plane (lin32_word layout) and the BF16 words (lin16_word layout;
+// words 70 and 71 zero), each optional.  All conversions are integer operations,
+// so that the pass runs at HBM speed rather than at the FP64 rate of the
+// conversion instructions.  One thread per octet of a point's words [0, 64)
+// (eight coalesced FP64 reads; two 128-bit writes for the plane, one for the BF16
+// octet), then one per tail plane of four words.  Writing these copies from the
+// pointwise kernel instead measured slower (64^3 Q4 residual 154 -> 176 ms): its
+// scattered narrow stores cost more than this pass.
+__global__ void k_level_words(const double* __restrict__ a, float* __restrict__ w32, uint16_t* __restrict__ b16,
+                              long long nblk, long long q3eb) {
   const long long bw = (long long)kLinWords * q3eb, ow = (long long)kLin16Words * q3eb;
   const long long opb = 8 * q3eb, tpb = 2 * q3eb;  // octet / tail units per block
   const long long no = nblk * opb, n = no + nblk * tpb;
@@ -185,20 +196,11 @@ __global__ void k_split_words(const double* __restrict__ a, float* __restrict__ 
       double x[8];
 #pragma unroll
       for (int c = 0; c < 8; ++c) x[c] = src[c * q3eb];
-      if (hi) {
-        float h[8], l[8];
+      if (w32) {
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const df64 v = df_split_rn(x[c]);
-          h[c] = v.hi;
-          l[c] = v.lo;
-        }
-#pragma unroll
-        for (int g = 0; g < 2; ++g) {
-          const long long o = b * bw + (2 * oc + g) * 4 * q3eb + 4 * r2;
-          *reinterpret_cast<float4*>(hi + o) = make_float4(h[4 * g], h[4 * g + 1], h[4 * g + 2], h[4 * g + 3]);
-          if (lo) *reinterpret_cast<float4*>(lo + o) = make_float4(l[4 * g], l[4 * g + 1], l[4 * g + 2], l[4 * g + 3]);
-        }
+        for (int g = 0; g < 2; ++g)
+          *reinterpret_cast<float4*>(w32 + b * bw + (2 * oc + g) * 4 * q3eb + 4 * r2) =
+              make_float4(f32_rne(x[4 * g]), f32_rne(x[4 * g + 1]), f32_rne(x[4 * g + 2]), f32_rne(x[4 * g + 3]));
       }
       if (b16) {
         unsigned v[4];
@@ -217,11 +219,7 @@ __global__ void k_split_words(const double* __restrict__ a, float* __restrict__ 
         if (wd < kLinWords) {
           const long long i = b * bw + wd * q3eb + r2;
           const double x = a[i];
-          if (hi) {
-            const df64 sv = df_split_rn(x);
-            hi[i] = sv.hi;
-            if (lo) lo[i] = sv.lo;
-          }
+          if (w32) w32[i] = f32_rne(x);
           v[c] = bf16_rne(x);
         }
       }
@@ -231,12 +229,11 @@ __global__ void k_split_words(const double* __restrict__ a, float* __restrict__ 
     }
   }
 }
-cudaError_t launch_split_words(const double* a, float* hi, float* lo, uint16_t* b16, long long nblk, int Q,
-                               cudaStream_t st) {
-  if (nblk == 0 || (!hi && !b16)) return cudaSuccess;
+cudaError_t launch_level_words(const double* a, float* w32, uint16_t* b16, long long nblk, int Q, cudaStream_t st) {
+  if (nblk == 0 || (!w32 && !b16)) return cudaSuccess;
   const long long q3eb = (long long)Q * Q * Q * elems_per_block(Q);
   const long long n = nblk * 10 * q3eb;
-  k_split_words<<<grid_for(n), kVecThreads, 0, st>>>(a, hi, lo, b16, nblk, q3eb); note_launch();
+  k_level_words<<<grid_for(n), kVecThreads, 0, st>>>(a, w32, b16, nblk, q3eb); note_launch();
   return cudaGetLastError();
 }
 
