@@ -364,6 +364,7 @@ int pff_create_context(pff_ctx** out, const pff_problem* pr) {
   c->glob.zeta = pr->zeta;
   c->glob.dt = pr->dt;
   c->glob.s_phi = pr->s_phi;
+  c->glob.zdt = pr->zeta / pr->dt;
   *out = c;
   return PFF_OK;
 }
@@ -392,6 +393,7 @@ int pff_context_set_time_step(pff_ctx* ctx, double dt) {
   PFF_REQUIRE(ctx, "pff_context_set_time_step: null context");
   PFF_REQUIRE(dt > 0.0 && std::isfinite(dt), "pff_context_set_time_step: dt must be positive and finite");
   ctx->glob.dt = dt;
+  ctx->glob.zdt = ctx->glob.zeta / dt;
   for (int i = 0; i < ctx->nphase; ++i) {
     PhaseDev& ph = ctx->phase[i];
     ph.cmax = (ph.has[1] && ph.eta_d > 0.0) ? ph.mu[1] * dt / ph.eta_d : 0.0;

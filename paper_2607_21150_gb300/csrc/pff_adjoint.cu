@@ -103,8 +103,8 @@ __global__ void __launch_bounds__(128) k_adjoint_point(const AdjArgs a) {
                           Hm[0][2] * (Hm[1][0] * Hm[2][1] - Hm[1][1] * Hm[2][0]);
       const double Jm1 = trH + 0.5 * (trH * trH - trHH) + detH;
       if (!(Jm1 > -1.0)) status |= 2;
-      theta = log1p(Jm1);
-      const double rJ = 1.0 / (1.0 + Jm1);
+      theta = 2.0 * half_log1p(Jm1);
+      const double rJ = rcp64(1.0 + Jm1);
 #pragma unroll
       for (int r = 0; r < 3; ++r)
 #pragma unroll
@@ -155,22 +155,12 @@ __global__ void __launch_bounds__(128) k_adjoint_point(const AdjArgs a) {
             X[r][c] += sm;
             if (c != r) X[c][r] += sm;
           }
-        // Jacobi in the Hooke branch's frame, where X is nearly diagonal
-        double Xt[3][3], Nt[3][3];
-        to_frame(Bs[0].N, X, Xt);
-        if (!jacobi3(Xt, Nt, B.x)) status |= 1;
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-#pragma unroll
-          for (int c = 0; c < 3; ++c)
-            B.N[r][c] = Bs[0].N[r][0] * Nt[0][c] + Bs[0].N[r][1] * Nt[1][c] + Bs[0].N[r][2] * Nt[2][c];
-      } else {
-        if (!jacobi3(X, B.N, B.x)) status |= 1;
       }
+      if (!eigh3(X, B.N, B.x)) status |= 1;
       double tr = 0.0;
 #pragma unroll
       for (int p = 0; p < 3; ++p) {
-        B.ed[p] = 0.5 * log1p(B.x[p]);
+        B.ed[p] = half_log1p(B.x[p]);
         tr += B.ed[p];
       }
 #pragma unroll
@@ -233,7 +223,7 @@ __global__ void __launch_bounds__(128) k_adjoint_point(const AdjArgs a) {
       gpar[0] = kap0bar / (3.0 * tnu);
       gpar[1] = 2.0 * kap0bar * ph.E0 / (3.0 * tnu * tnu);
       a.hbar_out[13 * nq + q] = active ? 0.0 : Hbar;
-      a.hbar_out[14 * nq + q] = -gl.zeta * Lbar / gl.dt;
+      a.hbar_out[14 * nq + q] = -gl.zdt * Lbar;
 #pragma unroll
       for (int r = 0; r < 3; ++r)
 #pragma unroll
@@ -290,7 +280,7 @@ __global__ void __launch_bounds__(128) k_adjoint_point(const AdjArgs a) {
           to_frame(B.N, M, G);
 #pragma unroll
           for (int p = 0; p < 3; ++p) {
-            ghat[p] = exp(2.0 * (B.af * B.ed[p] + theta * (1.0 / 3.0)));
+            ghat[p] = exp_near(2.0 * (B.af * B.ed[p] + theta * (1.0 / 3.0)));
             const double gg = 2.0 * ghat[p] * G[p][p];
             abar += gg * B.ed[p];
             edbar[p] += gg * B.af;

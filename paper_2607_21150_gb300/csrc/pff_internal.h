@@ -107,6 +107,7 @@ struct PhaseDev {
 struct GlobDev {
   int at;                 // 1 = AT1, 2 = AT2
   double eta, zeta, dt, s_phi;
+  double zdt;             // zeta / dt
 };
 
 // Geometry of the affine box elements.

@@ -6,10 +6,7 @@
 // takes eps_i = log1p(x_i) / 2 (the log1p form of Sec. 2.2), corrects the
 // deviatoric principal strains with the branch factor a_k (Box 1 step 2 and
 // Eq. principal-directions-format-1 with the degraded mu and q_tr of Sec. 3),
-// and rebuilds tau_d,k = N diag(2 mu a eps_d) N^T.  The Maxwell and Prandtl
-// branches are diagonalised in the Hooke branch's principal frame (their b_tr
-// differ from it by the inelastic strains, so Jacobi starts nearly
-// converged).  The volumetric strain
+// and rebuilds tau_d,k = N diag(2 mu a eps_d) N^T.  The volumetric strain
 // theta = ln J is shared by all branches and decides the Amor split
 // (Eqs. linear-Psi-plus, linear-degraded-stress).
 //
@@ -85,10 +82,10 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
                       Hm[0][2] * (Hm[1][0] * Hm[2][1] - Hm[1][1] * Hm[2][0]);
   const double Jm1 = trH + 0.5 * (trH * trH - trHH) + detH;
   if (!(Jm1 > -1.0)) status |= 2;
-  const double theta = log1p(Jm1);
+  const double theta = 2.0 * half_log1p(Jm1);
   const double J = 1.0 + Jm1;
   double Fi[3][3];
-  const double rJ = 1.0 / J;
+  const double rJ = rcp64(J);
   Fi[0][0] = (F[1][1] * F[2][2] - F[1][2] * F[2][1]) * rJ;
   Fi[0][1] = (F[0][2] * F[2][1] - F[0][1] * F[2][2]) * rJ;
   Fi[0][2] = (F[0][1] * F[1][2] - F[0][2] * F[1][1]) * rJ;
@@ -100,10 +97,11 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
   Fi[2][2] = (F[0][0] * F[1][1] - F[0][1] * F[1][0]) * rJ;
   double GG[3][3];  // F F^T - I
   for (int r = 0; r < 3; ++r)
-    for (int c = 0; c < 3; ++c) {
+    for (int c = r; c < 3; ++c) {
       double s = Hm[r][c] + Hm[c][r];
       for (int k = 0; k < 3; ++k) s += Hm[r][k] * Hm[c][k];
       GG[r][c] = s;
+      GG[c][r] = s;
     }
 
   // degradation g = (1 - phi)^2 + eta (Eq. degr-funct)
@@ -131,7 +129,6 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
   double hist_new[12];
   for (int v = 0; v < 12; ++v) hist_new[v] = a.hist[v * nq + q];
 
-  double N0[3][3];  // principal frame of the Hooke branch (always present): warm start of the others
   for (int br = 0; br < 3; ++br) {
     if (!ph.has[br]) continue;
     const double mu = ph.mu[br];
@@ -158,36 +155,16 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
         }
     }
     double N[3][3], x[3];
-    if (br == 0) {
-      if (!jacobi3(X, N, x)) status |= 1;
-      for (int r = 0; r < 3; ++r)
-        for (int c = 0; c < 3; ++c) N0[r][c] = N[r][c];
-    } else {
-      // the inelastic branches' b_tr differ from the elastic one by the
-      // (small) inelastic strains, so in the Hooke frame X is nearly
-      // diagonal: Jacobi on N0^T X N0 needs fewer sweeps, N = N0 N~
-      double T1[3][3], Xt[3][3], Nt[3][3];
-      for (int r = 0; r < 3; ++r)
-        for (int c = 0; c < 3; ++c) T1[r][c] = X[r][0] * N0[0][c] + X[r][1] * N0[1][c] + X[r][2] * N0[2][c];
-      for (int r = 0; r < 3; ++r)
-        for (int c = r; c < 3; ++c) {
-          const double v = N0[0][r] * T1[0][c] + N0[1][r] * T1[1][c] + N0[2][r] * T1[2][c];
-          Xt[r][c] = v;
-          Xt[c][r] = v;
-        }
-      if (!jacobi3(Xt, Nt, x)) status |= 1;
-      for (int r = 0; r < 3; ++r)
-        for (int c = 0; c < 3; ++c) N[r][c] = N0[r][0] * Nt[0][c] + N0[r][1] * Nt[1][c] + N0[r][2] * Nt[2][c];
-    }
+    if (!eigh3(X, N, x)) status |= 1;
     double eps[3], ed[3];
-    for (int p = 0; p < 3; ++p) eps[p] = 0.5 * log1p(x[p]);
+    for (int p = 0; p < 3; ++p) eps[p] = half_log1p(x[p]);
     const double tr = eps[0] + eps[1] + eps[2];
     for (int p = 0; p < 3; ++p) ed[p] = eps[p] - tr * (1.0 / 3.0);
     const double s2 = ed[0] * ed[0] + ed[1] * ed[1] + ed[2] * ed[2];
     double af = 1.0, da_dphi = 0.0, cq = 0.0;
     bool plastic = false;
     if (br == 1) {
-      af = 1.0 / (1.0 + ph.cmax * g);
+      af = rcp64(1.0 + ph.cmax * g);
       da_dphi = -af * af * ph.cmax * gp;
     } else if (br == 2) {
       // Box 2, degraded: admissible iff g q_tr <= sigma_y(ep_n); else the local Newton
@@ -222,7 +199,7 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
 
     if (br > 0) {  // trial history: C = F^-1 N diag(exp(2 eps_e)) N^T F^-T
       double ee[3];
-      for (int p = 0; p < 3; ++p) ee[p] = exp(2.0 * (af * ed[p] + theta / 3.0));
+      for (int p = 0; p < 3; ++p) ee[p] = exp_near(2.0 * (af * ed[p] + theta * (1.0 / 3.0)));
       double W[3][3];  // F^-1 N
       for (int r = 0; r < 3; ++r)
         for (int c = 0; c < 3; ++c) W[r][c] = Fi[r][0] * N[0][c] + Fi[r][1] * N[1][c] + Fi[r][2] * N[2][c];
@@ -359,7 +336,7 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
   const double Hh = active ? psip : Hn;
   const double alphap = (gl.at == 1) ? 1.0 : 2.0 * phi;
   const double phin = a.hist[14 * nq + q];
-  const double L = gp * Hh + ph.gc_c0l0 * alphap + gl.zeta * (phi - phin) / gl.dt;
+  const double L = gp * Hh + ph.gc_c0l0 * alphap + gl.zdt * (phi - phin);
 
   // residual integrands, parent frame with the weight folded in
   double Pm[3][3];
@@ -397,7 +374,7 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
     const int el = (int)(e % EB);
     double* lin = a.lin + blk * (long long)kLinWords * stride + (long long)qk * Q2 * EB + el * Q2 + qj * Q + qi;
     const double app = (gl.at == 1) ? 0.0 : 2.0;
-    const double cL = 2.0 * Hh + ph.gc_c0l0 * app + gl.zeta / gl.dt;
+    const double cL = 2.0 * Hh + ph.gc_c0l0 * app + gl.zdt;
     // mapped mesh: reference-frame columns kept, transformed to the parent frame below
     double Dm[9][9], Pv[9], Lv[9], Lphi = 0.0;
     // double-float copies of the point's scalars and matrices
