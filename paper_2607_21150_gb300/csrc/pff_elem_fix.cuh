@@ -20,10 +20,10 @@
 // converted by integer operations too, rounded to nearest.  Non-finite entries
 // make their field's values NaN in the element, as the dense contractions did.
 //
-// A block takes fix_elems(Q) elements (about 128 threads) of a group of
+// A block takes fix_elems(Q) elements (128 to 192 threads) of a group of
 // elems_per_block(Q) that the stored words are tiled by.  A thread is a node in
 // the gather and the scatter, a line in the contractions (4 Q^2 lines) and a
-// Gauss point in the map, Q^3 threads per element: 24 warps per SM (Q4) whose
+// Gauss point in the map, Q^3 threads per element: up to 30 warps per SM whose
 // integer and FP64 phases overlap, and short serial chains on meshes of a few
 // elements.  The 1D matrices are kernel parameters (constant-bank operands).
 //
@@ -32,7 +32,7 @@
 // busy, issue 52 %, DRAM 28 %).  With one thread per column of points (12 warps
 // per SM, as the FP64 kernel had it) 17 ms; with one copy of the line code per
 // direction instead of loops over the directions 9.1 ms (instruction cache).
-// 4^3 Q2: 56 -> 13.3 us (64 elements in sixteen blocks instead of three).
+// 4^3 Q2: 56 -> 13.3 us (64 elements in 21 blocks instead of three).
 #pragma once
 #include "pff_df.cuh"
 #include "pff_internal.h"
@@ -119,11 +119,11 @@ __device__ __forceinline__ double fx_to(long long m, int ex, int orv) {
 }
 constexpr int kFxNan = 0x7ff80000;
 // *m = max(*m, v) over the threads of an element: by warp where a warp holds one
-// element only (Q >= 4), so that the shared atomics do not queue up.
+// element only (Q >= 4), so that the shared atomics do not queue up (for Q = 3 a
+// reduction over the lanes of each element measured slower than the atomics).
 template <int Q> __device__ __forceinline__ void fx_max(int* m, int v) {
   if (Q >= 4) {
-    const unsigned lanes = __activemask();
-    v = __reduce_max_sync(lanes, v);
+    v = __reduce_max_sync(__activemask(), v);
     if ((threadIdx.x & 31) == 0) atomicMax(m, v);
   } else {
     atomicMax(m, v);
@@ -134,21 +134,28 @@ template <int Q> __device__ __forceinline__ void fx_max(int* m, int v) {
 // y-derivatives, or a ping-pong buffer of the contractions); C, Q^3 (the value
 // term of the phase field).
 template <int Q> __host__ __device__ constexpr int fix_elem_words() { return 13 * Q * Q * Q; }
-__host__ __device__ constexpr int fix_elems(int Q) { return Q == 5 ? 1 : Q == 4 ? 2 : Q == 3 ? 4 : 16; }
-// Resident blocks the register allocation is held to (24 warps per SM, 80 registers;
-// five blocks of 96 registers take 7.84 ms instead of 7.72 at 64^3 Q4).
-__host__ __device__ constexpr int fix_blocks() { return 6; }
+// Elements per block.  Q = 3: seven, whose 252 lines fill 189 threads better
+// (24x25x23 elements: 113.7 us, with four 123.4), but four on meshes too small to
+// give every SM two such blocks (4^3: 18.9 us, with seven 22.8).
+__host__ __device__ constexpr int fix_elems(int Q, bool small) {
+  return Q == 5 ? 1 : Q == 4 ? 2 : Q == 3 ? (small ? 4 : 7) : 16;
+}
+// Resident blocks the register allocation is held to: about 30 warps per SM
+// (40x33x37 elements, 20 / 24 / 30 / 36 warps: Q2 376 / 335 / 316 / 326 us, Q3 - /
+// 657 / 645 / 681 us, Q4 - / 1493 / 1495 / 1564 us).
+__host__ __device__ constexpr int fix_blocks(int threads) { return 30 / ((threads + 31) / 32); }
 
-template <int P, int Q, int MODE>
-__global__ void __launch_bounds__(Q * Q * Q * fix_elems(Q), fix_blocks())
+template <int P, int Q, int MODE, int EBS>
+__global__ void __launch_bounds__(Q * Q * Q * EBS, fix_blocks(Q * Q * Q * EBS))
 k_elem_fix(const ElemArgs<double> a) {
-  constexpr int EB = elems_per_block(Q), EBS = fix_elems(Q), NSUB = EB / EBS;
+  constexpr int EB = elems_per_block(Q), NSUB = EB / EBS;
   constexpr int Q2 = Q * Q, Q3 = Q * Q * Q, P2 = P * P, P3 = P * P * P;
   static_assert(NSUB * EBS == EB, "a block's elements divide the group");
   __shared__ long long sm[EBS * fix_elem_words<Q>()];
   __shared__ int emax[EBS][12];  // exponents: x per field, [4..7] gradient outputs, [8] value output
+  constexpr int NT = Q3 * EBS;
   const int t = threadIdx.x;
-  const int el = t / Q3, pt = t % Q3;  // node, line or point of the element
+  const int el = t / Q3, pt = t % Q3;  // element, and node or point of it
   const long long grp = a.blk0 + blockIdx.x / NSUB;
   const int sub = blockIdx.x % NSUB;
   const int e = (int)(grp * EB) + sub * EBS + el;
@@ -188,10 +195,11 @@ k_elem_fix(const ElemArgs<double> a) {
     for (int d = 0; d < 3; ++d) {
       const int lines = P == Q ? Q2 : d == 0 ? P2 : d == 1 ? P * Q : Q2, is = d == 0 ? 1 : d == 1 ? Q : Q2;
 #pragma unroll 1
-      for (int L = pt; L < 4 * lines; L += Q3) {
-        const int f = P == Q ? L / Q2 : d == 0 ? L / P2 : d == 1 ? L / (P * Q) : L / Q2, r = L - f * lines;
-        const long long* in = (d == 1 ? B : A) + f * Q3 + (d == 0 ? r * P : d == 1 ? r / Q * (P * Q) + r % Q : r);
-        long long* out = (d == 0 ? B : A) + f * Q3 + (d == 0 ? r * Q : d == 1 ? r / Q * Q2 + r % Q : r);
+      for (int L = t; L < 4 * EBS * lines; L += NT) {
+        const int ef = P == Q ? L / Q2 : d == 0 ? L / P2 : d == 1 ? L / (P * Q) : L / Q2, r = L - ef * lines;
+        long long* S = sm + (EBS == 1 ? ef * Q3 : ef / 4 * fix_elem_words<Q>() + ef % 4 * Q3);
+        const long long* in = (d == 1 ? S + 4 * Q3 : S) + (d == 0 ? r * P : d == 1 ? r / Q * (P * Q) + r % Q : r);
+        long long* out = (d == 0 ? S + 4 * Q3 : S) + (d == 0 ? r * Q : d == 1 ? r / Q * Q2 + r % Q : r);
         fx_line<P, Q, false>(fx.Bh, fx.Bl, in, is, out, is);
       }
       __syncthreads();
@@ -203,8 +211,9 @@ k_elem_fix(const ElemArgs<double> a) {
     for (int d = 0; d < 3; ++d) {
       if (d == 2) __syncthreads();
 #pragma unroll 1
-      for (int L = pt; L < 4 * Q2; L += Q3) {
-        const int f = L / Q2, r = L % Q2;
+      for (int L = t; L < 4 * EBS * Q2; L += NT) {
+        const int ef = L / Q2, r = L % Q2, f = EBS == 1 ? ef : ef % 4;
+        long long *A = sm + (EBS == 1 ? 0 : ef / 4 * fix_elem_words<Q>()), *B = A + 4 * Q3;
         const int o = d == 0 ? r * Q : d == 1 ? r / Q * Q2 + r % Q : r;  // lines (k, j), (k, i), (j, i)
         fx_line<Q, Q, false>(fx.Dh, fx.Dl, A + f * Q3 + o, d == 0 ? 1 : d == 1 ? Q : Q2,
                              d == 2 ? A + f * Q3 + o : B + (2 * f + d) * Q3 + o, d == 0 ? 1 : d == 1 ? Q : Q2);
@@ -279,15 +288,16 @@ k_elem_fix(const ElemArgs<double> a) {
   __syncthreads();
   // exponent of the column sums of field f: three derivative sums (2^eD bounds
   // their weights) and, in the phase field, the value term
-  auto sum_exponent = [&](int f) {
+  auto sum_exponent = [&](int el, int f) {
     const int eg = emax[el][4 + f] + fx.eD;
     return f < 3 ? eg : max(eg, emax[el][8]) + 1;
   };
   // transposed derivatives: x and y lines in place, then the z lines, which sum
   // the three (and the value term) and contract z into A [c][j][i]
 #pragma unroll 1
-  for (int L = pt; L < 4 * Q2; L += Q3) {
-    const int f = L / Q2, r = L % Q2, ey = sum_exponent(f);
+  for (int L = t; L < 4 * EBS * Q2; L += NT) {
+    const int ef = L / Q2, r = L % Q2, f = EBS == 1 ? ef : ef % 4, ey = sum_exponent(EBS == 1 ? 0 : ef / 4, f);
+    long long* B = sm + (EBS == 1 ? 0 : ef / 4 * fix_elem_words<Q>()) + 4 * Q3;
 #pragma unroll 1
     for (int dir = 0; dir < 2; ++dir) {
       long long* ln = B + (2 * f + dir) * Q3 + (dir ? (r / Q) * Q2 + r % Q : r * Q);
@@ -300,8 +310,10 @@ k_elem_fix(const ElemArgs<double> a) {
   }
   __syncthreads();
 #pragma unroll 1
-  for (int L = pt; L < 4 * Q2; L += Q3) {
-    const int f = L / Q2, r = L % Q2, ey = sum_exponent(f);
+  for (int L = t; L < 4 * EBS * Q2; L += NT) {
+    const int ef = L / Q2, r = L % Q2, f = EBS == 1 ? ef : ef % 4, ey = sum_exponent(EBS == 1 ? 0 : ef / 4, f);
+    long long *A = sm + (EBS == 1 ? 0 : ef / 4 * fix_elem_words<Q>()), *B = A + 4 * Q3;
+    const double* C = reinterpret_cast<const double*>(B + 8 * Q3);
     long long* col = A + f * Q3 + r;
     long long v[Q], y[Q];
 #pragma unroll
@@ -320,10 +332,11 @@ k_elem_fix(const ElemArgs<double> a) {
   for (int d = 1; d >= 0; --d) {
     const int lines = d == 1 ? P * Q : P2;
 #pragma unroll 1
-    for (int L = pt; L < 4 * lines; L += Q3) {
-      const int f = P == Q ? L / Q2 : d == 1 ? L / (P * Q) : L / P2, r = L - f * lines;
-      const long long* in = (d == 1 ? A : B) + f * Q3 + (d == 1 ? r / Q * Q2 + r % Q : r * Q);
-      long long* out = (d == 1 ? B : A) + f * Q3 + (d == 1 ? r / Q * (P * Q) + r % Q : r * P);
+    for (int L = t; L < 4 * EBS * lines; L += NT) {
+      const int ef = P == Q ? L / Q2 : d == 1 ? L / (P * Q) : L / P2, r = L - ef * lines;
+      long long* S = sm + (EBS == 1 ? ef * Q3 : ef / 4 * fix_elem_words<Q>() + ef % 4 * Q3);
+      const long long* in = (d == 1 ? S : S + 4 * Q3) + (d == 1 ? r / Q * Q2 + r % Q : r * Q);
+      long long* out = (d == 1 ? S + 4 * Q3 : S) + (d == 1 ? r / Q * (P * Q) + r % Q : r * P);
       fx_line<Q, P, true>(fx.Bh, fx.Bl, in, d == 1 ? Q : 1, out, d == 1 ? Q : 1);
     }
     __syncthreads();
@@ -332,7 +345,7 @@ k_elem_fix(const ElemArgs<double> a) {
 #pragma unroll
   for (int f = 0; f < 4; ++f) {
     const bool bad = emax[el][4 + f] == 2047 || (f == 3 && emax[el][8] == 2047);
-    const double v = fx_to(A[f * Q3 + pt], sum_exponent(f) - 1022 - fx.wb, bad ? kFxNan : 0);
+    const double v = fx_to(A[f * Q3 + pt], sum_exponent(el, f) - 1022 - fx.wb, bad ? kFxNan : 0);
     if (a.evec)  // deterministic transpose: element-local values, summed per node by k_node_gather
       static_cast<double*>(a.evec)[((long long)e * 4 + f) * P3 + pt] = v;
     else if (!(masked && __ldg(a.mask + f * nn + n)))
@@ -340,11 +353,16 @@ k_elem_fix(const ElemArgs<double> a) {
   }
 }
 
+template <int P, int Q, int MODE, int EBS>
+cudaError_t launch_fix(const ElemArgs<double>& a, int nblk, cudaStream_t st) {
+  k_elem_fix<P, Q, MODE, EBS><<<(unsigned)nblk * (elems_per_block(Q) / EBS), Q * Q * Q * EBS, 0, st>>>(a); note_launch();
+  return cudaGetLastError();
+}
 template <int P, int Q, int MODE>
 cudaError_t launch_elem_fix(const ElemArgs<double>& a, int nblk, cudaStream_t st) {
-  constexpr int EBS = fix_elems(Q);
-  k_elem_fix<P, Q, MODE><<<(unsigned)nblk * (elems_per_block(Q) / EBS), Q * Q * Q * EBS, 0, st>>>(a); note_launch();
-  return cudaGetLastError();
+  constexpr int big = fix_elems(Q, false), small = fix_elems(Q, true);
+  if (small != big && nblk * (elems_per_block(Q) / big) < 2 * 152) return launch_fix<P, Q, MODE, small>(a, nblk, st);
+  return launch_fix<P, Q, MODE, big>(a, nblk, st);
 }
 
 }  // namespace pff
