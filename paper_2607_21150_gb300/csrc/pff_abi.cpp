@@ -48,6 +48,14 @@ int upload(const std::vector<double>& h, T** d) {
 
 namespace {
 
+// v in FP32 in both halves of a packed pair
+unsigned long long twice(double v) {
+  const float h[2] = {(float)v, (float)v};
+  unsigned long long r;
+  std::memcpy(&r, h, sizeof(r));
+  return r;
+}
+
 long long stride_of(int Q) { return (long long)Q * Q * Q * elems_per_block(Q); }
 
 int make_tables(int p, int Q, Tables& t) {
@@ -64,11 +72,12 @@ int make_tables(int p, int Q, Tables& t) {
   for (int i = 0; i < Q; ++i)
     for (int k = 0; k < Q; ++k) Dc[i * Q + k] = lagrange_deriv(xq.data(), Q, k, xq[i]);
   for (int i = 0; i < Q * P; ++i) {
-    t.hB32[i] = (float)B[i];
+    t.hB2[i] = twice(B[i]);
+    t.hD2[i] = twice(Dt[i]);
     t.hB[i] = B[i];
     t.hDt[i] = Dt[i];
   }
-  for (int i = 0; i < Q * Q; ++i) t.hDc32[i] = (float)Dc[i];
+  for (int i = 0; i < Q * Q; ++i) t.hDc2[i] = twice(Dc[i]);
   t.fix = fix_table(P, Q, B.data(), Dc.data());
   int rc;
   if ((rc = upload(B, &t.B64))) return rc;
@@ -162,8 +171,9 @@ ElemArgs<T> level_args(const pff_level* L) {
   a.nq = L->op->nq;
   a.kx = L->op->geo != nullptr;
   for (int d = 0; d < 3; ++d) a.s[d] = L->op->geom.s[d];
-  std::memcpy(a.cB, L->tab.hB32, sizeof(a.cB));
-  std::memcpy(a.cDc, L->tab.hDc32, sizeof(a.cDc));
+  std::memcpy(a.cB2, L->tab.hB2, sizeof(a.cB2));
+  std::memcpy(a.cD2, L->tab.hD2, sizeof(a.cD2));
+  std::memcpy(a.cDc2, L->tab.hDc2, sizeof(a.cDc2));
   return a;
 }
 

@@ -21,10 +21,21 @@
 //
 // The x- and y-derivative outputs of slice k go through a double-buffered
 // slice buffer and are contracted at the next slice, after the barrier that
-// frees the slot; shared memory per element is then 8 Q^3 values (Q = 5), so
-// that two slots and two blocks fit on an SM.  The interpolation and its
-// transpose are line transforms (fwd_lines / bwd_lines, pff_elem.cuh) with the
-// 1D matrices as kernel parameters; the slice loop stays rolled for P >= 3.
+// frees the slot; the z direction is contracted as the slices come, into the
+// nodal column Z[c] += B[k][c] (xy part) + D_t[k][c] (z part).  Shared memory
+// per element is then 8 Q^3 values (Q = 5), so that two slots and two blocks
+// fit on an SM.  The slice loop stays rolled for P >= 3.
+//
+// Bound: shared-memory bandwidth (82 % of its cycles at 40^3 Q4 with BF16
+// words; a 128-bit access moves four fields but takes four cycles), with FP32
+// words and few contractions (Q3) the word stream.  What brought it there: the
+// four fields side by side in packed pairs and one line per thread, a third
+// fewer instructions than one field at a time; mask bytes loaded in one batch
+// by the elements that need them and kept as bits for the scatter -- tested
+// one by one they made elements at a masked face twice as slow, and blocks
+// that walk a row of such elements late.  40^3 Q4 BF16 words 462 -> 319 us,
+// 33x27x35 curved Q3 FP32 words 126.8 -> 99.5 us (stream alone about 87 us).
+// Keeping the own Gauss column in registers for the z gradients spills: 350 us.
 //
 // Every wait on an mbarrier is bounded (about one second of clock cycles); a
 // wait that runs out sets status bit 32 (the result is then invalid).  A wait
@@ -247,115 +258,265 @@ __device__ __forceinline__ void jac_words(const unsigned* r, const float g[4][3]
   }
 }
 
+// --- contractions on quads -------------------------------------------------
+// The contractions treat the four fields alike, so shared memory holds them
+// side by side: one quad (float4) per node or Gauss point, loaded and stored
+// whole, and contracted as two packed pairs (fma.rn.f32x2: each half rounds as
+// fmaf does).  A thread then moves a line of all four fields in P (Q) 128-bit
+// accesses, and one line per thread is the whole stage (P <= Q).
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pk(float lo, float hi) {
+  f32x2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ void unpk(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+struct alignas(16) Quad {
+  f32x2 a, b;  // fields 0, 1 and 2, 3
+};
+__device__ __forceinline__ void fmaq(Quad& acc, f32x2 w, const Quad& v) {
+  acc.a = fma2(w, v.a, acc.a);
+  acc.b = fma2(w, v.b, acc.b);
+}
+
+// Places of the quads in shared memory.  A 128-bit access is served eight
+// lanes at a time, and the rows of even length that the x- and y-lines step
+// through would put those lanes on the same banks; swapping places inside a
+// row (and, for Q = 4, neighbouring rows) keeps them apart.  Odd lengths need
+// nothing.  nodes [c][b][a], x-transformed [c][b][i], xy-transformed [c][j][i].
+template <int P> __device__ __forceinline__ int at_node(int cb, int a) {
+  if (P == 4) return cb * 4 + (a ^ ((cb >> 1) & 3));
+  if (P == 2) return cb * 2 + (a ^ ((cb >> 2) & 1));
+  return cb * P + a;
+}
+template <int P, int Q> __device__ __forceinline__ int at_x(int c, int b, int i) {
+  if (Q != 4) return (c * P + b) * Q + i;
+  const int row = c * P + b;
+  return 4 * (P == 4 ? row ^ (c & 1) : row) + (i ^ (b & 3));
+}
+template <int Q> __device__ __forceinline__ int at_xy(int c, int ij) {
+  return c * Q * Q + (Q == 4 ? ij ^ ((c & 1) << 2) : ij);
+}
+
+// Nodes of an element: pipe_base of the element, then node_at for the thread's
+// r-th node (node idx = ij + r Q^2 of the element; for P = Q that is node
+// (i, j, r), a plane apart from the one before).
+template <int P> __device__ __forceinline__ long long pipe_base(const MeshDev& m, int e) {
+  if (m.offsets) return (long long)e * (P * P * P);
+  const int t = e / m.nx, ex = e - t * m.nx, ez = t / m.ny, ey = t - ez * m.ny;
+  return (long long)m.p * (ex + (long long)m.nnx * (ey + (long long)m.nny * ez));
+}
+template <int P, int Q> __device__ __forceinline__ long long node_at(const MeshDev& m, long long base, int ij, int r) {
+  const int idx = ij + r * Q * Q;
+  if (m.offsets) return m.offsets[base + idx];
+  const long long plane = (long long)m.nnx * m.nny;
+  if (P == Q) return base + (ij % Q + m.nnx * (ij / Q)) + r * plane;
+  return base + (idx % P + m.nnx * ((idx / P) % P)) + (idx / (P * P)) * plane;
+}
+
 // Gather of an element's nodal values (structured map or explicit offsets),
 // split so that the loads of the next element block are in flight while the
 // present block runs its transposed contractions: pipe_gather_load issues the
-// loads of thread ij's nodes (masked entries read as zero), pipe_gather_store
-// writes them to bufA [4][c][b][a].
+// loads of thread ij's nodes (masked entries read as zero) and returns their
+// mask, bit 4 r + f, for the scatter; pipe_gather_store writes them to bufA.
+// Mask bytes are loaded all together, and only by elements that have masked
+// nodes: tested one by one behind each value, in gather and scatter, they cost
+// 120 of 470 us (40^3 Q4, BF16 words).
 template <int P, int Q> __host__ __device__ constexpr int pipe_gather_rounds() {
   return (P * P * P + Q * Q - 1) / (Q * Q);
 }
 template <int P, int Q>
-__device__ __forceinline__ void pipe_gather_load(const ElemArgs<float>& a, int e, bool valid, bool em, int ij,
-                                                 float xv[pipe_gather_rounds<P, Q>()][4]) {
-  constexpr int Q2 = Q * Q, P3 = P * P * P;
+__device__ __forceinline__ unsigned pipe_gather_load(const ElemArgs<float>& a, long long base, bool valid, bool em,
+                                                     int ij, float xv[pipe_gather_rounds<P, Q>()][4]) {
+  constexpr int Q2 = Q * Q, P3 = P * P * P, R = pipe_gather_rounds<P, Q>();
+  static_assert(4 * R <= 32, "mask bits");
   const long long nn = a.mesh.nn;
-  const bool masked = a.mask && valid && em;
 #pragma unroll
-  for (int r = 0; r < pipe_gather_rounds<P, Q>(); ++r) {
-    const int idx = ij + r * Q2;
-    const bool live = valid && idx < P3;
-    const int aa = idx % P, bb = (idx / P) % P, cc = idx / (P * P);
-    const long long n = live ? node_of<P, Q>(a.mesh, e, aa, bb, cc) : 0;
+  for (int r = 0; r < R; ++r) {
+    const bool live = valid && ij + r * Q2 < P3;
+    const long long n = live ? node_at<P, Q>(a.mesh, base, ij, r) : 0;
 #pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      const long long g = f * nn + n;
-      xv[r][f] = live ? __ldg(a.x + g) : 0.0f;
-      if (live && masked && __ldg(a.mask + g)) xv[r][f] = 0.0f;
-    }
+    for (int f = 0; f < 4; ++f) xv[r][f] = live ? __ldg(a.x + f * nn + n) : 0.0f;
   }
+  unsigned m = 0;
+  if (a.mask && valid && em) {
+    unsigned b[R][4];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const bool live = ij + r * Q2 < P3;
+      const long long n = live ? node_at<P, Q>(a.mesh, base, ij, r) : 0;
+#pragma unroll
+      for (int f = 0; f < 4; ++f) b[r][f] = __ldg(a.mask + f * nn + n);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int f = 0; f < 4; ++f)
+        if (b[r][f]) {
+          m |= 1u << (4 * r + f);
+          xv[r][f] = 0.0f;
+        }
+  }
+  return m;
 }
 template <int P, int Q>
-__device__ __forceinline__ void pipe_gather_store(float* bufA, int ij, const float xv[pipe_gather_rounds<P, Q>()][4]) {
-  constexpr int Q2 = Q * Q, Q3 = Q * Q * Q, P3 = P * P * P;
+__device__ __forceinline__ void pipe_gather_store(Quad* bufA, int ij, const float xv[pipe_gather_rounds<P, Q>()][4]) {
+  constexpr int Q2 = Q * Q, P3 = P * P * P;
 #pragma unroll
   for (int r = 0; r < pipe_gather_rounds<P, Q>(); ++r) {
     const int idx = ij + r * Q2;
-    if (idx < P3)
-#pragma unroll
-      for (int f = 0; f < 4; ++f) bufA[f * Q3 + idx] = xv[r][f];
+    if (idx < P3) bufA[at_node<P>(idx / P, idx % P)] = Quad{pk(xv[r][0], xv[r][1]), pk(xv[r][2], xv[r][3])};
   }
 }
 
-// Gradients of the four fields at point (i, j, k) from the Gauss-point values
-// V = bufB; the z-derivative row Dc[k][.] as kernel-parameter operands (k is
-// fixed at compile time), the x- and y-rows from shared memory.
+// Entry idx of the 1D interpolation matrix B [Q][P], both halves alike, from
+// the kernel parameters.
+__device__ __forceinline__ f32x2 basis_b2(const ElemArgs<float>& a, int idx) { return a.cB2[idx]; }
+
+// Interpolation to the Gauss points, one line per thread and stage: from bufA
+// (gathered) along x to bufB, along y to bufA, along z to bufB [k][j][i].
+template <int P, int Q>
+__device__ __forceinline__ void fwd_lines(const ElemArgs<float>& a, Quad* bufA, Quad* bufB, int ij) {
+  constexpr int Q2 = Q * Q;
+  Quad v[P];
+  __syncthreads();
+  if (ij < P * P) {  // x: line (c, b)
+#pragma unroll
+    for (int aa = 0; aa < P; ++aa) v[aa] = bufA[at_node<P>(ij, aa)];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      Quad acc{0, 0};
+#pragma unroll
+      for (int aa = 0; aa < P; ++aa) fmaq(acc, basis_b2(a, i * P + aa), v[aa]);
+      bufB[at_x<P, Q>(ij / P, ij % P, i)] = acc;
+    }
+  }
+  __syncthreads();
+  if (ij < P * Q) {  // y: line (c, i)
+    const int c = ij / Q, i = ij % Q;
+#pragma unroll
+    for (int b = 0; b < P; ++b) v[b] = bufB[at_x<P, Q>(c, b, i)];
+#pragma unroll
+    for (int j = 0; j < Q; ++j) {
+      Quad acc{0, 0};
+#pragma unroll
+      for (int b = 0; b < P; ++b) fmaq(acc, basis_b2(a, j * P + b), v[b]);
+      bufA[at_xy<Q>(c, j * Q + i)] = acc;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < P; ++c) v[c] = bufA[at_xy<Q>(c, ij)];  // z: the thread's own column (j, i)
+#pragma unroll
+  for (int k = 0; k < Q; ++k) {
+    Quad acc{0, 0};
+#pragma unroll
+    for (int c = 0; c < P; ++c) fmaq(acc, basis_b2(a, k * P + c), v[c]);
+    bufB[k * Q2 + ij] = acc;
+  }
+  __syncthreads();
+}
+
+// Transposed interpolation along y and x from the thread's own column Z[c] (the
+// z direction is contracted already), then the scatter-add (or the element
+// values of the deterministic mode).  base, m: pipe_base and the mask bits of the
+// element's nodes.
+template <int P, int Q>
+__device__ __forceinline__ void bwd_lines(const ElemArgs<float>& a, Quad* bufA, Quad* bufB, int e, long long base, bool valid,
+                                          unsigned m, int ij, const Quad Z[P]) {
+  constexpr int Q2 = Q * Q, P3 = P * P * P;
+  Quad v[Q];
+#pragma unroll
+  for (int c = 0; c < P; ++c) bufA[at_xy<Q>(c, ij)] = Z[c];
+  __syncthreads();
+  if (ij < P * Q) {  // y: line (c, i)
+    const int c = ij / Q, i = ij % Q;
+#pragma unroll
+    for (int j = 0; j < Q; ++j) v[j] = bufA[at_xy<Q>(c, j * Q + i)];
+#pragma unroll
+    for (int b = 0; b < P; ++b) {
+      Quad acc{0, 0};
+#pragma unroll
+      for (int j = 0; j < Q; ++j) fmaq(acc, basis_b2(a, j * P + b), v[j]);
+      bufB[at_x<P, Q>(c, b, i)] = acc;
+    }
+  }
+  __syncthreads();
+  if (ij < P * P) {  // x: line (c, b)
+#pragma unroll
+    for (int i = 0; i < Q; ++i) v[i] = bufB[at_x<P, Q>(ij / P, ij % P, i)];
+#pragma unroll
+    for (int aa = 0; aa < P; ++aa) {
+      Quad acc{0, 0};
+#pragma unroll
+      for (int i = 0; i < Q; ++i) fmaq(acc, basis_b2(a, i * P + aa), v[i]);
+      bufA[at_node<P>(ij, aa)] = acc;
+    }
+  }
+  __syncthreads();
+  if (!valid) return;
+  const long long nn = a.mesh.nn;
+#pragma unroll
+  for (int r = 0; r < pipe_gather_rounds<P, Q>(); ++r) {
+    const int idx = ij + r * Q2;
+    if (idx >= P3) break;
+    const Quad q = bufA[at_node<P>(idx / P, idx % P)];
+    float o[4];
+    unpk(q.a, o[0], o[1]);
+    unpk(q.b, o[2], o[3]);
+    if (a.evec) {  // deterministic mode: element-local values, summed per node by k_node_gather
+      float* ev = static_cast<float*>(a.evec) + (long long)e * 4 * P3;
+#pragma unroll
+      for (int f = 0; f < 4; ++f) ev[f * P3 + idx] = o[f];
+      continue;
+    }
+    float* y = a.y + node_at<P, Q>(a.mesh, base, ij, r);
+#pragma unroll
+    for (int f = 0; f < 4; ++f)
+      if (!(m >> (4 * r + f) & 1)) atomicAdd(y + f * nn, o[f]);
+  }
+}
+
+// Gradients of the four fields at point (i, j, k) from the Gauss-point values V.
+// The z-row of the collocated derivative is the same for all threads (kernel
+// parameters); the x- and y-rows come from shared memory.
 template <int Q>
-__device__ __forceinline__ void grad_at_c(const ElemArgs<float>& a, const float* V0, const float* Dc, int i, int j,
+__device__ __forceinline__ void grad_at_c(const ElemArgs<float>& a, const Quad* V, const float* Dc, int i, int j,
                                           int k, float g[4][3], float& phi) {
-  constexpr int Q2 = Q * Q, Q3 = Q * Q * Q;
-  float di[Q], dj[Q];
+  constexpr int Q2 = Q * Q;
+  Quad d[3] = {{0, 0}, {0, 0}, {0, 0}};
 #pragma unroll
   for (int m = 0; m < Q; ++m) {
-    di[m] = Dc[i * Q + m];
-    dj[m] = Dc[j * Q + m];
+    fmaq(d[0], pk(Dc[i * Q + m], Dc[i * Q + m]), V[k * Q2 + j * Q + m]);
+    fmaq(d[1], pk(Dc[j * Q + m], Dc[j * Q + m]), V[k * Q2 + m * Q + i]);
+    fmaq(d[2], a.cDc2[k * Q + m], V[m * Q2 + j * Q + i]);
   }
 #pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    const float* V = V0 + f * Q3;
-    float gx = 0.0f, gy = 0.0f, gz = 0.0f;
-#pragma unroll
-    for (int m = 0; m < Q; ++m) {
-      gx = fmaf(di[m], V[k * Q2 + j * Q + m], gx);
-      gy = fmaf(dj[m], V[k * Q2 + m * Q + i], gy);
-      gz = fmaf(a.cDc[k * Q + m], V[m * Q2 + j * Q + i], gz);
-    }
-    g[f][0] = gx; g[f][1] = gy; g[f][2] = gz;
+  for (int al = 0; al < 3; ++al) {
+    unpk(d[al].a, g[0][al], g[1][al]);
+    unpk(d[al].b, g[2][al], g[3][al]);
   }
-  phi = V0[3 * Q3 + k * Q2 + j * Q + i];
+  phi = reinterpret_cast<const float*>(V + k * Q2 + j * Q + i)[3];
 }
 
-// Transposed x- and y-derivatives of slice kc: Y[f][kc] += sum_m Dc[m, i] ox(m, j)
-// + Dc[m, j] oy(i, m), from the slice buffer sb = [8][Q^2] (ox, oy per field).
+// Transposed x- and y-derivatives of a slice at point (i, j): sum_m Dc[m, i]
+// ox(m, j) + Dc[m, j] oy(i, m), from the slice buffer sb = [2][Q^2] (ox, oy).
 template <int Q>
-__device__ __forceinline__ void pipe_contract_xy(const float* Dc, const float* sb, int i, int j, float Y[4][Q],
-                                                 int kc) {
-  constexpr int Q2 = Q * Q;
+__device__ __forceinline__ Quad pipe_contract_xy(const float* Dc, const Quad* sb, int i, int j) {
+  Quad acc{0, 0};
 #pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    float acc = Y[f][kc];
-#pragma unroll
-    for (int m = 0; m < Q; ++m) {
-      acc = fmaf(Dc[m * Q + i], sb[(2 * f) * Q2 + j * Q + m], acc);
-      acc = fmaf(Dc[m * Q + j], sb[(2 * f + 1) * Q2 + m * Q + i], acc);
-    }
-    Y[f][kc] = acc;
+  for (int m = 0; m < Q; ++m) {
+    fmaq(acc, pk(Dc[m * Q + i], Dc[m * Q + i]), sb[j * Q + m]);
+    fmaq(acc, pk(Dc[m * Q + j], Dc[m * Q + j]), sb[Q * Q + m * Q + i]);
   }
-}
-
-// The same contraction returned as the contribution c[f] to Y[f][kc], and its
-// addition at a slice index known only at run time (the rolled slice loop).
-template <int Q>
-__device__ __forceinline__ void pipe_contract_c(const float* Dc, const float* sb, int i, int j, float c[4]) {
-  constexpr int Q2 = Q * Q;
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    float acc = 0.0f;
-#pragma unroll
-    for (int m = 0; m < Q; ++m) {
-      acc = fmaf(Dc[m * Q + i], sb[(2 * f) * Q2 + j * Q + m], acc);
-      acc = fmaf(Dc[m * Q + j], sb[(2 * f + 1) * Q2 + m * Q + i], acc);
-    }
-    c[f] = acc;
-  }
-}
-template <int Q>
-__device__ __forceinline__ void add_at(float Y[4][Q], int kc, const float c[4]) {
-#pragma unroll
-  for (int kk = 0; kk < Q; ++kk)
-    if (kk == kc)
-#pragma unroll
-      for (int f = 0; f < 4; ++f) Y[f][kk] += c[f];
+  return acc;
 }
 
 template <int P, int Q, bool BF, bool KX, bool TR>
@@ -369,7 +530,7 @@ k_level_pipe(const ElemArgs<float> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* slots = smem_raw;                                    // [2][kSlot]
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + 2 * kSlot);  // one mbarrier per slot
-  float* sm = reinterpret_cast<float*>(smem_raw + 2 * kSlot + 16);
+  float* Dc = reinterpret_cast<float*>(smem_raw + 2 * kSlot + 16);  // [Q][Q] collocated derivative
   const int t = threadIdx.x;
   const int el = t / Q2, ij = t % Q2;
   const int i = ij % Q, j = ij / Q;
@@ -378,13 +539,11 @@ k_level_pipe(const ElemArgs<float> a) {
   const long long nstage = (long long)nmine * NS;
   const long long blk_first = (long long)a.blk0 + blockIdx.x;
 
-  float* Bs = sm;  // the 1D matrices where a thread's own index selects the row
-  float* Dcs = Bs + Q * P;
-  for (int idx = t; idx < Q * P; idx += blockDim.x) Bs[idx] = a.cB[idx];
-  for (int idx = t; idx < Q * Q; idx += blockDim.x) Dcs[idx] = a.cDc[idx];
-  float* base = sm + mat_smem_words<P, Q>() + el * pipe_elem_stride<Q>();
-  const ElemSmem<P, Q, float> s{base + 4 * Q3, base, Bs, Dcs};
-  float* sbuf = s.bufA;  // [2][8][Q^2] during the slice loop
+  // the 1D matrix whose row or column a thread's own index selects
+  for (int idx = t; idx < Q * Q; idx += blockDim.x) Dc[idx] = a.Dc[idx];
+  Quad* bufB = reinterpret_cast<Quad*>(smem_raw + 2 * kSlot + 16 + pipe_mat_bytes<Q>()) + el * pipe_elem_quads<Q>();
+  Quad* bufA = bufB + Q3;
+  Quad* sbuf = bufA;  // [2][2][Q^2] during the slice loop
   if (t == 0) {
     mbar_init(bar, 1);
     mbar_init(bar + 1, 1);
@@ -403,18 +562,17 @@ k_level_pipe(const ElemArgs<float> a) {
   bool valid = e < a.mesh.nel;
   bool em = valid && (!a.emask || a.emask[e]);
   float xv[pipe_gather_rounds<P, Q>()][4];
-  pipe_gather_load<P, Q>(a, e, valid, em, ij, xv);
+  long long base = pipe_base<P>(a.mesh, e);
+  unsigned m = pipe_gather_load<P, Q>(a, base, valid, em, ij, xv);
 
   for (int it = 0; it < nmine; ++it) {
     const long long blk = blk_first + (long long)it * G;
-    pipe_gather_store<P, Q>(s.bufA, ij, xv);
-    fwd_lines<P, Q>(a, s.bufA, s.bufB, ij);
+    pipe_gather_store<P, Q>(bufA, ij, xv);
+    fwd_lines<P, Q>(a, bufA, bufB, ij);
 
-    float Y[4][Q];
+    Quad Z[P];  // the own column, contracted along z as the slices come
 #pragma unroll
-    for (int f = 0; f < 4; ++f)
-#pragma unroll
-      for (int k = 0; k < Q; ++k) Y[f][k] = 0.0f;
+    for (int c = 0; c < P; ++c) Z[c] = Quad{0, 0};
     float g[4][3], phi = 0.0f, ou[9], s0 = 0.0f, o3[3] = {0.0f, 0.0f, 0.0f};
     // the slice loop stays rolled (smaller code: at 64^3 Q4 1 % faster with
     // FP32 words, 3 % with BF16 words) except on the order-1 level, whose
@@ -443,11 +601,11 @@ k_level_pipe(const ElemArgs<float> a) {
       ++seq;
       if (h == 0) {
         if (k > 0) {
-          float c[4];
-          pipe_contract_c<Q>(s.Dc, sbuf + ((k - 1) & 1) * 8 * Q2, i, j, c);
-          add_at<Q>(Y, k - 1, c);
+          const Quad y = pipe_contract_xy<Q>(Dc, sbuf + ((k - 1) & 1) * 2 * Q2, i, j);
+#pragma unroll
+          for (int c = 0; c < P; ++c) fmaq(Z[c], a.cB2[(k - 1) * P + c], y);
         }
-        grad_at_c<Q>(a, s.bufB, s.Dc, i, j, k, g, phi);
+        grad_at_c<Q>(a, bufB, Dc, i, j, k, g, phi);
 #pragma unroll
         for (int m = 0; m < 9; ++m) ou[m] = 0.0f;
         s0 = 0.0f;
@@ -464,39 +622,42 @@ k_level_pipe(const ElemArgs<float> a) {
           s0 = 0.0f;
           o3[0] = o3[1] = o3[2] = 0.0f;
         }
-        float* sb = sbuf + (k & 1) * 8 * Q2;
+        Quad* sb = sbuf + (k & 1) * 2 * Q2;
+        sb[ij] = Quad{pk(ou[0], ou[3]), pk(ou[6], o3[0])};
+        sb[Q2 + ij] = Quad{pk(ou[1], ou[4]), pk(ou[7], o3[1])};
+        const Quad oz{pk(ou[2], ou[5]), pk(ou[8], o3[2])};
+        const f32x2 ov = pk(0.0f, s0);
 #pragma unroll
-        for (int f = 0; f < 4; ++f) {
-          const float ox = f < 3 ? ou[3 * f] : o3[0];
-          const float oy = f < 3 ? ou[3 * f + 1] : o3[1];
-          const float oz = f < 3 ? ou[3 * f + 2] : o3[2];
-#pragma unroll
-          for (int kk = 0; kk < Q; ++kk) Y[f][kk] = fmaf(a.cDc[k * Q + kk], oz, Y[f][kk]);
-          sb[(2 * f) * Q2 + ij] = ox;
-          sb[(2 * f + 1) * Q2 + ij] = oy;
+        for (int c = 0; c < P; ++c) {
+          fmaq(Z[c], a.cD2[k * P + c], oz);
+          Z[c].b = fma2(a.cB2[k * P + c], ov, Z[c].b);
         }
-#pragma unroll
-        for (int kk = 0; kk < Q; ++kk)
-          if (kk == k) Y[3][kk] += s0;
       }
     }
     if (!staged) break;
     }
     if (!staged) break;
     __syncthreads();
-    pipe_contract_xy<Q>(s.Dc, sbuf + ((Q - 1) & 1) * 8 * Q2, i, j, Y, Q - 1);
+    {
+      const Quad y = pipe_contract_xy<Q>(Dc, sbuf + ((Q - 1) & 1) * 2 * Q2, i, j);
+#pragma unroll
+      for (int c = 0; c < P; ++c) fmaq(Z[c], a.cB2[(Q - 1) * P + c], y);
+    }
     // the next element block's nodal values are loaded while this one runs
     // its transposed contractions and scatter
     const int e_now = e;
-    const bool valid_now = valid, em_now = em;
+    const long long base_now = base;
+    const bool valid_now = valid;
+    const unsigned m_now = m;
     if (it + 1 < nmine) {
       e = (int)((blk + G) * EB) + el;
       valid = e < a.mesh.nel;
       em = valid && (!a.emask || a.emask[e]);
-      pipe_gather_load<P, Q>(a, e, valid, em, ij, xv);
+      base = pipe_base<P>(a.mesh, e);
+      m = pipe_gather_load<P, Q>(a, base, valid, em, ij, xv);
     }
     __syncthreads();  // the slice buffers are read; backward reuses them
-    bwd_lines<P, Q>(a, s.bufA, s.bufB, e_now, valid_now, em_now, ij, Y);
+    bwd_lines<P, Q>(a, bufA, bufB, e_now, base_now, valid_now, m_now, ij, Z);
     __syncthreads();  // the scatter has read bufA; the next gather writes it
   }
   // a wait gave up: the copies still in flight (stages [seq, issued), at most

@@ -32,7 +32,9 @@ struct pff_restr {
 struct Tables {  // per-level device copies of the 1D matrices, both precisions
   double *B64 = nullptr, *Dc64 = nullptr, *Dt64 = nullptr;
   float *B32 = nullptr, *Dc32 = nullptr, *Dt32 = nullptr;
-  float hB32[pff::kMaxQ * pff::kMaxQ] = {}, hDc32[pff::kMaxQ * pff::kMaxQ] = {};  // host copies (kernel parameters)
+  // B, D_t and D_c in FP32, each entry twice (kernel parameters)
+  unsigned long long hB2[pff::kMaxQ * pff::kMaxQ] = {}, hD2[pff::kMaxQ * pff::kMaxQ] = {},
+                     hDc2[pff::kMaxQ * pff::kMaxQ] = {};
   double hB[pff::kMaxQ * pff::kMaxQ] = {}, hDt[pff::kMaxQ * pff::kMaxQ] = {};
   pff::FixTab fix = {};  // the same for the FP64 kernels' fixed-point contractions
 };

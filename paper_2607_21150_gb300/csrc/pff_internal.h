@@ -77,9 +77,16 @@ template <int Q> __host__ __device__ constexpr int pipe_elem_words() {
 template <int Q> __host__ __device__ constexpr int pipe_elem_stride() {
   return pipe_elem_words<Q>() + ((Q * Q - pipe_elem_words<Q>()) % 32 + 32) % 32;
 }
+// The same stride in quads (one float4 of the four fields per node or point):
+// eight lanes share a 128-bit access, so it is Q^2 mod 8.
+template <int Q> __host__ __device__ constexpr int pipe_elem_quads() {
+  return (pipe_elem_stride<Q>() + 3) / 4 + ((Q * Q - (pipe_elem_stride<Q>() + 3) / 4) % 8 + 8) % 8;
+}
+// The collocated derivative of the persistent kernel.
+template <int Q> __host__ __device__ constexpr int pipe_mat_bytes() { return (4 * Q * Q + 15) / 16 * 16; }
 template <int P, int Q, bool BF, bool KX> __host__ __device__ constexpr int pipe_smem_bytes() {
-  return 2 * pipe_slot_bytes<Q, BF, KX>() + 16 +
-         4 * (mat_smem_words<P, Q>() + elems_per_block(Q) * pipe_elem_stride<Q>());
+  return 2 * pipe_slot_bytes<Q, BF, KX>() + 16 + pipe_mat_bytes<Q>() +
+         elems_per_block(Q) * 16 * pipe_elem_quads<Q>();
 }
 // Two resident blocks per SM: 228 KB of shared memory per SM, 1 KB reserved per block.
 template <int P, int Q, bool BF, bool KX> __host__ __device__ constexpr bool pipe_fits() {
@@ -214,10 +221,9 @@ struct ElemArgs {
   int blk0;               // first element block of the launch (actions; 0 = from the first)
   int ctas;               // FP32-arithmetic actions: resident blocks of the persistent kernel (0 = one per element block)
   int nblk;               // element blocks of the launch (actions; 0 = all blocks from blk0 = 0)
-  // FP32-arithmetic actions: the 1D matrices B [Q][P] and Dc [Q][Q] as kernel
-  // parameters, read as constant-bank operands where the index is fixed at compile time
-  float cB[kMaxQ * kMaxQ];
-  float cDc[kMaxQ * kMaxQ];
+  // FP32-arithmetic actions: the 1D matrices B [Q][P], its derivative D_t [Q][P]
+  // and D_c [Q][Q] as kernel parameters, each entry doubled (packed pairs of FP32)
+  unsigned long long cB2[kMaxQ * kMaxQ], cD2[kMaxQ * kMaxQ], cDc2[kMaxQ * kMaxQ];
   FixTab fix;             // FP64 kernels
 };
 
