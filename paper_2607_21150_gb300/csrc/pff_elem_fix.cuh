@@ -28,7 +28,7 @@
 // elements.  The 1D matrices are kernel parameters (constant-bank operands).
 //
 // Measured, 64^3 Q4 action: 20.08 ms with FP64 contractions (88.7 % of the FP64
-// pipe), 7.72 ms now; the map alone is 5.4 ms of that pipe (ncu, 24^3: pipe 69 %
+// pipe), 7.70 ms now; the map alone is 5.4 ms of that pipe (ncu, 24^3: pipe 69 %
 // busy, issue 52 %, DRAM 28 %).  With one thread per column of points (12 warps
 // per SM, as the FP64 kernel had it) 17 ms; with one copy of the line code per
 // direction instead of loops over the directions 9.1 ms (instruction cache).
@@ -174,14 +174,21 @@ k_elem_fix(const ElemArgs<double> a) {
   const bool node = valid && pt < P3;
   long long n = 0;
   if (MODE != kEval || node) n = node ? node_of<P, Q>(a.mesh, e, pt % P, (pt / P) % P, pt / P2) : 0;
-  double phi = 0.0;
+  // gather, and which entries are prescribed: bytes that only elements with
+  // masked nodes load, all of them at once, and that the scatter finds here
+  double phi = 0.0, xv[4] = {0.0, 0.0, 0.0, 0.0};
+  bool fixed[4] = {false, false, false, false};
+  if (MODE != kBack && node)
+#pragma unroll
+    for (int f = 0; f < 4; ++f) xv[f] = __ldg(a.x + f * nn + n);
+  if (masked && node)
+#pragma unroll
+    for (int f = 0; f < 4; ++f) fixed[f] = __ldg(a.mask + f * nn + n);
   if constexpr (MODE != kBack) {
-    // gather (prescribed entries zero) and the fields' exponents
-    double xv[4];
+    // prescribed entries zero; the fields' exponents
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-      xv[f] = node ? __ldg(a.x + f * nn + n) : 0.0;
-      if (node && masked && __ldg(a.mask + f * nn + n)) xv[f] = 0.0;
+      if (fixed[f]) xv[f] = 0.0;
       fx_max<Q>(&emax[el][f], fx_exponent(xv[f]));
     }
     __syncthreads();
@@ -348,7 +355,7 @@ k_elem_fix(const ElemArgs<double> a) {
     const double v = fx_to(A[f * Q3 + pt], sum_exponent(el, f) - 1022 - fx.wb, bad ? kFxNan : 0);
     if (a.evec)  // deterministic transpose: element-local values, summed per node by k_node_gather
       static_cast<double*>(a.evec)[((long long)e * 4 + f) * P3 + pt] = v;
-    else if (!(masked && __ldg(a.mask + f * nn + n)))
+    else if (!fixed[f])
       atomicAdd(a.y + f * nn + n, v);
   }
 }
