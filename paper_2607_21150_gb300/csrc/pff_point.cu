@@ -39,7 +39,35 @@
 
 namespace pff {
 
-__global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
+// A thread's arrays whose index is known only at run time, kept in shared memory
+// (slot n of thread t at n kPointThreads + t: no bank conflicts): the tangent's
+// dtau [10][6], dpsi [10] and the principal basis E [6][6].  As local arrays they
+// were 2.1 KB per thread, twice the L1 cache at two blocks per SM: half of
+// their accesses went to L2 and 1 KB per point to DRAM.  32^3 Q4 13.7 -> 12.1 ms,
+// 24^3 Q2 curved 2.35 -> 2.06 ms.  What is left is latency at eight warps per SM
+// (FP64 pipe 51 % busy, instruction fetch and dependent chains the rest); more
+// warps with fewer registers each spill: 15.5 ms with three blocks.
+constexpr int kPointThreads = 128, kPointSlots = 106;
+struct PointSlots {
+  double* p;
+  __device__ __forceinline__ double& d(int n) const { return p[n * kPointThreads]; }
+  __device__ __forceinline__ df64 get(int n) const {
+    const double v = d(n);
+    return df_make(__int_as_float(__double2hiint(v)), __int_as_float(__double2loint(v)));
+  }
+  __device__ __forceinline__ void put(int n, df64 v) const {
+    d(n) = __hiloint2double(__float_as_int(v.hi), __float_as_int(v.lo));
+  }
+  static __device__ __forceinline__ int dtau(int dir, int v) { return 6 * dir + v; }
+  static __device__ __forceinline__ int dpsi(int dir) { return 60 + dir; }
+  static __device__ __forceinline__ int E(int n, int v) { return 70 + 6 * n + v; }
+  // entry m of direction dir's column of dP, in the slots of its dtau and of E
+  static __device__ __forceinline__ int col(int dir, int m) { return m < 6 ? dtau(dir, m) : 70 + 3 * dir + m - 6; }
+};
+
+__global__ void __launch_bounds__(kPointThreads, 2) k_pointwise(const PointArgs a) {
+  extern __shared__ double point_sm[];  // [kPointSlots][kPointThreads]; no thread reads another's
+  const PointSlots sl{point_sm + threadIdx.x};
   const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (q >= a.nq) return;
   const int Q = a.Q, Q2 = Q * Q, Q3 = Q2 * Q;
@@ -113,17 +141,12 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
   double psid = 0.0;
   // the tangent's products and sums run in double-float on the FP32 pipes
   // (the FP64 pipe is this kernel's bound), converted by integer operations
-  df64 dtau[10][6];
-  df64 dpsi[10];
   df64 Fid[3][3];
-  const df64 dz = df_make(0.0f, 0.0f);
-  for (int d = 0; d < 10; ++d) {
-    dpsi[d] = dz;
-    for (int v = 0; v < 6; ++v) dtau[d][v] = dz;
-  }
-  if (a.want_tangent)
+  if (a.want_tangent) {
+    for (int n = 0; n < 70; ++n) sl.d(n) = 0.0;  // dtau, dpsi (both halves zero)
     for (int r = 0; r < 3; ++r)
       for (int c = 0; c < 3; ++c) Fid[r][c] = df_split(Fi[r][c]);
+  }
   uint8_t flag = 0;
   double dgam = 0.0;
   double hist_new[12];
@@ -232,16 +255,15 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
       }
       // symmetric basis of the principal frame in Voigt order: N dh N^T =
       // sum_p dh_pp n_p n_p^T + sum_{p<t} dh_pt (n_p n_t^T + n_t n_p^T)
-      df64 E[6][6];
       for (int v = 0; v < 6; ++v) {
         int r, c;
         vo_idx(v, r, c);
-        E[0][v] = df_mul(Nd[r][0], Nd[c][0]);
-        E[1][v] = df_mul(Nd[r][1], Nd[c][1]);
-        E[2][v] = df_mul(Nd[r][2], Nd[c][2]);
-        E[3][v] = df_madd(df_mul(Nd[r][1], Nd[c][2]), Nd[r][2], Nd[c][1]);
-        E[4][v] = df_madd(df_mul(Nd[r][0], Nd[c][2]), Nd[r][2], Nd[c][0]);
-        E[5][v] = df_madd(df_mul(Nd[r][0], Nd[c][1]), Nd[r][1], Nd[c][0]);
+        sl.put(sl.E(0, v), df_mul(Nd[r][0], Nd[c][0]));
+        sl.put(sl.E(1, v), df_mul(Nd[r][1], Nd[c][1]));
+        sl.put(sl.E(2, v), df_mul(Nd[r][2], Nd[c][2]));
+        sl.put(sl.E(3, v), df_madd(df_mul(Nd[r][1], Nd[c][2]), Nd[r][2], Nd[c][1]));
+        sl.put(sl.E(4, v), df_madd(df_mul(Nd[r][0], Nd[c][2]), Nd[r][2], Nd[c][0]));
+        sl.put(sl.E(5, v), df_madd(df_mul(Nd[r][0], Nd[c][1]), Nd[r][1], Nd[c][0]));
       }
       const df64 mud = df_split(mu), afd = df_split(af);
       const df64 mua = df_mul(mud, afd);
@@ -269,28 +291,29 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
       const df64 cphi = df_mul(df_add(mud, mud), df_split(da_dphi));  // phi direction: dh_q = 2 mu da_dphi ed_q
 #pragma unroll 1
       for (int v = 0; v < 6; ++v) {
-        df64 M[3][3];
+        df64 M[3][3], E[6];
+        for (int n = 0; n < 6; ++n) E[n] = sl.get(sl.E(n, v));
         for (int p = 0; p < 3; ++p)
-          M[p][p] = df_madd(df_madd(df_mul(cdiag[0][p], E[0][v]), cdiag[1][p], E[1][v]), cdiag[2][p], E[2][v]);
-        M[1][2] = df_mul(c12, E[3][v]);
-        M[2][1] = df_mul(c21, E[3][v]);
-        M[0][2] = df_mul(c02, E[4][v]);
-        M[2][0] = df_mul(c20, E[4][v]);
-        M[0][1] = df_mul(c01, E[5][v]);
-        M[1][0] = df_mul(c10, E[5][v]);
+          M[p][p] = df_madd(df_madd(df_mul(cdiag[0][p], E[0]), cdiag[1][p], E[1]), cdiag[2][p], E[2]);
+        M[1][2] = df_mul(c12, E[3]);
+        M[2][1] = df_mul(c21, E[3]);
+        M[0][2] = df_mul(c02, E[4]);
+        M[2][0] = df_mul(c20, E[4]);
+        M[0][1] = df_mul(c01, E[5]);
+        M[1][0] = df_mul(c10, E[5]);
         df64 T[3][3];  // N M
         for (int r = 0; r < 3; ++r)
           for (int c = 0; c < 3; ++c)
             T[r][c] = df_madd(df_madd(df_mul(Nd[r][0], M[0][c]), Nd[r][1], M[1][c]), Nd[r][2], M[2][c]);
         for (int aa = 0; aa < 3; ++aa)
           for (int BB = 0; BB < 3; ++BB) {
-            df64 acc = dtau[3 * aa + BB][v];
+            df64 acc = sl.get(sl.dtau(3 * aa + BB, v));
             acc = df_madd(acc, T[aa][0], Vd[BB][0]);
             acc = df_madd(acc, T[aa][1], Vd[BB][1]);
-            dtau[3 * aa + BB][v] = df_madd(acc, T[aa][2], Vd[BB][2]);
+            sl.put(sl.dtau(3 * aa + BB, v), df_madd(acc, T[aa][2], Vd[BB][2]));
           }
-        const df64 edE = df_madd(df_madd(df_mul(edd[0], E[0][v]), edd[1], E[1][v]), edd[2], E[2][v]);
-        dtau[9][v] = df_madd(dtau[9][v], cphi, edE);
+        const df64 edE = df_madd(df_madd(df_mul(edd[0], E[0]), edd[1], E[1]), edd[2], E[2]);
+        sl.put(sl.dtau(9, v), df_madd(sl.get(sl.dtau(9, v)), cphi, edE));
       }
       // energy: dpsi = 2 mu a^2 edde + 2 mu a s2 da = 2 mu a (a + cq) edde in the F-directions
       const df64 cpsi = df_mul(two_mua, df_add(afd, df_split(plastic ? cq : 0.0)));
@@ -300,9 +323,9 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
       for (int aa = 0; aa < 3; ++aa)
         for (int BB = 0; BB < 3; ++BB) {
           const df64 t = df_madd(df_madd(df_mul(Ne[aa][0], Vd[BB][0]), Ne[aa][1], Vd[BB][1]), Ne[aa][2], Vd[BB][2]);
-          dpsi[3 * aa + BB] = df_madd(dpsi[3 * aa + BB], cpsi, t);
+          sl.put(sl.dpsi(3 * aa + BB), df_madd(sl.get(sl.dpsi(3 * aa + BB)), cpsi, t));
         }
-      dpsi[9] = df_madd(dpsi[9], df_mul(two_mua, df_split(s2)), df_split(da_dphi));
+      sl.put(sl.dpsi(9), df_madd(sl.get(sl.dpsi(9)), df_mul(two_mua, df_split(s2)), df_split(da_dphi)));
     }
   }
 
@@ -375,8 +398,8 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
     double* lin = a.lin + blk * (long long)kLinWords * stride + (long long)qk * Q2 * EB + el * Q2 + qj * Q + qi;
     const double app = (gl.at == 1) ? 0.0 : 2.0;
     const double cL = 2.0 * Hh + ph.gc_c0l0 * app + gl.zdt;
-    // mapped mesh: reference-frame columns kept, transformed to the parent frame below
-    double Dm[9][9], Pv[9], Lv[9], Lphi = 0.0;
+    // mapped mesh: reference-frame columns kept (in the slots of their direction),
+    // transformed to the parent frame below
     // double-float copies of the point's scalars and matrices
     const df64 gd = df_split(g), gpd = df_split(gp), tvd = df_split(tv), kapd = df_split(ph.kap_tot);
     const df64 kth = df_mul(kapd, df_split(theta)), cLd = df_split(cL);
@@ -410,7 +433,7 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
       for (int v = 0; v < 6; ++v) {
         int r, c;
         vo_idx(v, r, c);
-        df64 val = df_mul(gd, dtau[d][v]);
+        df64 val = df_mul(gd, sl.get(sl.dtau(d, v)));
         if (dphi) val = df_madd(val, gpd, taudd[v]);
         if (r == c) {
           if (tens) {
@@ -422,7 +445,8 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
         }
         M[r][c] = val; M[c][r] = val;
       }
-      const df64 dpsip = tens ? df_madd(dpsi[d], kth, trl) : dpsi[d];
+      const df64 dps = sl.get(sl.dpsi(d));
+      const df64 dpsip = tens ? df_madd(dps, kth, trl) : dps;
       if (d < 9)  // geometric term: - tau_degr ell^T, (tau ell^T)_{i aa} = (tau F^-T e_BB)_i
         for (int r = 0; r < 3; ++r) M[r][aa] = df_sub(M[r][aa], TF[r][BB]);
       df64 dP[3][3];
@@ -432,13 +456,8 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
       df64 dL = active ? df_mul(gpd, dpsip) : df_make(0.0f, 0.0f);
       if (dphi) dL = df_add(dL, cLd);
       if (mapped) {
-        if (d < 9) {
-          for (int m = 0; m < 9; ++m) Dm[m][d] = df_join(dP[m / 3][m % 3]);
-          Lv[d] = df_join(dL);
-        } else {
-          for (int m = 0; m < 9; ++m) Pv[m] = df_join(dP[m / 3][m % 3]);
-          Lphi = df_join(dL);
-        }
+        for (int m = 0; m < 9; ++m) sl.d(sl.col(d, m)) = df_join(dP[m / 3][m % 3]);
+        sl.d(sl.dpsi(d)) = df_join(dL);
       } else if (d < 9) {
         const int n = 3 * aa + BB;
         for (int m = 0; m <= n; ++m) {
@@ -456,25 +475,28 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
       for (int pr = 0; pr < 3; ++pr) lin[(long long)(kWKX + pr) * stride] = 0.0;
     } else {
       // parent frame: A_hat[(r, al), (c, be)] = w det J sum_{A,B} G[al][A] D[(r, A), (c, B)] G[be][B]
-      double T[9][9];
       for (int m = 0; m < 9; ++m)
-        for (int c = 0; c < 3; ++c)
-          for (int be = 0; be < 3; ++be)
-            T[m][3 * c + be] = Dm[m][3 * c] * Gx[be][0] + Dm[m][3 * c + 1] * Gx[be][1] + Dm[m][3 * c + 2] * Gx[be][2];
+        for (int c = 0; c < 3; ++c) {
+          const double d0 = sl.d(sl.col(3 * c, m)), d1 = sl.d(sl.col(3 * c + 1, m)), d2 = sl.d(sl.col(3 * c + 2, m));
+          for (int be = 0; be < 3; ++be) sl.d(sl.col(3 * c + be, m)) = d0 * Gx[be][0] + d1 * Gx[be][1] + d2 * Gx[be][2];
+        }
       for (int n = 0; n < 9; ++n)
         for (int m = 0; m <= n; ++m) {
           const int r = m / 3, al = m % 3;
-          const double v = Gx[al][0] * T[3 * r][n] + Gx[al][1] * T[3 * r + 1][n] + Gx[al][2] * T[3 * r + 2][n];
+          const double v = Gx[al][0] * sl.d(sl.col(n, 3 * r)) + Gx[al][1] * sl.d(sl.col(n, 3 * r + 1)) +
+                           Gx[al][2] * sl.d(sl.col(n, 3 * r + 2));
           lin[(long long)(kWA + sym9(m, n)) * stride] = wdet * v;
         }
       for (int r = 0; r < 3; ++r)
         for (int al = 0; al < 3; ++al) {
           lin[(long long)(kWP + 3 * r + al) * stride] =
-              wdet * (Gx[al][0] * Pv[3 * r] + Gx[al][1] * Pv[3 * r + 1] + Gx[al][2] * Pv[3 * r + 2]);
+              wdet * (Gx[al][0] * sl.d(sl.col(9, 3 * r)) + Gx[al][1] * sl.d(sl.col(9, 3 * r + 1)) +
+                      Gx[al][2] * sl.d(sl.col(9, 3 * r + 2)));
           lin[(long long)(kWC + 3 * r + al) * stride] =
-              wdet * gl.s_phi * (Gx[al][0] * Lv[3 * r] + Gx[al][1] * Lv[3 * r + 1] + Gx[al][2] * Lv[3 * r + 2]);
+              wdet * gl.s_phi * (Gx[al][0] * sl.d(sl.dpsi(3 * r)) + Gx[al][1] * sl.d(sl.dpsi(3 * r + 1)) +
+                                 Gx[al][2] * sl.d(sl.dpsi(3 * r + 2)));
         }
-      lin[(long long)kWD * stride] = wdet * gl.s_phi * Lphi;
+      lin[(long long)kWD * stride] = wdet * gl.s_phi * sl.d(sl.dpsi(9));
       double K[3][3];
       for (int al = 0; al < 3; ++al)
         for (int be = 0; be < 3; ++be)
@@ -490,8 +512,12 @@ __global__ void __launch_bounds__(128) k_pointwise(const PointArgs a) {
 
 cudaError_t launch_pointwise(const PointArgs& a, cudaStream_t st) {
   if (a.nq == 0) return cudaSuccess;
-  long long nb = (a.nq + 127) / 128;
-  k_pointwise<<<(unsigned)nb, 128, 0, st>>>(a); note_launch();
+  const long long nb = (a.nq + kPointThreads - 1) / kPointThreads;
+  const int smem = a.want_tangent ? kPointSlots * kPointThreads * (int)sizeof(double) : 0;
+  const cudaError_t rc = cudaFuncSetAttribute(k_pointwise, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              kPointSlots * kPointThreads * (int)sizeof(double));
+  if (rc != cudaSuccess) return rc;
+  k_pointwise<<<(unsigned)nb, kPointThreads, smem, st>>>(a); note_launch();
   return cudaGetLastError();
 }
 
