@@ -4,7 +4,7 @@
 //
 // * Outer: Newton on the FP64 residual with a backtracking line search; each
 //   linear solve is FGMRES(m) with FP64 vectors and inner products, its
-//   operator the FP64 or the double-float fine action (outer_prec), right-
+//   operator the FP64 fine action (outer_prec), right-
 //   preconditioned by one V-cycle (flexible because the coarse solve and the
 //   mixed-precision cycle are not exactly linear in FP64).
 // * V-cycle: Chebyshev(k) pre- and post-smoothing on D^-1 J of every

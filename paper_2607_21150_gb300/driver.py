@@ -80,9 +80,8 @@ class StepController:
 class LoadStepper:
     def __init__(self, w: Workload, levels=None, mixed: bool = True, session: Session | None = None,
                  df: bool | None = None, max_cuts: int = 6, grow_after: int = 1, **solver_params):
-        """df: the fine-level action inside FGMRES in double-float arithmetic
-        (PFF_DF64) instead of FP64; by default on with mixed precision (same
-        converged fields to ~1e-15, half the time of the FP64 action).
+        """df: the fine-level action inside FGMRES by PFF_DF64 (served by the
+        FP64 action); by default on with mixed precision.
         max_cuts: consecutive halvings of a failing load increment before
         `advance` gives up; grow_after: successes in a row before a cut
         increment grows again (StepController).  solver_params: fields of pff_solver_params, e.g.
