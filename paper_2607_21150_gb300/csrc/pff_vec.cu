@@ -22,28 +22,52 @@ static unsigned grid_for(long long n) {
 // mode 0: y = mask ? x : 0      (Jacobian action: identity rows of Dirichlet DoFs)
 // mode 1: y = mask ? x - u : 0  (residual: z - ubar on Dirichlet DoFs)
 // mode 2: y = mask ? 1 : 0      (diagonal)
-template <typename T>
+// Bound by the store of y (x is read where masked only).  V entries per thread:
+// FP32 takes four where n is a multiple of four and the addresses allow 16-byte
+// stores and 4-byte mask loads (every vector from its allocation's start): 3.7 M
+// entries 12.3 -> 6.2 us, 17 M 28 -> 20 us.  FP64 goes one by one: with four,
+// 68 M entries took 103 us instead of 101.
+template <typename T, int V>
 __global__ void k_init_masked(T* __restrict__ y, const T* __restrict__ x, const double* __restrict__ ubar,
                               const uint8_t* __restrict__ mask, long long n, int mode) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    bool m = mask && mask[i];
-    T v = T(0);
-    if (m) {
-      if (mode == 0) v = x[i];
-      else if (mode == 1) v = x[i] - (ubar ? (T)ubar[i] : T(0));
-      else v = T(1);
+  struct alignas(V * sizeof(T)) Out { T v[V]; };
+  const long long nv = n / V;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nv; i += (long long)gridDim.x * blockDim.x) {
+    unsigned m = 0;  // V mask bytes
+    if (mask) m = V == 4 ? *reinterpret_cast<const unsigned*>(mask + 4 * i) : mask[i];
+    Out o;
+#pragma unroll
+    for (int c = 0; c < V; ++c) {
+      T v = T(0);
+      if (m >> (8 * c) & 255u) {
+        const long long k = i * V + c;
+        if (mode == 0) v = x[k];
+        else if (mode == 1) v = x[k] - (ubar ? (T)ubar[k] : T(0));
+        else v = T(1);
+      }
+      o.v[c] = v;
     }
-    y[i] = v;
+    *reinterpret_cast<Out*>(y + i * V) = o;
   }
+}
+
+template <typename T>
+static void init_masked(T* y, const T* x, const double* ubar, const uint8_t* mask, long long n, int mode,
+                        cudaStream_t st) {
+  if constexpr (sizeof(T) == 4) {
+    if (n % 4 == 0 && (reinterpret_cast<uintptr_t>(y) & 15) == 0 && (reinterpret_cast<uintptr_t>(mask) & 3) == 0) {
+      k_init_masked<T, 4><<<grid_for(n / 4), kVecThreads, 0, st>>>(y, x, ubar, mask, n, mode);
+      return;
+    }
+  }
+  k_init_masked<T, 1><<<grid_for(n), kVecThreads, 0, st>>>(y, x, ubar, mask, n, mode);
 }
 
 cudaError_t launch_init_masked(int prec, void* y, const void* x, const double* ubar, const uint8_t* mask,
                                long long n, int mode, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  if (prec == 0)
-    k_init_masked<double><<<grid_for(n), kVecThreads, 0, st>>>((double*)y, (const double*)x, ubar, mask, n, mode);
-  else
-    k_init_masked<float><<<grid_for(n), kVecThreads, 0, st>>>((float*)y, (const float*)x, ubar, mask, n, mode);
+  if (prec == 0) init_masked((double*)y, (const double*)x, ubar, mask, n, mode, st);
+  else init_masked((float*)y, (const float*)x, ubar, mask, n, mode, st);
   note_launch();
   return cudaGetLastError();
 }

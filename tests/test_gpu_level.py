@@ -57,3 +57,28 @@ def test_level_actions_follow_fp64(p, mapped, scattered):
                         assert e <= tol, (pl, transpose, prec, offsets, det, e)
         assert s.status() == 0
         s.close()
+
+
+@pytest.mark.parametrize("offset", [0, 1, 2, 3])
+@pytest.mark.parametrize("prec", ["f64", "f32", "bf16"])
+def test_output_at_any_entry(prec, offset):
+    """y may start at any entry of an allocation: masked rows are x bit for bit,
+    the others the aligned action up to the order of the additions."""
+    w = _workload(3, True, True)
+    s = Session(w, f32=True, bf16=True)
+    s.residual(w.z)
+    code = {"f64": pff.PFF_F64, "f32": pff.PFF_F32, "bf16": pff.PFF_F32_BF16}[prec]
+    dt = torch.float64 if prec == "f64" else torch.float32
+    n = w.mesh.ndof
+    x = torch.from_numpy(inputs.random_vector(n, 3)).cuda().to(dt)
+    ref = s.apply(x, prec=code)
+    buf = torch.full((n + 8,), 7.0, dtype=dt, device="cuda")
+    y = buf[offset:offset + n]
+    pff.pff_jacobian_apply(s.levels[3], code, x, y, s.stream)
+    m = torch.from_numpy(w.mask.astype(bool)).cuda()
+    assert torch.equal(y[m], x[m])
+    # at most eight additions per row, in any order
+    tol = 8 * torch.finfo(dt).eps
+    assert ((y - ref).norm() <= tol * ref.norm()).item()
+    assert (buf[:offset] == 7.0).all() and (buf[offset + n:] == 7.0).all()
+    s.close()
