@@ -121,9 +121,11 @@ constexpr int kFxNan = 0x7ff80000;
 // *m = max(*m, v) over the threads of an element: by warp where a warp holds one
 // element only (Q >= 4), so that the shared atomics do not queue up (for Q = 3 a
 // reduction over the lanes of each element measured slower than the atomics).
-template <int Q> __device__ __forceinline__ void fx_max(int* m, int v) {
+// Every thread of the block calls it; the lanes are named, not those that happen
+// to be together after the branches before it, so that lane 0 has all of them.
+template <int Q, int THREADS> __device__ __forceinline__ void fx_max(int* m, int v) {
   if (Q >= 4) {
-    v = __reduce_max_sync(__activemask(), v);
+    v = __reduce_max_sync(warp_lanes(THREADS, threadIdx.x / 32), v);
     if ((threadIdx.x & 31) == 0) atomicMax(m, v);
   } else {
     atomicMax(m, v);
@@ -134,12 +136,6 @@ template <int Q> __device__ __forceinline__ void fx_max(int* m, int v) {
 // y-derivatives, or a ping-pong buffer of the contractions); C, Q^3 (the value
 // term of the phase field).
 template <int Q> __host__ __device__ constexpr int fix_elem_words() { return 13 * Q * Q * Q; }
-// Elements per block.  Q = 3: seven, whose 252 lines fill 189 threads better
-// (24x25x23 elements: 113.7 us, with four 123.4), but four on meshes too small to
-// give every SM two such blocks (4^3: 18.9 us, with seven 22.8).
-__host__ __device__ constexpr int fix_elems(int Q, bool small) {
-  return Q == 5 ? 1 : Q == 4 ? 2 : Q == 3 ? (small ? 4 : 7) : 16;
-}
 // Resident blocks the register allocation is held to: about 30 warps per SM
 // (40x33x37 elements, 20 / 24 / 30 / 36 warps: Q2 376 / 335 / 316 / 326 us, Q3 - /
 // 657 / 645 / 681 us, Q4 - / 1493 / 1495 / 1564 us).
@@ -151,6 +147,7 @@ k_elem_fix(const ElemArgs<double> a) {
   constexpr int EB = elems_per_block(Q), NSUB = EB / EBS;
   constexpr int Q2 = Q * Q, Q3 = Q * Q * Q, P2 = P * P, P3 = P * P * P;
   static_assert(NSUB * EBS == EB, "a block's elements divide the group");
+  static_assert(Q < 4 || Q3 % 32 == 0 || EBS == 1, "fx_max: one element per warp");
   __shared__ long long sm[EBS * fix_elem_words<Q>()];
   __shared__ int emax[EBS][12];  // exponents: x per field, [4..7] gradient outputs, [8] value output
   constexpr int NT = Q3 * EBS;
@@ -189,7 +186,7 @@ k_elem_fix(const ElemArgs<double> a) {
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
       if (fixed[f]) xv[f] = 0.0;
-      fx_max<Q>(&emax[el][f], fx_exponent(xv[f]));
+      fx_max<Q, NT>(&emax[el][f], fx_exponent(xv[f]));
     }
     __syncthreads();
     if (pt < P3)
@@ -286,10 +283,10 @@ k_elem_fix(const ElemArgs<double> a) {
         B[2 * f * Q3 + pt] = __double_as_longlong(o[f][0]);
         B[(2 * f + 1) * Q3 + pt] = __double_as_longlong(o[f][1]);
         A[f * Q3 + pt] = __double_as_longlong(o[f][2]);
-        fx_max<Q>(&emax[el][4 + f], max(fx_exponent(o[f][0]), max(fx_exponent(o[f][1]), fx_exponent(o[f][2]))));
+        fx_max<Q, NT>(&emax[el][4 + f], max(fx_exponent(o[f][0]), max(fx_exponent(o[f][1]), fx_exponent(o[f][2]))));
       }
       C[pt] = v0;
-      fx_max<Q>(&emax[el][8], fx_exponent(v0));
+      fx_max<Q, NT>(&emax[el][8], fx_exponent(v0));
     }
   }
   __syncthreads();

@@ -49,6 +49,18 @@ static_assert((2 * 2 * 2 * elems_per_block(2)) % 2 == 0 && (3 * 3 * 3 * elems_pe
               (4 * 4 * 4 * elems_per_block(4)) % 2 == 0 && (5 * 5 * 5 * elems_per_block(5)) % 2 == 0,
               "FP32 quad layout needs Q^3 EB even");
 
+// Elements per block of the FP64 element kernels (pff_elem_fix.cuh).  Q = 3: seven,
+// whose 252 lines fill 189 threads better (24x25x23 elements: 113.7 us, with four
+// 123.4), but four on meshes too small to give every SM two such blocks (4^3:
+// 18.9 us, with seven 22.8).
+__host__ __device__ constexpr int fix_elems(int Q, bool small) {
+  return Q == 5 ? 1 : Q == 4 ? 2 : Q == 3 ? (small ? 4 : 7) : 16;
+}
+// Lanes of a block's warp that hold threads.
+__host__ __device__ constexpr unsigned warp_lanes(int threads, int warp) {
+  return threads - 32 * warp >= 32 ? 0xffffffffu : (1u << (threads - 32 * warp)) - 1u;
+}
+
 // Shared-memory words of the 1D matrices in an element kernel (B, D_t, and
 // the collocated derivative D_c; the persistent kernel keeps B and D_c).
 template <int P, int Q> __host__ __device__ constexpr int mat_smem_words() { return 3 * Q * P + Q * Q; }
