@@ -604,8 +604,7 @@ int pff_set_dirichlet(pff_op* op, const uint8_t* mask, const double* values, voi
   long long n = 4 * op->mesh.nn;
   if (!mask) {
     cudaFree(op->mask); op->mask = nullptr;
-    cudaFree(op->emask);
-  cudaFree(op->evec); op->emask = nullptr;
+    cudaFree(op->emask); op->emask = nullptr;
     cudaFree(op->dvals); op->dvals = nullptr;
     return PFF_OK;
   }
