@@ -121,11 +121,13 @@ constexpr int kFxNan = 0x7ff80000;
 // *m = max(*m, v) over the threads of an element: by warp where a warp holds one
 // element only (Q >= 4), so that the shared atomics do not queue up (for Q = 3 a
 // reduction over the lanes of each element measured slower than the atomics).
-// Every thread of the block calls it; the lanes are named, not those that happen
-// to be together after the branches before it, so that lane 0 has all of them.
-template <int Q, int THREADS> __device__ __forceinline__ void fx_max(int* m, int v) {
+// Every thread of the block calls it, and those warps are full (fix_threads): all
+// lanes are named, so that lane 0 has the whole warp's maximum whatever branches
+// went before.  With 29 lanes in the last warp of Q = 5 and their mask here,
+// 64^3 Q4 took 7.95 ms instead of 7.72.
+template <int Q> __device__ __forceinline__ void fx_max(int* m, int v) {
   if (Q >= 4) {
-    v = __reduce_max_sync(warp_lanes(THREADS, threadIdx.x / 32), v);
+    v = __reduce_max_sync(0xffffffffu, v);
     if ((threadIdx.x & 31) == 0) atomicMax(m, v);
   } else {
     atomicMax(m, v);
@@ -142,7 +144,7 @@ template <int Q> __host__ __device__ constexpr int fix_elem_words() { return 13 
 __host__ __device__ constexpr int fix_blocks(int threads) { return 30 / ((threads + 31) / 32); }
 
 template <int P, int Q, int MODE, int EBS>
-__global__ void __launch_bounds__(Q * Q * Q * EBS, fix_blocks(Q * Q * Q * EBS))
+__global__ void __launch_bounds__(fix_threads(Q, EBS), fix_blocks(fix_threads(Q, EBS)))
 k_elem_fix(const ElemArgs<double> a) {
   constexpr int EB = elems_per_block(Q), NSUB = EB / EBS;
   constexpr int Q2 = Q * Q, Q3 = Q * Q * Q, P2 = P * P, P3 = P * P * P;
@@ -150,13 +152,14 @@ k_elem_fix(const ElemArgs<double> a) {
   static_assert(Q < 4 || Q3 % 32 == 0 || EBS == 1, "fx_max: one element per warp");
   __shared__ long long sm[EBS * fix_elem_words<Q>()];
   __shared__ int emax[EBS][12];  // exponents: x per field, [4..7] gradient outputs, [8] value output
-  constexpr int NT = Q3 * EBS;
+  constexpr int NT = fix_threads(Q, EBS);
   const int t = threadIdx.x;
-  const int el = t / Q3, pt = t % Q3;  // element, and node or point of it
+  const bool live = NT == Q3 * EBS || t < Q3 * EBS;  // the others fill the last warp of Q = 5
+  const int el = EBS == 1 ? 0 : t / Q3, pt = EBS == 1 ? t : t % Q3;  // element, and node or point of it
   const long long grp = a.blk0 + blockIdx.x / NSUB;
   const int sub = blockIdx.x % NSUB;
   const int e = (int)(grp * EB) + sub * EBS + el;
-  const bool valid = e < a.mesh.nel;
+  const bool valid = live && e < a.mesh.nel;
   const long long nn = a.mesh.nn;
   const FixTab& fx = a.fix;
   const int dd = 60 - fx.sD;
@@ -186,7 +189,7 @@ k_elem_fix(const ElemArgs<double> a) {
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
       if (fixed[f]) xv[f] = 0.0;
-      fx_max<Q, NT>(&emax[el][f], fx_exponent(xv[f]));
+      fx_max<Q>(&emax[el][f], fx_exponent(xv[f]));
     }
     __syncthreads();
     if (pt < P3)
@@ -280,13 +283,15 @@ k_elem_fix(const ElemArgs<double> a) {
       }
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
-        B[2 * f * Q3 + pt] = __double_as_longlong(o[f][0]);
-        B[(2 * f + 1) * Q3 + pt] = __double_as_longlong(o[f][1]);
-        A[f * Q3 + pt] = __double_as_longlong(o[f][2]);
-        fx_max<Q, NT>(&emax[el][4 + f], max(fx_exponent(o[f][0]), max(fx_exponent(o[f][1]), fx_exponent(o[f][2]))));
+        if (live) {
+          B[2 * f * Q3 + pt] = __double_as_longlong(o[f][0]);
+          B[(2 * f + 1) * Q3 + pt] = __double_as_longlong(o[f][1]);
+          A[f * Q3 + pt] = __double_as_longlong(o[f][2]);
+        }
+        fx_max<Q>(&emax[el][4 + f], max(fx_exponent(o[f][0]), max(fx_exponent(o[f][1]), fx_exponent(o[f][2]))));
       }
-      C[pt] = v0;
-      fx_max<Q, NT>(&emax[el][8], fx_exponent(v0));
+      if (live) C[pt] = v0;
+      fx_max<Q>(&emax[el][8], fx_exponent(v0));
     }
   }
   __syncthreads();
@@ -359,7 +364,7 @@ k_elem_fix(const ElemArgs<double> a) {
 
 template <int P, int Q, int MODE, int EBS>
 cudaError_t launch_fix(const ElemArgs<double>& a, int nblk, cudaStream_t st) {
-  k_elem_fix<P, Q, MODE, EBS><<<(unsigned)nblk * (elems_per_block(Q) / EBS), Q * Q * Q * EBS, 0, st>>>(a); note_launch();
+  k_elem_fix<P, Q, MODE, EBS><<<(unsigned)nblk * (elems_per_block(Q) / EBS), fix_threads(Q, EBS), 0, st>>>(a); note_launch();
   return cudaGetLastError();
 }
 template <int P, int Q, int MODE>

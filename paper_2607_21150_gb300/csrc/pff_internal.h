@@ -56,9 +56,9 @@ static_assert((2 * 2 * 2 * elems_per_block(2)) % 2 == 0 && (3 * 3 * 3 * elems_pe
 __host__ __device__ constexpr int fix_elems(int Q, bool small) {
   return Q == 5 ? 1 : Q == 4 ? 2 : Q == 3 ? (small ? 4 : 7) : 16;
 }
-// Lanes of a block's warp that hold threads.
-__host__ __device__ constexpr unsigned warp_lanes(int threads, int warp) {
-  return threads - 32 * warp >= 32 ? 0xffffffffu : (1u << (threads - 32 * warp)) - 1u;
+// Their threads: one per point, in whole warps where warps reduce (Q >= 4).
+__host__ __device__ constexpr int fix_threads(int Q, int elems) {
+  return Q >= 4 ? (Q * Q * Q * elems + 31) / 32 * 32 : Q * Q * Q * elems;
 }
 
 // Shared-memory words of the 1D matrices in an element kernel (B, D_t, and

@@ -1,13 +1,13 @@
 """Lanes that take part in the warp reductions of the element kernels (no GPU).
 
 A warp intrinsic with a lane mask waits for exactly the lanes of its mask, so the
-mask has to name the threads of the block, all of them: a mask taken from the
-lanes that are together by chance (the active mask) may leave some out after a
-branch, and their part of the result is lost without a sign.
+mask has to name all threads of the warp: a mask taken from the lanes that are
+together by chance (the active mask) may leave some out after a branch, and their
+part of the result is lost without a sign.
 
 * no kernel derives a mask from the active lanes;
-* warp_lanes names the lanes of every warp that hold threads, for the block sizes
-  of the FP64 element kernels, and a warp that reduces holds one element only.
+* the blocks of the FP64 element kernels whose warps reduce (Q >= 4) consist of
+  full warps, and the points of a warp belong to one element.
 """
 import glob
 import os
@@ -26,16 +26,11 @@ int main() {
   int bad = 0;
   for (int Q = 4; Q <= 5; ++Q)
     for (int small = 0; small < 2; ++small) {
-      const int q3 = Q * Q * Q, threads = q3 * fix_elems(Q, small != 0);
-      for (int warp = 0; 32 * warp < threads; ++warp) {
-        const unsigned m = warp_lanes(threads, warp);
-        if (!(m & 1u)) { std::printf("Q=%d warp %d without lane 0\n", Q, warp); ++bad; }
-        for (int lane = 0; lane < 32; ++lane) {
-          const int t = 32 * warp + lane;
-          if (((m >> lane & 1u) != 0) != (t < threads)) { std::printf("Q=%d thread %d\n", Q, t); ++bad; }
-          if (t < threads && t / q3 != 32 * warp / q3) { std::printf("Q=%d warp %d holds two elements\n", Q, warp); ++bad; }
-        }
-      }
+      const int q3 = Q * Q * Q, elems = fix_elems(Q, small != 0), threads = fix_threads(Q, elems);
+      if (threads % 32) { std::printf("Q=%d: the last warp is not full\n", Q); ++bad; }
+      if (threads < q3 * elems) { std::printf("Q=%d: points without a thread\n", Q); ++bad; }
+      for (int t = 0; t < q3 * elems; ++t)
+        if (t / q3 != t / 32 * 32 / q3) { std::printf("Q=%d warp %d holds two elements\n", Q, t / 32); ++bad; }
     }
   std::printf(bad ? "FAIL\n" : "OK\n");
   return bad ? 1 : 0;
