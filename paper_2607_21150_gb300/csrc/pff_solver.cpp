@@ -429,13 +429,16 @@ int power_coarse(pff_solver* s, cudaStream_t st) {
 // Gram-Schmidt with a second pass when the first one loses accuracy (the
 // adaptive CGS refinement of Sec. 5).  V: (m+1) n, Z: m n device doubles.
 // sc, slot: its three sets of dot scalars on the device and in host memory (an
-// inner solve runs between an outer one's and must not share them).
+// inner solve runs between an outer one's and must not share them).  late: the
+// host learns ||b|| with the first Hessenberg column only, which saves an inner
+// solve a wait per call; a zero b then costs one preconditioner and one product.
 struct Krylov {
   long long n = 0;
   int m = 0;
   double *V = nullptr, *Z = nullptr;
   DotScalars* sc = nullptr;
   int slot = 0;
+  bool late = false;
 };
 
 template <typename ApplyA, typename ApplyM>
@@ -454,8 +457,7 @@ int gmres_flex(pff_solver* s, const Krylov& kw, ApplyA&& applyA, ApplyM&& applyM
       S_RC(applyA(x, v0));
       S_CK(launch_bminus<double>(v0, b, n, st));
     }
-    // ||r|| and v0 = r / ||r|| on the device; the host learns the norm with the
-    // first Hessenberg column, except where it may end the iteration
+    // ||r|| and v0 = r / ||r|| on the device
     const double* r0 = first ? b : v0;
     unsigned long long seq_b = 0;
     S_RC(dots(s, r0, 0, 1, r0, n, 0, nullptr, kw.sc, kw.slot, &seq_b, st));
@@ -468,7 +470,7 @@ int gmres_flex(pff_solver* s, const Krylov& kw, ApplyA&& applyA, ApplyM&& applyM
       known = true;
       return PFF_OK;
     };
-    if (!first || !(rtol < 1.0) || total >= maxit) {
+    if (!first || !kw.late || !(rtol < 1.0) || total >= maxit) {
       S_RC(read_beta());
       if (beta == 0.0 || beta0 == 0.0) { res = 0.0; break; }
       res = beta;
@@ -476,7 +478,7 @@ int gmres_flex(pff_solver* s, const Krylov& kw, ApplyA&& applyA, ApplyM&& applyM
     }
     S_CK(launch_normalise(v0, r0, kw.sc, n, st));
     int jend = 0;
-    bool zero = false;
+    bool ended = false;
     for (int j = 0; j < m && total < maxit; ++j) {
       double* vj = kw.V + (long long)j * n;
       double* zj = kw.Z + (long long)j * n;
@@ -485,7 +487,7 @@ int gmres_flex(pff_solver* s, const Krylov& kw, ApplyA&& applyA, ApplyM&& applyM
       S_RC(applyA(zj, w));
       if (!known) {
         S_RC(read_beta());
-        if (beta == 0.0) { zero = true; break; }
+        if (beta <= rtol * beta0) { ended = true; break; }  // zero, or a square beyond FP64: x = 0
       }
       if (j == 0) {
         std::fill(g.begin(), g.end(), 0.0);
@@ -529,7 +531,7 @@ int gmres_flex(pff_solver* s, const Krylov& kw, ApplyA&& applyA, ApplyM&& applyM
       res = std::fabs(g[j + 1]);
       if (res <= rtol * beta0 || hn == 0.0) break;
     }
-    if (zero) { res = 0.0; break; }
+    if (ended) { res = beta; break; }
     LinCoef y;
     for (int i = jend - 1; i >= 0; --i) {
       double sum = g[i];
@@ -595,6 +597,7 @@ int coarse_gmres(pff_solver* s, cudaStream_t st) {
   kw.Z = s->cZ;
   kw.sc = s->sc + 3;
   kw.slot = 3;
+  kw.late = true;
   auto A = [&](const double* in, double* out) -> int { return h_spmv(s, lev, in, out, st); };
   auto M = [&](const double* in, double* out) -> int {
     if (s->prm.coarse_solver == 2) return hcycle_top(s, in, out, st);
