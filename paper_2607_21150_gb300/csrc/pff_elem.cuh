@@ -444,6 +444,14 @@ k_elem(const ElemArgs<float> a) {
 // field is contracted.  Term by term, as before, a block passed 66 barriers and
 // waited for each term's words: 290 us at 24x24x72 Q3 FP32, 113 us now (the
 // quads that hold the words are 456 MB, 68 us at the copy rate).
+//
+// In FP64 the pipe binds (16 clocks per warp instruction and SM), so that idle
+// lanes and products with zeros count: there the lines of the y and x stages are
+// spread over the block's warps (at order 1 and Q4 half and a quarter of an
+// element's threads have one), and the terms that a field does not have are left
+// out (the value term of a displacement, the mixed terms of the phase field on a
+// box).  41x40x37 Q3, FP64: order 1 1155 -> 685 us, order 3 2206 -> 1919 us (term
+// by term 973 and 2339 us).  In FP32 an element's threads keep their own lines.
 constexpr int kDiagTerms = 6;
 // Words of field f at the thread's points, one value per term (f = 3: term 5
 // gets the value word besides, in v).
@@ -516,14 +524,15 @@ __global__ void __launch_bounds__(Q * Q * elems_per_block(Q), 2)
 k_diag(const ElemArgs<T> a, const DiagMats<T, P, Q> mats) {
   constexpr int EB = elems_per_block(Q);
   constexpr int Q2 = Q * Q, P3 = P * P * P;
+  constexpr bool kPipe64 = sizeof(T) == 8;  // bound by the FP64 pipe
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sm = reinterpret_cast<T*>(smem_raw);
   const int t = threadIdx.x;
   const int el = t / Q2, ij = t % Q2;
   const int e = (a.blk0 + blockIdx.x) * EB + el;
   const bool valid = e < a.mesh.nel;
-  T* Zb = sm + el * diag_smem_words<P, Q>();  // [term][c][j][i], then [c][b][a]
-  T* Yb = Zb + kDiagTerms * P * Q2;                                     // [kx][c][b][i]
+  constexpr int W = diag_smem_words<P, Q>(), NT = Q2 * EB;
+  T* Zb = sm + el * W;  // [term][c][j][i], then [c][b][a]; behind it Yb [kx][c][b][i]
   const bool masked = a.mask && valid && (!a.emask || a.emask[e]);
   const long long nn = a.mesh.nn;
   // kinds of the terms 00, 01, 02, 11, 12, 22
@@ -532,14 +541,16 @@ k_diag(const ElemArgs<T> a, const DiagMats<T, P, Q> mats) {
   diag_words<Q, T>(a, 0, t, valid, w, v);
 #pragma unroll 1
   for (int f = 0; f < 4; ++f) {
+    auto absent = [&](int m) { return kPipe64 && f == 3 && !a.kx && (m == 1 || m == 2 || m == 4); };
 #pragma unroll
     for (int c = 0; c < P; ++c)
 #pragma unroll
       for (int m = 0; m < kDiagTerms; ++m) {
+        if (absent(m)) continue;
         T s = T(0);
 #pragma unroll
         for (int k = 0; k < Q; ++k) s += mats.m[(KZ[m] * Q + k) * P + c] * w[m][k];
-        if (m == 5) {
+        if (m == 5 && (!kPipe64 || f == 3)) {
           T u = T(0);
 #pragma unroll
           for (int k = 0; k < Q; ++k) u += mats.m[k * P + c] * v[k];
@@ -549,7 +560,15 @@ k_diag(const ElemArgs<T> a, const DiagMats<T, P, Q> mats) {
       }
     __syncthreads();
     if (f < 3) diag_words<Q, T>(a, f + 1, t, valid, w, v);
-    for (int idx = ij; idx < P * Q; idx += Q2) {  // y: lines (c, i)
+    // lines of the thread's own element, or (kPipe64) of the whole block in turn
+    auto lines = [&](int per_element, auto line) {
+      if constexpr (kPipe64)
+        for (int idx = t; idx < EB * per_element; idx += NT) line(sm + idx / per_element * W, idx % per_element);
+      else
+        for (int idx = ij; idx < per_element; idx += Q2) line(Zb, idx);
+    };
+    lines(P * Q, [&](T* Zb, int idx) {  // y: lines (c, i)
+      T* Yb = Zb + kDiagTerms * P * Q2;
       const int i = idx % Q, c = idx / Q;
       T s[3][P];
 #pragma unroll
@@ -558,6 +577,7 @@ k_diag(const ElemArgs<T> a, const DiagMats<T, P, Q> mats) {
         for (int bb = 0; bb < P; ++bb) s[g][bb] = T(0);
 #pragma unroll
       for (int m = 0; m < kDiagTerms; ++m) {
+        if (absent(m)) continue;
         T u[P];  // each term's sum by itself (short chains keep FP32's error at the former level)
 #pragma unroll
         for (int bb = 0; bb < P; ++bb) u[bb] = T(0);
@@ -574,9 +594,10 @@ k_diag(const ElemArgs<T> a, const DiagMats<T, P, Q> mats) {
       for (int g = 0; g < 3; ++g)
 #pragma unroll
         for (int bb = 0; bb < P; ++bb) Yb[((g * P + c) * P + bb) * Q + i] = s[g][bb];
-    }
+    });
     __syncthreads();
-    for (int idx = ij; idx < P * P; idx += Q2) {  // x: lines (c, b)
+    lines(P * P, [&](T* Zb, int idx) {  // x: lines (c, b)
+      const T* Yb = Zb + kDiagTerms * P * Q2;
       T s[P];
 #pragma unroll
       for (int aa = 0; aa < P; ++aa) s[aa] = T(0);
@@ -596,7 +617,7 @@ k_diag(const ElemArgs<T> a, const DiagMats<T, P, Q> mats) {
       }
 #pragma unroll
       for (int aa = 0; aa < P; ++aa) Zb[idx * P + aa] = s[aa];
-    }
+    });
     __syncthreads();
     if (valid) {
       if (a.evec) {  // deterministic: element-local values, summed per node by k_node_gather
