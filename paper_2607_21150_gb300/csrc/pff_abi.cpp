@@ -266,11 +266,11 @@ static int cheb_t(pff_level* L, bool w16, bool transpose, bool from_zero, int de
   const bool init = L->op->det && L->op->evec;
   int rc;
   if (!from_zero && (rc = apply_t<T>(L, x, Ad, transpose, st, w16))) return rc;
-  PFF_CK(launch_cheb_first<T>(n, b, from_zero ? nullptr : Ad, diag, mask, r, d, Ad, 1.0 / theta, st));
   if (degree == 1) {
-    if (from_zero) PFF_CK(cudaMemcpyAsync(x, d, sizeof(T) * n, cudaMemcpyDeviceToDevice, st));
-    else PFF_CK(launch_axpby<T>(x, d, 1.0, 1.0, n, st));
+    PFF_CK(launch_cheb_only<T>(n, b, from_zero ? nullptr : Ad, diag, x, 1.0 / theta, from_zero, st));
+    return PFF_OK;
   }
+  PFF_CK(launch_cheb_first<T>(n, b, from_zero ? nullptr : Ad, diag, mask, r, d, Ad, 1.0 / theta, st));
   for (int k = 0; k + 1 < degree; ++k) {
     if ((rc = apply_t<T>(L, d, Ad, transpose, st, w16, 0, 0, init))) return rc;
     const double rho_new = 1.0 / (2.0 * sigma - rho);

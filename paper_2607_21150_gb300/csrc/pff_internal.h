@@ -298,6 +298,9 @@ template <typename T>
 cudaError_t launch_cheb_first(long long n, const T* b, const T* Ax, const T* diag, const uint8_t* mask, T* r, T* d,
                               T* Ad, double inv_theta, cudaStream_t st);
 template <typename T>
+cudaError_t launch_cheb_only(long long n, const T* b, const T* Ax, const T* diag, T* x, double inv_theta, int xset,
+                             cudaStream_t st);
+template <typename T>
 cudaError_t launch_cheb_next(long long n, T* x, T* d, T* r, T* Ad, const T* diag, const uint8_t* mask, double c_d,
                              double c_r, int xset, int last, cudaStream_t st);
 

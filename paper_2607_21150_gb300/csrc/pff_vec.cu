@@ -265,13 +265,34 @@ cudaError_t launch_level_words(const double* a, float* w32, uint16_t* b16, long 
 //   first: r = D^-1 (b - A x),  d = r / theta          (A x absent: x = 0)
 //   next:  x += d (xset: x = d);  r -= D^-1 A d;  d = c_d d + c_r r
 //          last: x += that d too, which ends the smoothing (r, d not written)
-// Both leave in Ad what the action expects there, its next input's prescribed
+//   only:  x += D^-1 (b - A x) / theta, a smoothing of degree one (xset: x = that)
+// The first two leave in Ad what the action expects there, its next input's prescribed
 // entries and zeros elsewhere, so that no pass of its own prepares it.  Bound by
 // HBM: a degree-3 smoothing moves 21 vectors instead of 30 (64 bit or 32 bit;
 // 40^3 Q4 FP32, 67 MB each: 383 -> 226 us with the clears).  V entries per thread, 16-byte
 // accesses where every pointer allows them.
 template <typename T, int V> struct alignas(sizeof(T) * V) VecOf { T v[V]; };
 
+// As first with an axpby in FP64 arithmetic, which moves ten vectors instead of five,
+// a smoothing of degree one took 354 us at 32x31x33 Q4 FP32 (341 us with separate
+// updates), now 264 us.
+template <typename T, int V>
+__global__ void __launch_bounds__(kVecThreads) k_cheb_only(long long n, const T* b, const T* Ax, const T* diag, T* x,
+                                                           T inv_theta, int xset) {
+  using W = VecOf<T, V>;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n / V; i += (long long)gridDim.x * blockDim.x) {
+    const W bi = reinterpret_cast<const W*>(b)[i], gi = reinterpret_cast<const W*>(diag)[i];
+    W ax, xi;
+    if (Ax) ax = reinterpret_cast<const W*>(Ax)[i];
+    if (!xset) xi = reinterpret_cast<const W*>(x)[i];
+#pragma unroll
+    for (int c = 0; c < V; ++c) {
+      const T d = (Ax ? bi.v[c] - ax.v[c] : bi.v[c]) / gi.v[c] * inv_theta;
+      xi.v[c] = xset ? d : xi.v[c] + d;
+    }
+    reinterpret_cast<W*>(x)[i] = xi;
+  }
+}
 template <typename T, int V>
 __global__ void __launch_bounds__(kVecThreads) k_cheb_first(long long n, const T* b, const T* Ax, const T* diag,
                                                             const uint8_t* mask, T* r, T* d, T* Ad, T inv_theta) {
@@ -340,6 +361,18 @@ cudaError_t launch_cheb_first(long long n, const T* b, const T* Ax, const T* dia
   return cudaGetLastError();
 }
 template <typename T>
+cudaError_t launch_cheb_only(long long n, const T* b, const T* Ax, const T* diag, T* x, double inv_theta, int xset,
+                             cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  constexpr int V = 16 / sizeof(T);
+  if (n % V == 0 && aligned16({b, Ax, diag, x}))
+    k_cheb_only<T, V><<<grid_for(n / V), kVecThreads, 0, st>>>(n, b, Ax, diag, x, (T)inv_theta, xset);
+  else
+    k_cheb_only<T, 1><<<grid_for(n), kVecThreads, 0, st>>>(n, b, Ax, diag, x, (T)inv_theta, xset);
+  note_launch();
+  return cudaGetLastError();
+}
+template <typename T>
 cudaError_t launch_cheb_next(long long n, T* x, T* d, T* r, T* Ad, const T* diag, const uint8_t* mask, double c_d,
                              double c_r, int xset, int last, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
@@ -357,6 +390,10 @@ template cudaError_t launch_cheb_first<double>(long long, const double*, const d
                                                double*, double*, double*, double, cudaStream_t);
 template cudaError_t launch_cheb_first<float>(long long, const float*, const float*, const float*, const uint8_t*,
                                               float*, float*, float*, double, cudaStream_t);
+template cudaError_t launch_cheb_only<double>(long long, const double*, const double*, const double*, double*, double,
+                                              int, cudaStream_t);
+template cudaError_t launch_cheb_only<float>(long long, const float*, const float*, const float*, float*, double, int,
+                                             cudaStream_t);
 template cudaError_t launch_cheb_next<double>(long long, double*, double*, double*, double*, const double*,
                                               const uint8_t*, double, double, int, int, cudaStream_t);
 template cudaError_t launch_cheb_next<float>(long long, float*, float*, float*, float*, const float*, const uint8_t*,
