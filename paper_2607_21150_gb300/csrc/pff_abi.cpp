@@ -82,16 +82,14 @@ int make_tables(int p, int Q, Tables& t) {
   int rc;
   if ((rc = upload(B, &t.B64))) return rc;
   if ((rc = upload(B, &t.B32))) return rc;
-  if ((rc = upload(Dc, &t.Dc64))) return rc;
   if ((rc = upload(Dc, &t.Dc32))) return rc;
   if ((rc = upload(Dt, &t.Dt64))) return rc;
-  if ((rc = upload(Dt, &t.Dt32))) return rc;
   return PFF_OK;
 }
 
 void free_tables(Tables& t) {
-  cudaFree(t.B64); cudaFree(t.Dc64); cudaFree(t.Dt64);
-  cudaFree(t.B32); cudaFree(t.Dc32); cudaFree(t.Dt32);
+  cudaFree(t.B64); cudaFree(t.Dt64);
+  cudaFree(t.B32); cudaFree(t.Dc32);
   t = Tables();
 }
 
@@ -128,15 +126,6 @@ cudaError_t diag_dispatch(int Q, int P, const ElemArgs<T>& a, const Tables& t, c
   return cudaErrorInvalidValue;
 }
 
-template <typename T> const T* tabB(const Tables& t);
-template <> const double* tabB<double>(const Tables& t) { return t.B64; }
-template <> const float* tabB<float>(const Tables& t) { return t.B32; }
-template <typename T> const T* tabDc(const Tables& t);
-template <> const double* tabDc<double>(const Tables& t) { return t.Dc64; }
-template <> const float* tabDc<float>(const Tables& t) { return t.Dc32; }
-template <typename T> const T* tabDt(const Tables& t);
-template <> const double* tabDt<double>(const Tables& t) { return t.Dt64; }
-template <> const float* tabDt<float>(const Tables& t) { return t.Dt32; }
 template <typename T> const T* linOf(const pff_op* op);
 template <> const double* linOf<double>(const pff_op* op) { return op->lin64; }
 template <> const float* linOf<float>(const pff_op* op) { return op->lin32; }
@@ -163,9 +152,8 @@ ElemArgs<T> level_args(const pff_level* L) {
   a.mesh = L->mesh;
   a.mask = level_mask(L);
   a.emask = a.mask ? level_emask(L) : nullptr;
-  a.B = tabB<T>(L->tab);
-  a.Dc = tabDc<T>(L->tab);
-  a.Dt = tabDt<T>(L->tab);
+  a.B = L->tab.B32;
+  a.Dc = L->tab.Dc32;
   a.lin = linOf<T>(L->op);
   a.fix = L->tab.fix;
   a.nq = L->op->nq;
@@ -648,9 +636,6 @@ int pff_op_set_geometry(pff_op* op, const double* X, void* stream) {
   std::memset(&a, 0, sizeof(a));
   a.mesh = op->mesh;
   a.x = xc;
-  a.B = op->tab.B64;
-  a.Dc = op->tab.Dc64;
-  a.Dt = op->tab.Dt64;
   a.fix = op->tab.fix;
   a.scratch = op->io;
   a.nq = nq;
@@ -682,9 +667,6 @@ int pff_residual(pff_op* op, const double* z, double* r, void* stream) {
   a.mesh = op->mesh;
   a.x = z;
   a.mask = nullptr;
-  a.B = op->tab.B64;
-  a.Dc = op->tab.Dc64;
-  a.Dt = op->tab.Dt64;
   a.fix = op->tab.fix;
   a.scratch = op->io;
   a.nq = op->nq;
@@ -740,9 +722,6 @@ int pff_reaction(pff_op* op, const uint8_t* sel, double* out4, void* stream) {
   a.mesh = op->mesh;
   a.y = op->fint;
   a.mask = nullptr;
-  a.B = op->tab.B64;
-  a.Dc = op->tab.Dc64;
-  a.Dt = op->tab.Dt64;
   a.fix = op->tab.fix;
   a.scratch = op->io;
   a.nq = op->nq;

@@ -42,17 +42,16 @@ __device__ __forceinline__ long long node_of(const MeshDev& m, int e, int a, int
 // of all slices (8 Q^3), so that the pointwise stage runs without barriers.
 template <int Q> __host__ __device__ constexpr int elem_smem_words() { return 12 * Q * Q * Q; }
 
-template <int P, int Q, typename T>
 struct ElemSmem {
-  T* bufA;  // [4][Q^3]
-  T* bufB;  // [4][Q^3]
-  const T* B;
-  const T* Dc;
+  float* bufA;  // [4][Q^3]
+  float* bufB;  // [4][Q^3]
+  const float* B;
+  const float* Dc;
 };
 
 // Gather x into bufA [4][c][b][a] (masked entries zero).
-template <int P, int Q, typename T>
-__device__ __forceinline__ void gather(const ElemArgs<T>& a, T* bufA, int e, bool valid, int ij) {
+template <int P, int Q>
+__device__ __forceinline__ void gather(const ElemArgs<float>& a, float* bufA, int e, bool valid, int ij) {
   constexpr int Q2 = Q * Q, Q3 = Q * Q * Q, P3 = P * P * P;
   const long long nn = a.mesh.nn;
   // the node mask is read only for elements flagged as having masked nodes
@@ -68,12 +67,12 @@ __device__ __forceinline__ void gather(const ElemArgs<T>& a, T* bufA, int e, boo
     long long n = valid ? node_of<P, Q>(a.mesh, e, aa, bb, cc) : 0;
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-      T v = T(0);
+      float v = 0.0f;
       if (valid) {
         long long g = f * nn + n;
         const auto xv = ldg(a.x + g);
         const bool fixed = masked && ldg(a.mask + g);
-        if (!fixed) v = (T)(xv);
+        if (!fixed) v = xv;
       }
       bufA[f * Q3 + idx] = v;
     }
@@ -81,18 +80,18 @@ __device__ __forceinline__ void gather(const ElemArgs<T>& a, T* bufA, int e, boo
 }
 
 // Forward: gather x into bufA, interpolate to Gauss points into bufB.
-template <int P, int Q, typename T>
-__device__ __forceinline__ void forward(const ElemArgs<T>& a, const ElemSmem<P, Q, T>& s, int e, bool valid, int ij) {
+template <int P, int Q>
+__device__ __forceinline__ void forward(const ElemArgs<float>& a, const ElemSmem& s, int e, bool valid, int ij) {
   constexpr int Q2 = Q * Q, Q3 = Q * Q * Q;
-  gather<P, Q, T>(a, s.bufA, e, valid, ij);
+  gather<P, Q>(a, s.bufA, e, valid, ij);
   __syncthreads();
   // x: [c][b][a] -> [c][b][i]
   for (int idx = ij; idx < P * P * Q; idx += Q2) {
     int i = idx % Q, r = idx / Q;  // r = b + P c
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-      const T* in = s.bufA + f * Q3 + r * P;
-      T acc = T(0);
+      const float* in = s.bufA + f * Q3 + r * P;
+      float acc = 0.0f;
 #pragma unroll
       for (int k = 0; k < P; ++k) acc = madd(acc, s.B[i * P + k], in[k]);
       s.bufB[f * Q3 + idx] = acc;
@@ -104,8 +103,8 @@ __device__ __forceinline__ void forward(const ElemArgs<T>& a, const ElemSmem<P, 
     int i = idx % Q, j = (idx / Q) % Q, c = idx / Q2;
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-      const T* in = s.bufB + f * Q3 + c * (P * Q) + i;
-      T acc = T(0);
+      const float* in = s.bufB + f * Q3 + c * (P * Q) + i;
+      float acc = 0.0f;
 #pragma unroll
       for (int k = 0; k < P; ++k) acc = madd(acc, s.B[j * P + k], in[k * Q]);
       s.bufA[f * Q3 + idx] = acc;
@@ -117,12 +116,12 @@ __device__ __forceinline__ void forward(const ElemArgs<T>& a, const ElemSmem<P, 
     const int i = ij % Q, j = ij / Q;
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-      T col[P];
+      float col[P];
 #pragma unroll
       for (int c = 0; c < P; ++c) col[c] = s.bufA[f * Q3 + c * Q2 + j * Q + i];
 #pragma unroll
       for (int k = 0; k < Q; ++k) {
-        T acc = T(0);
+        float acc = 0.0f;
 #pragma unroll
         for (int c = 0; c < P; ++c) acc = madd(acc, s.B[k * P + c], col[c]);
         s.bufB[f * Q3 + k * Q2 + j * Q + i] = acc;
@@ -133,13 +132,13 @@ __device__ __forceinline__ void forward(const ElemArgs<T>& a, const ElemSmem<P, 
 }
 
 // Parent-frame gradients of the four fields at point (i, j, k) from bufB.
-template <int P, int Q, typename T>
-__device__ __forceinline__ void grad_at(const ElemSmem<P, Q, T>& s, int i, int j, int k, T g[4][3], T& phi) {
+template <int Q>
+__device__ __forceinline__ void grad_at(const ElemSmem& s, int i, int j, int k, float g[4][3], float& phi) {
   constexpr int Q2 = Q * Q, Q3 = Q * Q * Q;
 #pragma unroll
   for (int f = 0; f < 4; ++f) {
-    const T* V = s.bufB + f * Q3;
-    T gx = T(0), gy = T(0), gz = T(0);
+    const float* V = s.bufB + f * Q3;
+    float gx = 0.0f, gy = 0.0f, gz = 0.0f;
 #pragma unroll
     for (int m = 0; m < Q; ++m) {
       gx = madd(gx, s.Dc[i * Q + m], V[k * Q2 + j * Q + m]);
@@ -153,9 +152,9 @@ __device__ __forceinline__ void grad_at(const ElemSmem<P, Q, T>& s, int i, int j
 
 // Backward: from accumulated column values Y[f][k] (transposed derivative
 // already applied) to nodal element values, then scatter-add.
-template <int P, int Q, typename T>
-__device__ __forceinline__ void backward(const ElemArgs<T>& a, const ElemSmem<P, Q, T>& s, int e, bool valid, int ij,
-                                         T Y[4][Q]) {
+template <int P, int Q>
+__device__ __forceinline__ void backward(const ElemArgs<float>& a, const ElemSmem& s, int e, bool valid, int ij,
+                                         float Y[4][Q]) {
   constexpr int Q2 = Q * Q, Q3 = Q * Q * Q, P3 = P * P * P;
   const int i = ij % Q, j = ij / Q;
   // z (registers): [k][j][i] -> [c][j][i]
@@ -163,7 +162,7 @@ __device__ __forceinline__ void backward(const ElemArgs<T>& a, const ElemSmem<P,
   for (int f = 0; f < 4; ++f)
 #pragma unroll
     for (int c = 0; c < P; ++c) {
-      T acc = T(0);
+      float acc = 0.0f;
 #pragma unroll
       for (int k = 0; k < Q; ++k) acc = madd(acc, s.B[k * P + c], Y[f][k]);
       s.bufA[f * Q3 + c * Q2 + j * Q + i] = acc;
@@ -174,8 +173,8 @@ __device__ __forceinline__ void backward(const ElemArgs<T>& a, const ElemSmem<P,
     int ii = idx % Q, bb = (idx / Q) % P, c = idx / (P * Q);
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-      const T* in = s.bufA + f * Q3 + c * Q2 + ii;
-      T acc = T(0);
+      const float* in = s.bufA + f * Q3 + c * Q2 + ii;
+      float acc = 0.0f;
 #pragma unroll
       for (int jj = 0; jj < Q; ++jj) acc = madd(acc, s.B[jj * P + bb], in[jj * Q]);
       s.bufB[f * Q3 + idx] = acc;
@@ -187,8 +186,8 @@ __device__ __forceinline__ void backward(const ElemArgs<T>& a, const ElemSmem<P,
     int aa = idx % P, r = idx / P;
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-      const T* in = s.bufB + f * Q3 + r * Q;
-      T acc = T(0);
+      const float* in = s.bufB + f * Q3 + r * Q;
+      float acc = 0.0f;
 #pragma unroll
       for (int ii = 0; ii < Q; ++ii) acc = madd(acc, s.B[ii * P + aa], in[ii]);
       s.bufA[f * Q3 + idx] = acc;
@@ -197,7 +196,7 @@ __device__ __forceinline__ void backward(const ElemArgs<T>& a, const ElemSmem<P,
   __syncthreads();
   if (!valid) return;
   if (a.evec) {  // deterministic transpose: element-local values, summed per node by k_node_gather
-    T* ev = static_cast<T*>(a.evec) + (long long)e * 4 * P3;
+    float* ev = static_cast<float*>(a.evec) + (long long)e * 4 * P3;
     for (int idx = ij; idx < P3; idx += Q2)
 #pragma unroll
       for (int f = 0; f < 4; ++f) ev[f * P3 + idx] = (s.bufA[f * Q3 + idx]);
@@ -375,10 +374,10 @@ k_elem(const ElemArgs<float> a) {
   float* base = sm + mat_smem_words<P, Q>() + el * elem_smem_words<Q>();
   // bufB first (read by every slice's gradients), then bufA which extends to the
   // 8 x Q^3 derivative outputs of the pointwise stage
-  const ElemSmem<P, Q, float> s{base + 4 * Q3, base, Bs, Dcs};
+  const ElemSmem s{base + 4 * Q3, base, Bs, Dcs};
   __syncthreads();
   for (int k = 0; k < kPrefetchAhead; ++k) prefetch_slice<Q>(a, k, t);
-  forward<P, Q, float>(a, s, e, valid, ij);
+  forward<P, Q>(a, s, e, valid, ij);
 
   float Y[4][Q];
 #pragma unroll
@@ -393,7 +392,7 @@ k_elem(const ElemArgs<float> a) {
   for (int k = 0; k < Q; ++k) {
     float g[4][3], phi, o[4][3], o0 = 0.0f;
     prefetch_slice<Q>(a, k + kPrefetchAhead, t);
-    grad_at<P, Q, float>(s, i, j, k, g, phi);
+    grad_at<Q>(s, i, j, k, g, phi);
     if (valid) {
       const float* q = blk + lin32_word(0, k, t, stride, run);
       const float* tl = blk + lin32_word(kLinQuadWords, k, t, stride, run);
@@ -428,7 +427,7 @@ k_elem(const ElemArgs<float> a) {
       Y[f][k] = acc;
     }
   __syncthreads();  // the derivative outputs are read; backward reuses the buffers
-  backward<P, Q, float>(a, s, e, valid, ij, Y);
+  backward<P, Q>(a, s, e, valid, ij, Y);
 }
 
 // Diagonal of the element operators: for each field f and node a,

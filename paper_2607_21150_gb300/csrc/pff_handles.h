@@ -29,9 +29,9 @@ struct pff_restr {
   int64_t nn;
 };
 
-struct Tables {  // per-level device copies of the 1D matrices, both precisions
-  double *B64 = nullptr, *Dc64 = nullptr, *Dt64 = nullptr;
-  float *B32 = nullptr, *Dc32 = nullptr, *Dt32 = nullptr;
+struct Tables {  // 1D matrices of a level: device copies for the assembled level (FP64) and the FP32 actions
+  double *B64 = nullptr, *Dt64 = nullptr;
+  float *B32 = nullptr, *Dc32 = nullptr;
   // B, D_t and D_c in FP32, each entry twice (kernel parameters)
   unsigned long long hB2[pff::kMaxQ * pff::kMaxQ] = {}, hD2[pff::kMaxQ * pff::kMaxQ] = {},
                      hDc2[pff::kMaxQ * pff::kMaxQ] = {};

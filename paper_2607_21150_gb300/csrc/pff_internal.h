@@ -61,9 +61,9 @@ __host__ __device__ constexpr int fix_threads(int Q, int elems) {
   return Q >= 4 ? (Q * Q * Q * elems + 31) / 32 * 32 : Q * Q * Q * elems;
 }
 
-// Shared-memory words of the 1D matrices in an element kernel (B, D_t, and
-// the collocated derivative D_c; the persistent kernel keeps B and D_c).
-template <int P, int Q> __host__ __device__ constexpr int mat_smem_words() { return 3 * Q * P + Q * Q; }
+// Shared-memory words of the 1D matrices B and D_c of the FP32 action without the
+// persistent kernel (which keeps D_c alone).
+template <int P, int Q> __host__ __device__ constexpr int mat_smem_words() { return Q * P + Q * Q; }
 
 // Geometry of the persistent FP32-arithmetic level kernel (pff_elem_pipe.cuh);
 // here so that the host tests can check the bulk copies it issues.
@@ -214,9 +214,8 @@ struct ElemArgs {
   const T* x;             // [4][nn] input (apply) / unused
   T* y;                   // [4][nn] output (scatter-add)
   const uint8_t* mask;    // [4][nn] Dirichlet mask or nullptr
-  const T* B;             // [Q][P] interpolation to Gauss points
-  const T* Dc;            // [Q][Q] collocated derivative at Gauss points
-  const T* Dt;            // [Q][P] derivative of the basis at Gauss points (diagonal)
+  const float* B;         // FP32 actions: [Q][P] interpolation to Gauss points
+  const float* Dc;        // FP32 actions: [Q][Q] collocated derivative at Gauss points
   const T* lin;           // tiled stored linearisation (apply / diagonal)
   const T* linP;          // words multiplying dphi in the u rows (dP/dphi or, transposed, dL/dF)
   const T* linC;          // words multiplying grad u in the phi row

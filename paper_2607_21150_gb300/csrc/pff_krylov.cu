@@ -218,7 +218,6 @@ cudaError_t launch_bminus(T* y, const T* b, long long n, cudaStream_t st) {
   return cudaGetLastError();
 }
 template cudaError_t launch_bminus<double>(double*, const double*, long long, cudaStream_t);
-template cudaError_t launch_bminus<float>(float*, const float*, long long, cudaStream_t);
 
 // y = x / d elementwise
 template <typename T>

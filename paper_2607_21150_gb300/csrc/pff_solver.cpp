@@ -100,7 +100,6 @@ struct pff_solver {
   DotScalars *host = nullptr, *host_dev = nullptr;  // page-locked copies and their device address
   unsigned long long seq = 0;
   double* pw64 = nullptr;  // power-iteration start vector (FP64, fine size)
-  float* pw32 = nullptr;
   int transpose = 0;       // 1 while solving with J^T (adjoint)
   // adjoint work space (allocated on the first pff_adjoint_step)
   double *a_in = nullptr, *pbuf = nullptr, *qa = nullptr, *ag = nullptr, *alam = nullptr, *av = nullptr, *gth = nullptr;
@@ -667,7 +666,7 @@ void free_solver(pff_solver* s) {
   }
   cudaFree(s->V); cudaFree(s->Z); cudaFree(s->r); cudaFree(s->dz); cudaFree(s->zold);
   cudaFree(s->partial); cudaFree(s->arrived); cudaFree(s->sc); cudaFreeHost(s->host);
-  cudaFree(s->pw64); cudaFree(s->pw32);
+  cudaFree(s->pw64);
   cudaFree(s->a_in); cudaFree(s->pbuf); cudaFree(s->qa); cudaFree(s->ag); cudaFree(s->alam); cudaFree(s->av);
   cudaFree(s->gth);
 }
@@ -811,20 +810,16 @@ int pff_create_solver(pff_op* op, int nlevels, pff_level* const* levels, const p
   if (e == cudaSuccess) std::memset(s->host, 0, sizeof(DotScalars) * kHostSlots);
   if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&s->host_dev, s->host, 0);
   if (e == cudaSuccess) e = cudaMalloc(&s->pw64, sizeof(double) * s->n);
-  if (e == cudaSuccess) e = cudaMalloc(&s->pw32, sizeof(float) * s->n);
   if (e == cudaSuccess) {
     // seeded start vector of the eigenvalue estimates (xorshift64*, random signs)
     std::vector<double> h(s->n);
-    std::vector<float> hf(s->n);
     unsigned long long st = 0x9E3779B97F4A7C15ull;
     for (long long i = 0; i < s->n; ++i) {
       st ^= st >> 12; st ^= st << 25; st ^= st >> 27;
       double u = (double)((st * 0x2545F4914F6CDD1Dull) >> 11) * (1.0 / 9007199254740992.0);
       h[i] = (u < 0.5) ? -1.0 : 1.0;
-      hf[i] = (float)h[i];
     }
     e = cudaMemcpy(s->pw64, h.data(), sizeof(double) * s->n, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(s->pw32, hf.data(), sizeof(float) * s->n, cudaMemcpyHostToDevice);
   }
   if (e != cudaSuccess) {
     free_solver(s);
@@ -1018,9 +1013,6 @@ ElemArgs<double> fine_args(pff_op* op) {
   ElemArgs<double> a;
   std::memset(&a, 0, sizeof(a));
   a.mesh = op->mesh;
-  a.B = op->tab.B64;
-  a.Dc = op->tab.Dc64;
-  a.Dt = op->tab.Dt64;
   a.fix = op->tab.fix;
   a.lin = op->lin64;
   a.nq = op->nq;
