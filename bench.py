@@ -29,13 +29,12 @@ sys.path.insert(0, ROOT)
 METRIC = "Q4 Jacobian-apply GDoF/s & %HBM roofline; Newton step time FP64 vs mixed p-MG"
 FP64_PEAK_TFLOPS = 152 * 4 * 2.070e9 / 1e12  # 152 SMs x 2 DFMA/clk x 2 flop x max SM clock
 # DRAM bytes (read + write) per element of one Jacobian action, Q4 (P = Q = 5),
-# from one ncu capture of the same kernels on the 24^3 tension workload
-# (python bench.py --config tension_q4 --n 24 ...): FP64 220.06 + 5.48 MB over
-# a 3 040-element launch, FP32 words 495.72 + 3.87 MB and BF16 words 265.13 +
-# 3.72 MB over 13 824 elements; scaled to a launch by the element count.  None
-# where the kernel has changed since its counters were taken.
-TRAFFIC_PER_ELEMENT = {"f64": (220.06e6 + 5.48e6) / 3040, "f32": (495.72e6 + 3.87e6) / 13824,
-                       "bf16": (265.13e6 + 3.72e6) / 13824}
+# from ncu captures of the same kernels (k_elem_fix, k_level_pipe) on 24^3 elements
+# (13 824): FP64 986.50 + 33.99 MB, FP32 words 495.79 + 4.12 MB, BF16 words 265.14 +
+# 3.68 MB; scaled to a launch by the element count.  None where the kernel has
+# changed since its counters were taken.
+TRAFFIC_PER_ELEMENT = {"f64": (986.50e6 + 33.99e6) / 13824, "f32": (495.79e6 + 4.12e6) / 13824,
+                       "bf16": (265.14e6 + 3.68e6) / 13824}
 
 
 def peaks():

@@ -58,7 +58,7 @@ extern "C" {
 #define PFF_ERR_UNSUPPORTED -4
 
 /* kernel status bits returned by pff_get_status */
-#define PFF_STATUS_EIGEN 1       /* Jacobi eigen sweeps hit their cap (20) */
+#define PFF_STATUS_EIGEN 1       /* Jacobi eigen sweeps hit their cap (20), or their matrix is not finite */
 #define PFF_STATUS_DETF 2        /* det F <= 0 at some quadrature point */
 #define PFF_STATUS_NONFINITE 4   /* non-finite residual integrand */
 #define PFF_STATUS_PHASE 8       /* phase id >= nphase (phase 0 used) */
@@ -66,8 +66,8 @@ extern "C" {
 #define PFF_STATUS_PIPE 32       /* FP32-arithmetic level action (PFF_F32 or PFF_F32_BF16 words): a wait for staged words gave up (result invalid) */
 
 /* PFF_DF64: FP64 vectors, an accuracy of at least double-float (about 2^-47 of the
- * magnitudes per operation) asked for; served by the FP64 action, which takes less
- * time than pairs of floats did.  Needs pff_op_enable_df; accepted by
+ * magnitudes per operation) asked for; served by the FP64 action, whose results it
+ * repeats.  Needs pff_op_enable_df; accepted by
  * pff_jacobian_apply, pff_jacobian_transpose_apply and pff_jacobian_apply_host only.
  * PFF_F32_BF16: FP32 vectors and arithmetic, the stored linearisation read as
  * BF16 words (8 significant bits, relative rounding error <= 2^-9 per word;
@@ -229,8 +229,8 @@ int pff_jacobian_transpose_apply(pff_level* level, pff_prec prec, const void* x,
  * memory (4 N_n entries each, FP64 for PFF_F64 / PFF_DF64, FP32 for PFF_F32 /
  * PFF_F32_BF16; page-locked memory, e.g. cudaHostAlloc or cudaHostRegister,
  * lets the copies overlap the computation, pageable memory serialises them).
- * The element blocks run in `nchunks` chunks in element order (rounded to whole
- * waves of the element kernel); each chunk's node layers are uploaded ahead of
+ * The element blocks run in about `nchunks` chunks in element order (long enough
+ * to fill the GPU each); each chunk's node layers are uploaded ahead of
  * it on a second stream and the node layers no later chunk touches are
  * downloaded on a third while later chunks compute.  Asynchronous on
  * `stream`: x_host must stay unchanged and y_host unread until the stream has

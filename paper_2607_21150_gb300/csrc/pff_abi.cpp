@@ -200,8 +200,12 @@ int apply_t(pff_level* L, const T* x, T* y, int transpose, cudaStream_t st, bool
 }
 
 // PFF_DF64: the FP64 action, which has more accuracy than that precision asks for
-// and takes less time than contractions in pairs of floats did (64^3 Q4: 7.8
-// against 8.9 ms).
+// and takes less time on the fine level than contractions in pairs of floats did
+// (64^3 Q4: 7.6 against 8.9 ms).  On the low-order levels of large meshes the pairs
+// had been up to 18 % faster (order 1 of Q4, 32x31x33: 775 against 869 us): there
+// the map is nearly all of the action, and its 103 FP64 multiply-adds per point
+// keep the pipe 83 % busy.  The second plane of words that the pairs read would
+// cost 9.2 GB at 64^3 and a third of the residual's copies.
 int apply_df(pff_level* L, const double* x, double* y, int transpose, cudaStream_t st, int blk0 = 0, int nblk = 0,
              bool init = true) {
   PFF_REQUIRE(L->op->df && L->op->lin32, "PFF_DF64 apply needs pff_op_enable_df before pff_residual");

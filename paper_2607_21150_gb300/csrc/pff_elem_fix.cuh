@@ -28,8 +28,8 @@
 // elements.  The 1D matrices are kernel parameters (constant-bank operands).
 //
 // Measured, 64^3 Q4 action: 20.08 ms with FP64 contractions (88.7 % of the FP64
-// pipe), 7.70 ms now; the map alone is 5.4 ms of that pipe (ncu, 24^3: pipe 69 %
-// busy, issue 52 %, DRAM 28 %).  With one thread per column of points (12 warps
+// pipe), 7.64 ms now; the map alone is 5.4 ms of that pipe (ncu, 24^3: pipe 74 %
+// busy, issue 55 %, DRAM 31 %).  With one thread per column of points (12 warps
 // per SM, as the FP64 kernel had it) 17 ms; with one copy of the line code per
 // direction instead of loops over the directions 9.1 ms (instruction cache).
 // 4^3 Q2: 56 -> 13.3 us (64 elements in 21 blocks instead of three).

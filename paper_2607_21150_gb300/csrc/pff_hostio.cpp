@@ -12,8 +12,8 @@
 //   - the download stream copies the final layers back while later chunks run.
 // The uploads of chunk c + 1 and the downloads of chunk c - 1 then run while
 // chunk c computes; only the first chunk's upload and the last chunk's
-// download stay exposed.  Chunks are whole multiples of the blocks one wave of
-// the element kernel holds, so that no chunk ends in a partly filled wave.
+// download stay exposed.  Chunks are multiples of two or three element groups per
+// SM, so that none is too short to fill the GPU; they need not be whole waves.
 #include <algorithm>
 #include <string>
 #include <vector>
@@ -119,11 +119,14 @@ extern "C" int pff_jacobian_apply_host(pff_level* L, pff_prec prec, const void* 
   const int Q = L->op->Q;
   const int EB = elems_per_block(Q);
   const long long nel = m.nel, nblk = (nel + EB - 1) / EB;
-  // blocks per wave: two resident blocks per SM for the FP64, double-float and
-  // BF16-word kernels, three for the FP32 one
-  const long long wave = (long long)h->sms * (prec == PFF_F32 ? 3 : 2);
+  // granularity of the chunks in element groups.  With one group per block and two
+  // or three blocks per SM this was a wave; the FP64 kernel now takes a group in
+  // several blocks (Q4: ten, seven resident per SM) and the FP32-arithmetic kernel
+  // is persistent with two blocks per SM, so that a chunk may end in a partly
+  // filled wave (40^3 Q4, FP64: seven chunks of 912 groups and one of 16).
+  const long long unit = (long long)h->sms * (prec == PFF_F32 ? 3 : 2);
   long long cb = (nblk + nchunks - 1) / nchunks;
-  if (nblk > wave) cb = std::max(wave, (cb + wave - 1) / wave * wave);
+  if (nblk > unit) cb = std::max(unit, (cb + unit - 1) / unit * unit);
   char* xd = static_cast<char*>(h->xd);
   char* yd = static_cast<char*>(h->yd);
   const char* xh = static_cast<const char*>(x_host);

@@ -5,10 +5,12 @@
 // Both are sum-factorised over a tile of elements in shared memory, one element
 // layer and one field per block, and both are gathers: every fine (coarse) node
 // is written by the one block that owns it, so that no transfer needs atomics, a
-// cleared output or node multiplicities, and reruns give the same bits.  The
-// reads and writes of the fine vector bound both kernels (HBM), so a tile is 64
-// fine nodes wide (FP64: 32), its halo of one element width costs the
-// restriction about a quarter more reads (L2), every loop has constant bounds
+// cleared output or node multiplicities, and reruns give the same bits.  They are
+// bound by the latency of the tiles' gathers and stages (L2 mostly: DRAM 4 % busy
+// at 40x24x24).  The tile is 64 fine nodes wide (FP64: 32); its halo of one element
+// width costs the restriction about a quarter more reads, and as a block takes one
+// layer of vertices, it reads 2 p_f - 1 fine planes to own p_f (Q4: 7 for 4): about
+// 2.2 times the fine vector in all.  Every loop has constant bounds
 // (divisions by run-time widths made the kernels issue-bound: 107 and 87 us for the two) and
 // the Dirichlet mask is read only by blocks that have flagged elements.  The end
 // rows of the 1D matrix are those of the identity (both GLL sets hold -1 and 1),
